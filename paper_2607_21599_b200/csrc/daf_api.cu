@@ -94,7 +94,7 @@ static int carve_workspace(const ResolvedParams& rp, void* workspace, size_t byt
 static int do_select(const ResolvedParams& rp, const float* scores, int32_t n_sig, const int32_t* idx_in,
                      const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                      int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack, const Workspace& ws, cudaStream_t st,
-                     bool scores_from_previous_kernel = false, bool beside_previous_kernel = false, bool rows_far = false) {
+                     bool beside_previous_kernel = false, bool rows_far = false) {
     if (scores != nullptr && n_sig < 1) return DAF_ERR_INVALID_ARG;
     if (rp.k > 0) {
         if (scores == nullptr && idx_in == nullptr) return DAF_ERR_INVALID_ARG;
@@ -109,7 +109,7 @@ static int do_select(const ResolvedParams& rp, const float* scores, int32_t n_si
     for (const void* ptr : ptrs)
         if (ptr != nullptr && !aligned16(ptr)) return DAF_ERR_ALIGNMENT;
     return launch_select(rp, scores, n_sig, idx_in, q_fresh, k_fresh, v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
-                         v_pack, ws.status, ws.select_scratch, st, scores_from_previous_kernel, beside_previous_kernel,
+                         v_pack, ws.status, ws.select_scratch, st, beside_previous_kernel,
                          /*select_only=*/false, rows_far);
 }
 
@@ -178,7 +178,7 @@ int daf_select_from_kv(const daf_params* p, int32_t n_sig, const void* const* si
         if (int rc = launch_deviation_sum(rp, n_sig, sig_k_fresh, sig_v_fresh, sig_k_cached, sig_v_cached, sums, st)) return rc;
     // the sums are one signal row: from here on this is daf_select, launched right behind the signal kernel
     return do_select(rp, rp.L_d > 0 ? sums : nullptr, 1, nullptr, q_fresh, k_fresh, v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
-                     v_pack, ws, st, /*scores_from_previous_kernel=*/true);
+                     v_pack, ws, st);
 }
 
 int daf_important_attn(const daf_params* p, int32_t k, const void* q_pack, const void* k_pack, const void* v_pack,
@@ -242,7 +242,7 @@ int daf_imp_qd_attn_launches(const daf_params* p, const void* q_pack, const void
     const int64_t first_row = rp.fuse_mode == 1 ? rp.L_d : rp.k;
     return launch_attention_joint(q_pack, q_fresh, idx, k_pack, v_pack, nullptr, nullptr, rp.k, h, rp.fuse_mode == 1 ? idx : nullptr, q_question, kv_k, kv_v,
                                   rp.L_q, rp.L_d, h + first_row * row_bytes, row_bytes, rp.Hq, rp.Hkv, rp.scale, ws.status,
-                                  ws.attn_scratch, ws.attn_bytes, (cudaStream_t)stream, /*after_kernel=*/false, launches);
+                                  ws.attn_scratch, ws.attn_bytes, (cudaStream_t)stream, launches);
 }
 
 int daf_blend_attn(const daf_params* p, int32_t n_rows, const void* q_rows, const void* kv_k, const void* kv_v,
@@ -260,7 +260,7 @@ int daf_blend_attn(const daf_params* p, int32_t n_rows, const void* q_rows, cons
     // causal_off = N - n_rows only sizes the launch (last row sees at most N keys); the limits come from row_pos
     return launch_attention(q_rows, kv_k, kv_v, n_rows, rp.N, rp.Hq, rp.Hkv, rp.N - n_rows, rp.scale, false, false, out,
                             out_row_stride_bytes, nullptr, lse, ws.status, ws.attn_scratch, ws.attn_bytes,
-                            (cudaStream_t)stream, false, row_pos);
+                            (cudaStream_t)stream, row_pos);
 }
 
 int daf_deviation_scores(const daf_params* p, const void* k_fresh, const void* v_fresh, const void* k_cached,
@@ -344,7 +344,7 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
         if (int rc = launch_expand_fp8(rp, fp8->k8, fp8->v8, fp8->k_scale, fp8->v_scale, kv_k, kv_v, st)) return rc;
     if (int rc = do_select(rp, scores, n_sig, idx_in, rows ? rows->q : q_fresh, rows ? rows->k : k_fresh,
                            rows ? rows->v : v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
-                           v_pack, ws, st, false, /*beside_previous_kernel=*/fp8 != nullptr && rp.L_d > 0,
+                           v_pack, ws, st, /*beside_previous_kernel=*/fp8 != nullptr && rp.L_d > 0,
                            /*rows_far=*/rows != nullptr)) return rc;
     char* h = reinterpret_cast<char*>(hidden);
     // State fusion is done by the attention epilogues: each stage writes its final rows.  When both
@@ -356,15 +356,14 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     if (rp.k > 0 && rp.L_q > 0) {
         if (int rc = launch_attention_joint(q_pack, q_fresh, idx_out, k_pack, v_pack, k_fresh, v_fresh, rp.k, h, dst, qq, kv_k, kv_v, rp.L_q, rp.L_d,
                                             h + first_row * row_bytes, row_bytes, rp.Hq, rp.Hkv, rp.scale, ws.status,
-                                            ws.attn_scratch, ws.attn_bytes, st, /*after_kernel=*/true)) return rc;
+                                            ws.attn_scratch, ws.attn_bytes, st)) return rc;
     } else if (rp.L_q > 0) {
         if (int rc = launch_attention(qq, kv_k, kv_v, rp.L_q, rp.N, rp.Hq, rp.Hkv, rp.L_d, rp.scale, true, true,
                                       h + first_row * row_bytes, row_bytes, nullptr, nullptr, ws.status, ws.attn_scratch,
-                                      ws.attn_bytes, st, /*after_kernel=*/true)) return rc;
+                                      ws.attn_bytes, st)) return rc;
     } else {
         if (int rc = launch_attention(q_pack, k_pack, v_pack, rp.k, rp.k, rp.Hq, rp.Hkv, 0, rp.scale, false, false, h,
-                                      row_bytes, dst, nullptr, ws.status, ws.attn_scratch, ws.attn_bytes, st,
-                                      /*after_kernel=*/true)) return rc;
+                                      row_bytes, dst, nullptr, ws.status, ws.attn_scratch, ws.attn_bytes, st)) return rc;
     }
     if (row_pos_out != nullptr) {
         if (int rc = launch_fuse(rp, idx_out, nullptr, nullptr, nullptr, row_pos_out, st)) return rc;
@@ -407,7 +406,7 @@ int daf_select_topk(const daf_params* p, const float* scores, int32_t n_sig, int
     ResolvedParams sel = rp;
     sel.L_q = 0;
     return launch_select(sel, scores, n_sig, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, idx_out, nullptr, nullptr,
-                         nullptr, ws.status, ws.select_scratch, (cudaStream_t)stream, false, false, /*select_only=*/true);
+                         nullptr, ws.status, ws.select_scratch, (cudaStream_t)stream, false, /*select_only=*/true);
 }
 
 int daf_check_indices(const daf_params* p, int32_t k, const int32_t* idx, void* workspace, size_t workspace_bytes_,

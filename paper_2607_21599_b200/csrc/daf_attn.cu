@@ -1248,8 +1248,7 @@ static void fill_combine(CombineSeg* c, const SegArgs& s) {
 static int launch_combine(const CombineSeg& c0, const CombineSeg& c1, cudaStream_t stream) {
     const int rows = c0.n_rows + c1.n_rows;
     if (rows <= 0) return DAF_OK;
-    cudaError_t e = launch_kernel(attn_combine_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, stream,
-                                  /*after_kernel=*/true, c0, c1);
+    cudaError_t e = launch_kernel(attn_combine_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, stream, c0, c1);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
@@ -1258,7 +1257,7 @@ static int launch_combine(const CombineSeg& c0, const CombineSeg& c1, cudaStream
 int launch_attention(const void* q, const void* k, const void* v, int n_q, int n_kv, int Hq, int Hkv, int causal_off,
                      float scale, bool pack_group, bool allow_split, void* out, long long out_row_stride_bytes,
                      const int32_t* dst_rows, float* lse, DeviceStatus* status, void* scratch, size_t scratch_bytes,
-                     cudaStream_t stream, bool after_kernel, const int32_t* q_pos) {
+                     cudaStream_t stream, const int32_t* q_pos) {
     if (n_q <= 0) return DAF_OK;
     const int G = Hq / Hkv;
     AttnPlan pl = plan_attention(n_q, n_kv, Hq, G, causal_off, pack_group, allow_split);
@@ -1292,7 +1291,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     a.joint = 0;
     a.status = status;
     dim3 grid((unsigned)pl.head_blocks, (unsigned)pl.n_tb, (unsigned)pl.n_splits);
-    cudaError_t e = launch_kernel(attn_fwd_kernel<false>, grid, dim3(kAttnThreads), kAttnSmemBytes, stream, after_kernel, tq, tk, tv, tq, tk, tv,
+    cudaError_t e = launch_kernel(attn_fwd_kernel<false>, grid, dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
                                   to, to, a);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
@@ -1335,7 +1334,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
                            const void* kv_v,
                            int L_q, int L_d, void* out_question, long long out_row_stride_bytes, int Hq, int Hkv,
                            float scale, DeviceStatus* status, void* scratch, size_t scratch_bytes, cudaStream_t stream,
-                           bool after_kernel, int launches) {
+                           int launches) {
     const int G = Hq / Hkv, N = L_d + L_q;
     const JointPlan jp = plan_joint(k, L_q, L_d, Hq, G);
     if (joint_partial_bytes(jp) > scratch_bytes) return DAF_ERR_WORKSPACE;
@@ -1408,9 +1407,9 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     if (launches & 1) {
         const cudaError_t e = gather_kv
             ? launch_kernel(attn_fwd_kernel<true>, dim3((unsigned)items), dim3(kAttnThreadsGather), kAttnSmemBytes, stream,
-                            after_kernel, tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, a)
+                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, a)
             : launch_kernel(attn_fwd_kernel<false>, dim3((unsigned)items), dim3(kAttnThreads), kAttnSmemBytes, stream,
-                            after_kernel, tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, a);
+                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, a);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         if (int rc = check_launch()) return rc;

@@ -523,6 +523,7 @@ struct FuseArgs {
 
 __global__ void __launch_bounds__(kRowThreads)
 fuse_rows_kernel(const FuseArgs a) {
+    pdl_wait();
     const int row = blockIdx.x;
     int pos;
     const int4* src;
@@ -558,6 +559,7 @@ __global__ void __launch_bounds__(256)
 deviation_scores_kernel(const int4* __restrict__ k_fresh, const int4* __restrict__ v_fresh,
                         const int4* __restrict__ k_cached, const int4* __restrict__ v_cached,
                         int L_d, int chunks_per_row, float* __restrict__ scores) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int warps_per_grid = (int)(gridDim.x * (blockDim.x >> 5));
     for (int tok = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); tok < L_d; tok += warps_per_grid) {
@@ -590,6 +592,7 @@ struct SignalLayers {
 
 __global__ void __launch_bounds__(256)
 deviation_sum_kernel(const SignalLayers layers, int L_d, int chunks_per_row, float* __restrict__ sums) {
+    pdl_wait();
     pdl_launch_dependents();   // the selection kernel may start launching; it waits for this grid before reading sums
     const int lane = threadIdx.x & 31;
     const int warps_per_grid = (int)(gridDim.x * (blockDim.x >> 5));
@@ -633,11 +636,9 @@ static size_t select_smem_bytes(int L_d) {
 int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, const int32_t* idx_in,
                   const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                   int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack,
-                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool scores_from_previous_kernel,
-                  bool beside_previous_kernel, bool select_only, bool rows_far) {
+                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool beside_previous_kernel, bool select_only, bool rows_far) {
     // beside_previous_kernel: the kernel launched just before (the fp8 cache expansion) is independent of the
     // selection; the selection kernel starts while it runs and only waits for it before it retires
-    const bool dependent = scores_from_previous_kernel || beside_previous_kernel;
     const int wait_at_end = beside_previous_kernel ? 1 : 0;
     const int32_t* idx_src = idx_in;
     if (scores != nullptr && rp.L_d > 0 && rp.k > 0) {
@@ -656,12 +657,12 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         if (rp.L_d <= g_sel1_max_keys) {
             const size_t smem1 = sizeof(Sel1Shared) + ((size_t)padded(rp.L_d) + rp.L_d) * sizeof(uint32_t);   // keys and candidate list
             const cudaError_t e = launch_kernel(select_topk_cta_kernel, dim3(1), dim3(kSel1Threads), smem1, stream,
-                                                dependent, scores, n_sig, rp.L_d, rp.k, idx_out, wait_at_end);
+                                                scores, n_sig, rp.L_d, rp.k, idx_out, wait_at_end);
             if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         } else {
             const size_t smem = select_smem_bytes(rp.L_d);
             const cudaError_t e = launch_kernel(select_topk_kernel, dim3(kSelCluster), dim3(kSelThreads), smem, stream,
-                                                dependent, scores, n_sig, rp.L_d, rp.k,
+                                                scores, n_sig, rp.L_d, rp.k,
                                                 reinterpret_cast<uint32_t*>(scratch), idx_out, wait_at_end);
             if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         }
@@ -690,10 +691,8 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         // kernel to complete before it touches anything (so the result is that of a plain launch), but its CTAs are
         // already in place then -- after this library's selection kernel, and equally after the previous layer's
         // merge when layers are issued back to back.
-        cudaError_t e = rows_far ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream,
-                                                 /*after_kernel=*/true, a)
-                                 : launch_kernel(gather_update_kernel<false>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream,
-                                                 /*after_kernel=*/true, a);
+        cudaError_t e = rows_far ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a)
+                                 : launch_kernel(gather_update_kernel<false>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         if (int rc = check_launch()) return rc;
@@ -708,10 +707,11 @@ int launch_deviation_scores(const ResolvedParams& rp, const void* k_fresh, const
     int blocks = (rp.L_d + warps - 1) / warps;
     const int max_blocks = 148 * 8;          // a few waves of 256-thread CTAs; each warp then walks several tokens
     if (blocks > max_blocks) blocks = max_blocks;
-    deviation_scores_kernel<<<blocks, warps * 32, 0, stream>>>(
+    const cudaError_t e = launch_kernel(deviation_scores_kernel, dim3(blocks), dim3(warps * 32), 0, stream,
         reinterpret_cast<const int4*>(k_fresh), reinterpret_cast<const int4*>(v_fresh),
         reinterpret_cast<const int4*>(k_cached), reinterpret_cast<const int4*>(v_cached), rp.L_d, rp.Hkv * 16, scores);
     count_launch();
+    if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
 }
 
@@ -732,8 +732,10 @@ int launch_deviation_sum(const ResolvedParams& rp, int n_sig, const void* const*
     int blocks = (rp.L_d + warps - 1) / warps;
     const int max_blocks = 148 * 8;
     if (blocks > max_blocks) blocks = max_blocks;
-    deviation_sum_kernel<<<blocks, warps * 32, 0, stream>>>(layers, rp.L_d, rp.Hkv * 16, sums);
+    const cudaError_t e = launch_kernel(deviation_sum_kernel, dim3(blocks), dim3(warps * 32), 0, stream, layers, rp.L_d,
+                                        rp.Hkv * 16, sums);
     count_launch();
+    if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
 }
 
@@ -784,6 +786,7 @@ __global__ void __launch_bounds__(256)
 expand_fp8_cache_kernel(const uint4* __restrict__ k8, const uint4* __restrict__ v8, const float* __restrict__ k_scale,
                         const float* __restrict__ v_scale, uint4* __restrict__ kv_k, uint4* __restrict__ kv_v,
                         long long n_chunks, int Hkv) {
+    pdl_wait();                // first: what starts beside this grid may rely on everything before it being complete
     pdl_launch_dependents();   // the selection kernel does not depend on this grid and may run beside it
     // chunk c = 16 consecutive elements; a head is 128 elements = 8 chunks
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -806,10 +809,11 @@ int launch_expand_fp8(const ResolvedParams& rp, const void* k8, const void* v8, 
     if (n_chunks == 0) return DAF_OK;
     long long blocks = (2 * n_chunks + 255) / 256;
     if (blocks > 148 * 16) blocks = 148 * 16;
-    expand_fp8_cache_kernel<<<(unsigned)blocks, 256, 0, stream>>>(
+    const cudaError_t e = launch_kernel(expand_fp8_cache_kernel, dim3((unsigned)blocks), dim3(256), 0, stream,
         reinterpret_cast<const uint4*>(k8), reinterpret_cast<const uint4*>(v8), k_scale, v_scale,
         reinterpret_cast<uint4*>(kv_k), reinterpret_cast<uint4*>(kv_v), n_chunks, rp.Hkv);
     count_launch();
+    if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
 }
 
@@ -823,8 +827,9 @@ int launch_fuse(const ResolvedParams& rp, const int32_t* idx, const void* o_imp,
     a.hidden = reinterpret_cast<int4*>(hidden);
     a.idx = idx; a.row_pos = row_pos_out;
     a.k = rp.k; a.L_d = rp.L_d; a.L_q = rp.L_q; a.cq = rp.Hq * 16; a.mode = rp.fuse_mode;
-    fuse_rows_kernel<<<rows, kRowThreads, 0, stream>>>(a);
+    const cudaError_t e = launch_kernel(fuse_rows_kernel, dim3(rows), dim3(kRowThreads), 0, stream, a);
     count_launch();
+    if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
 }
 
