@@ -40,7 +40,7 @@ struct SegArgs {
     int n_tb;           // token blocks = ceil(n_q / Tt)
     int causal_off;     // token t sees keys <= t + causal_off ...
     const int32_t* q_pos; // ... or, when given, keys <= q_pos[t] (ascending positions of the query tokens)
-    // Query rows read in place instead of from a packed copy (Gp == 1 only): query token t is row q_idx[t]
+    // Query rows read in place instead of from a packed copy: query token t is row q_idx[t]
     // of q_src, a [q_src_rows, Hq, 128] tensor.  q_idx == nullptr: the Q tensor map covers packed rows.
     const __nv_bfloat16* q_src;
     const int32_t* q_idx;
@@ -51,22 +51,19 @@ struct SegArgs {
     const __nv_bfloat16* v_src;
     const int32_t* kv_idx;
     int kv_src_rows, kv_heads;
-    // Work items.  A CTA owns one token block (a unit).  Either every unit is cut into the same n_splits
-    // KV ranges of tiles_per_split tiles (chunk == 0), or -- packed causal attention only, where unit u
-    // sees min(u + 1, n_tb) tiles -- units [g chunk, (g + 1) chunk) are cut into g + 1 balanced ranges
-    // each, so that no item walks more than about `chunk` tiles.
+    // Work items.  A CTA owns one token block (a unit) of one head block, and one of n_splits KV ranges of
+    // tiles_per_split tiles.
     int head_blocks, n_units;
     int n_splits, tiles_per_split;
-    int chunk, n_slots;    // n_slots: number of (unit, range) pairs = partial-result slots
-    int n_items;           // head_blocks * (n_units * n_splits  or  n_slots)
+    int n_items;           // head_blocks * n_units * n_splits
     float scale;        // softmax scale
     float scale_log2;   // scale * log2(e)
     __nv_bfloat16* out; long long out_row_stride;  // elements
     const int32_t* dst_rows;
     int out_tiled;      // final rows leave by one tiled bulk store per tile (rows in token order, no dst_rows)
     float* lse;         // [Hq, n_q] or null
-    float* part_o;      // partial results, fp32, normalised per range: [slot rows][Hq][128]
-    float* part_lse;    // [slot rows][Hq]
+    float* part_o;      // partial results, fp32, normalised per range: [n_splits][n_q][Hq][128]
+    float* part_lse;    // [n_splits][n_q][Hq]
 };
 
 // A launch runs one problem on a 3-D grid (head block, unit, split), or two problems from one list of
@@ -192,8 +189,8 @@ struct CtaWork {
     int n_q, n_kv, G, Gp, Tt, n_tb, causal_off;
     const int32_t* q_pos;
     float scale_log2;
-    int seg_id, hb, unit, j_begin, j_end, item_splits, tok_base;
-    long long part_row0;      // the item's first row in the partial-result arrays, in tokens
+    int seg_id, hb, unit, j_begin, j_end, item_splits;
+    long long part_row0;      // first row of the item's range in the partial-result arrays, in tokens
 };
 
 __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
@@ -206,47 +203,23 @@ __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
     a.n_q = DAF_SEG(n_q); a.n_kv = DAF_SEG(n_kv); a.G = DAF_SEG(G); a.Gp = DAF_SEG(Gp); a.Tt = DAF_SEG(Tt);
     a.n_tb = DAF_SEG(n_tb); a.causal_off = DAF_SEG(causal_off); a.q_pos = DAF_SEG(q_pos); a.scale_log2 = DAF_SEG(scale_log2);
 
-    int hb, unit, j_begin, j_end, item_splits, tok_base;
-    long long part_row0;      // this item's first row in the partial-result arrays, in tokens
-    if (!args.joint || DAF_SEG(chunk) == 0) {
-        int split;
-        if (!args.joint) {
-            // blocks are dispatched x-fastest: all head blocks of the heaviest (last) unit go first
-            hb = (int)blockIdx.x; unit = (int)gridDim.y - 1 - (int)blockIdx.y; split = (int)blockIdx.z;
-        } else {
-            const int n_hb = DAF_SEG(head_blocks), n_units = DAF_SEG(n_units);
-            hb = item % n_hb;
-            const int rest = item / n_hb;
-            unit = n_units - 1 - rest % n_units;
-            split = rest / n_units;
-        }
-        const int tps = DAF_SEG(tiles_per_split);
-        j_begin = split * tps;
-        j_end = j_begin + tps;
-        item_splits = DAF_SEG(n_splits);
-        part_row0 = (long long)split * a.n_q;
-        tok_base = 0;
+    int hb, unit, split;
+    if (!args.joint) {
+        // blocks are dispatched x-fastest: all head blocks of the heaviest (last) unit go first
+        hb = (int)blockIdx.x; unit = (int)gridDim.y - 1 - (int)blockIdx.y; split = (int)blockIdx.z;
     } else {
-        // packed causal attention cut into balanced ranges: slot numbers ascend with the unit, the
-        // grid walks them from the top so that the longest items start first
-        const int n_hb = DAF_SEG(head_blocks), chunk = DAF_SEG(chunk);
+        const int n_hb = DAF_SEG(head_blocks), n_units = DAF_SEG(n_units);
         hb = item % n_hb;
-        const int slot = DAF_SEG(n_slots) - 1 - item / n_hb;
-        int g = (int)((sqrtf(1.f + 8.f * (float)slot / (float)chunk) - 1.f) * 0.5f);
-        while (chunk * (g + 1) * (g + 2) / 2 <= slot) ++g;
-        while (g > 0 && chunk * g * (g + 1) / 2 > slot) --g;
-        const int rem = slot - chunk * g * (g + 1) / 2;
-        unit = g * chunk + rem / (g + 1);
-        const int range = rem % (g + 1);
-        const int n_tiles = min(unit + 1, a.n_tb);
-        j_begin = range * n_tiles / (g + 1);
-        j_end = (range + 1) * n_tiles / (g + 1);
-        item_splits = g + 1;
-        part_row0 = (long long)slot * kBlockM;
-        tok_base = unit * kBlockM;
+        const int rest = item / n_hb;
+        unit = n_units - 1 - rest % n_units;
+        split = rest / n_units;
     }
-    a.seg_id = seg_id; a.hb = hb; a.unit = unit; a.j_begin = j_begin; a.j_end = j_end;
-    a.item_splits = item_splits; a.tok_base = tok_base; a.part_row0 = part_row0;
+    const int tps = DAF_SEG(tiles_per_split);
+    a.seg_id = seg_id; a.hb = hb; a.unit = unit;
+    a.j_begin = split * tps;
+    a.j_end = a.j_begin + tps;
+    a.item_splits = DAF_SEG(n_splits);
+    a.part_row0 = (long long)split * a.n_q;
 }
 
 // Final step of a tile: the warp's 32 rows of O (fp32 in tensor memory at o_addr, this thread's row
@@ -351,7 +324,7 @@ __device__ __forceinline__ void write_rows(const AttnArgs& args, const CtaWork& 
             }
         }
     } else {
-        const long long prow0 = a.part_row0 - a.tok_base;
+        const long long prow0 = a.part_row0;
         if (row_valid) e.part_lse[(prow0 + tok) * e.Hq + head] = lse_val;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {   // 64 fp32 columns (256 bytes per row) at a time
@@ -593,12 +566,12 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         uint4 w[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const int tokr = t0 + quad * 32 + 2 * i + sub;
+            const int rr = quad * 32 + 2 * i + sub, dt = rr / a.Gp, tokr = t0 + dt;
             w[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (tokr < a.n_q) {
+            if (dt < a.Tt && tokr < a.n_q) {
                 const int src = __ldg(q_idx + tokr);
                 if ((unsigned)src < (unsigned)q_src_rows)   // a bad position is reported by the gather kernel
-                    w[i] = __ldg(reinterpret_cast<const uint4*>(q_src + ((size_t)src * Hq + h0) * kD) + cidx);
+                    w[i] = __ldg(reinterpret_cast<const uint4*>(q_src + ((size_t)src * Hq + h0 + (rr - dt * a.Gp)) * kD) + cidx);
             }
         }
 #pragma unroll
@@ -854,47 +827,27 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
 
 #undef DAF_SEG
 
-// Merge of partial results: one warp per (token, head) row.  A launch merges the rows of up to two
-// problems (those of s0 first).  A row's partials sit `stride` rows apart; how many there are is the
-// same for every row (n_splits) or, for a problem cut into balanced ranges, follows from its unit.
-struct CombineSeg {
+// Merge of partial results: one warp per (token, head) row.
+struct CombineArgs {
     const float* part_o; const float* part_lse;
     int n_q, Hq;
-    int tok_first;       // rows of tokens below this were written in final form by the attention kernel
-    int n_rows;          // (n_q - tok_first) * Hq
-    int n_splits;        // > 0: every row has this many partials, n_q * Hq rows apart
-    int unit_tokens, chunk;   // n_splits == 0: tokens per unit, units per group (see SegArgs)
+    int n_splits;        // partials per row, n_q * Hq rows apart
     __nv_bfloat16* out; long long out_row_stride; const int32_t* dst_rows; float* lse;
 };
 
 __global__ void __launch_bounds__(256)
-attn_combine_kernel(const CombineSeg s0, const CombineSeg s1) {
+attn_combine_kernel(const CombineArgs a) {
     DAF_KT_BEGIN(2);
     pdl_wait();                // partial results come from the attention kernel launched just before
     DAF_KT_BEGIN(3);
-    int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    const bool second = row >= s0.n_rows;
-    if (second) row -= s0.n_rows;
-#define DAF_CS(field) (second ? s1.field : s0.field)
-    if (row >= DAF_CS(n_rows)) return;
-    const int Hq = DAF_CS(Hq), n_q = DAF_CS(n_q);
-    const int tok = DAF_CS(tok_first) + row / Hq, head = row % Hq;
-    int n_splits = DAF_CS(n_splits);
-    size_t first, stride;      // in rows of the partial arrays
-    if (n_splits > 0) {
-        first = (size_t)tok * Hq + head;
-        stride = (size_t)n_q * Hq;
-    } else {
-        const int ut = DAF_CS(unit_tokens), chunk = DAF_CS(chunk);
-        const int unit = tok / ut, g = unit / chunk;
-        n_splits = g + 1;
-        const int slot0 = chunk * g * (g + 1) / 2 + (unit - g * chunk) * (g + 1);
-        first = ((size_t)slot0 * ut + (size_t)(tok - unit * ut)) * Hq + head;
-        stride = (size_t)ut * Hq;
-    }
-    const float* part_o = DAF_CS(part_o);
-    const float* part_lse = DAF_CS(part_lse);
+    const int Hq = a.Hq, n_q = a.n_q, n_splits = a.n_splits;
+    if (row >= n_q * Hq) return;
+    const int tok = row / Hq, head = row % Hq;
+    const size_t first = row, stride = (size_t)n_q * Hq;      // in rows of the partial arrays
+    const float* part_o = a.part_o;
+    const float* part_lse = a.part_lse;
     // lane s holds the log-sum-exp of partial s (at most 32 of them), so all of them are fetched at once;
     // the first eight partial rows are requested in the same breath, before the weights are known
     const float4* src = reinterpret_cast<const float4*>(part_o + first * kD) + lane;
@@ -933,16 +886,13 @@ attn_combine_kernel(const CombineSeg s0, const CombineSeg s1) {
         acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
     }
     const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-    const int32_t* dst_rows = DAF_CS(dst_rows);
-    const long long drow = dst_rows ? (long long)dst_rows[tok] : (long long)tok;
+    const long long drow = a.dst_rows ? (long long)a.dst_rows[tok] : (long long)tok;
     uint2 w2;
     w2.x = pack_bf16(acc.x * inv, acc.y * inv);
     w2.y = pack_bf16(acc.z * inv, acc.w * inv);
-    reinterpret_cast<uint2*>(DAF_CS(out) + drow * DAF_CS(out_row_stride) + (long long)head * kD)[lane] = w2;
-    float* lse = DAF_CS(lse);
-    if (lse != nullptr && lane == 0) lse[(size_t)head * n_q + tok] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
+    reinterpret_cast<uint2*>(a.out + drow * a.out_row_stride + (long long)head * kD)[lane] = w2;
+    if (a.lse != nullptr && lane == 0) a.lse[(size_t)head * n_q + tok] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
     DAF_KT_END(2);
-#undef DAF_CS
 }
 
 // ----------------------------------------------------------------- host side
@@ -1036,6 +986,27 @@ static int num_sms() {
     return n;
 }
 
+// Query heads per tile of a causal problem over its own keys.  With the whole group in a tile (rows = G heads x 128/G
+// tokens) the causal staircase of a tile is only 128/G tokens deep instead of 128, so fewer masked sub-steps are computed;
+// against that stand the rows that a group leaves over in a tile (128 - G * (128/G), e.g. 2 of 128 for G = 7).  Both are
+// counted, in sub-steps of all tiles: at 922 tokens and G = 7 it is 413 against 497 (28 layers of 6k 787 -> 747 us), at
+// 2201 and G = 5 1608 against 1705 (layer 116 -> 113 us), at 41780 and G = 7 1.2 % more, so there tiles keep one head.
+static long long causal_substeps(int n, int G, int Gp) {
+    const int Tt = kBlockM / Gp, last = (n + Tt - 1) / Tt;      // tiles 1 .. last see ceil(min(j Tt, n) / kSubN) sub-steps each
+    auto below = [&](int m) {                                   // sum of ceil(j Tt / kSubN) for j = 1 .. m; kSubN tiles advance Tt sub-steps
+        long long period = 0, part = 0;
+        const int q = m / kSubN, r = m % kSubN;
+        for (int j = 1; j <= kSubN; ++j) period += (j * Tt + kSubN - 1) / kSubN;
+        for (int j = 1; j <= r; ++j) part += (long long)q * Tt + (j * Tt + kSubN - 1) / kSubN;
+        return q * period + (long long)kSubN * Tt * q * (q - 1) / 2 + part;
+    };
+    return (below(last - 1) + (n + kSubN - 1) / kSubN) * (G / Gp);
+}
+static int causal_heads_per_tile(int n, int G) {
+    if (G == 1 || G > kBlockM) return 1;
+    return causal_substeps(n, G, G) <= causal_substeps(n, G, 1) ? G : 1;
+}
+
 // How a single problem is cut into CTAs: one per (head block, token block), and for the question rows,
 // where there are few query tiles and a long KV axis, also per range of the KV axis.
 
@@ -1072,27 +1043,18 @@ size_t attn_partial_bytes(int n_q, int Hq, int n_splits) {
     return o + l;
 }
 
-// Number of (unit, range) slots of units [0, n_units) when groups of `chunk` units are cut into 1, 2, 3, ... ranges.
-static int slots_before(int n_units, int chunk) {
-    const int g = n_units / chunk;
-    return chunk * g * (g + 1) / 2 + (n_units - g * chunk) * (g + 1);
-}
-
-// Steps 2 and 3 of one layer as one list of work items.  Two things are free: into how many balanced
-// ranges the long causal chains of the important-token stage are cut (`chunk`), and into how many KV
-// ranges the question rows are cut.  Finer ranges balance the 296 CTA slots better but cost a fixed
-// time per item, partial-result traffic and a longer merge, and the optimum jumps around with the tile
-// counts.  So the choice is made by replaying the hardware's dispatch (items in grid order onto the
-// slot that frees first) for a handful of candidates with a three-constant cost model and keeping the
-// cheapest; the result is cached per problem shape.
+// Steps 2 and 3 of one layer as one list of work items.  One thing is free: into how many KV ranges the question rows
+// are cut.  Finer ranges balance the 296 CTA slots better but cost a fixed time per item, partial-result traffic and a
+// longer merge, and the optimum jumps around with the tile counts.  So the choice is made by replaying the hardware's
+// dispatch (items in grid order onto the slot that frees first) for every distinct number of ranges with a
+// three-constant cost model and keeping the cheapest; the result is cached per problem shape.
 namespace {
 constexpr float kCostItemUs = 7.0f;        // set-up, first logits and row epilogue of an item (5-6 us alone; fitted)
 constexpr float kCostSubStepUs = 1.05f;    // 64 keys through one tile with two CTAs per SM (measured 0.95-1.1 us)
 constexpr float kCostMergeUs = 2.0f;       // merge launch
 constexpr float kCostMergeUsPerMB = 0.15f; // plus re-reading the partial rows of the question ranges (fitted together with the item cost)
-constexpr float kCostMergeUsPerMBCut = 0.45f;  // partial rows of cut causal chains (measured: 7.0 us for 14.8 MB, 13.3 for 25, 42.6 for 96)
 
-int g_force_chunk = 0, g_force_splits_q = 0;   // tuning builds can pin the choice
+int g_force_splits_q = 0;   // tuning builds can pin the choice
 float g_last_predicted_us = 0.f;
 
 struct JointShape { int k, L_q, L_d, Hq, G; };
@@ -1104,19 +1066,8 @@ bool operator<(const JointShape& a, const JointShape& b) {
     return a.G < b.G;
 }
 
-// Fills the fields of `jp` that follow from (chunk, n_splits_q).
-void set_choice(JointPlan& jp, int chunk, int n_splits_q, int L_q, int L_d, int Hq) {
-    if (chunk < (jp.n_tb_i + 31) / 32) chunk = (jp.n_tb_i + 31) / 32;   // at most 32 ranges per token block
-    if (chunk < 1) chunk = 1;
-    if (chunk > jp.n_tb_i) chunk = jp.n_tb_i;
-    jp.chunk = chunk;
-    jp.n_slots = slots_before(jp.n_tb_i, chunk);
-    jp.part_bytes_i = 0;
-    if (chunk < jp.n_tb_i) {
-        const size_t rows = (size_t)jp.n_slots * kBlockM * Hq;
-        jp.part_bytes_i = rows * kD * sizeof(float) + (rows * sizeof(float) + 255) / 256 * 256;
-    }
-    jp.items_i = Hq * jp.n_slots;
+// Fills the fields of `jp` that follow from n_splits_q.
+void set_choice(JointPlan& jp, int n_splits_q, int L_q, int L_d, int Hq) {
     const int tiles_q = (L_d + L_q + kBlockN - 1) / kBlockN;
     if (n_splits_q < 1) n_splits_q = 1;
     jp.tiles_per_split_q = (tiles_q + n_splits_q - 1) / n_splits_q;
@@ -1126,13 +1077,13 @@ void set_choice(JointPlan& jp, int chunk, int n_splits_q, int L_q, int L_d, int 
 }
 
 // Predicted time of the attention launch + merge for a filled plan, in microseconds.
-float predict_us(const JointPlan& jp, int k, int L_q, int L_d, int Hq) {
+float predict_us(const JointPlan& jp, int k, int L_q, int L_d) {
     const int slots = num_sms() * 2;
     std::priority_queue<float, std::vector<float>, std::greater<float>> free_at;
     for (int i = 0; i < slots; ++i) free_at.push(0.f);
     float makespan = 0.f;
-    auto run = [&](int count, int tiles) {
-        const float cost = kCostItemUs + kCostSubStepUs * 2.f * (float)tiles;
+    auto run = [&](int count, int substeps) {
+        const float cost = kCostItemUs + kCostSubStepUs * (float)substeps;
         for (int i = 0; i < count; ++i) {
             const float t = free_at.top() + cost;
             free_at.pop();
@@ -1144,27 +1095,15 @@ float predict_us(const JointPlan& jp, int k, int L_q, int L_d, int Hq) {
     for (int s = 0; s < jp.n_splits_q; ++s)
         for (int u = jp.n_tb_q - 1; u >= 0; --u) {
             const int last_tok = (u + 1) * jp.Tt_q < L_q ? (u + 1) * jp.Tt_q : L_q;
-            const int tiles_total = (L_d + last_tok + kBlockN - 1) / kBlockN;
-            int tiles = tiles_total - s * jp.tiles_per_split_q;
-            if (tiles > jp.tiles_per_split_q) tiles = jp.tiles_per_split_q;
-            if (tiles > 0) run(jp.head_blocks_q, tiles);
+            const int begin = s * jp.tiles_per_split_q * kBlockN;
+            int end = begin + jp.tiles_per_split_q * kBlockN;
+            if (end > L_d + last_tok) end = L_d + last_tok;
+            if (end > begin) run(jp.head_blocks_q, (end - begin + kSubN - 1) / kSubN);
         }
-    // important-token items: slots from the top down, all heads together
-    size_t part_rows_i = 0;
-    for (int slot = jp.n_slots - 1; slot >= 0; --slot) {
-        int g = 0;
-        while (jp.chunk * (g + 1) * (g + 2) / 2 <= slot) ++g;
-        const int rem = slot - jp.chunk * g * (g + 1) / 2;
-        const int unit = g * jp.chunk + rem / (g + 1), range = rem % (g + 1);
-        const int n_tiles = unit + 1 < jp.n_tb_i ? unit + 1 : jp.n_tb_i;
-        run(Hq, (range + 1) * n_tiles / (g + 1) - range * n_tiles / (g + 1));
-        if (g >= 1) part_rows_i += (size_t)kBlockM * Hq;
-    }
-    (void)k;
-    const float merge_us = kCostMergeUs + kCostMergeUsPerMB * (float)jp.part_bytes_q / 1e6f +
-                           kCostMergeUsPerMBCut * (float)(part_rows_i * 516) / 1e6f;
-    const bool merges = jp.n_splits_q > 1 || jp.chunk < jp.n_tb_i;
-    return makespan + (merges ? merge_us : 0.f);
+    // important-token items: units from the last one down, head blocks together
+    for (int u = jp.n_tb_i - 1; u >= 0; --u)
+        run(jp.head_blocks_i, (((u + 1) * jp.Tt_i < k ? (u + 1) * jp.Tt_i : k) + kSubN - 1) / kSubN);
+    return makespan + (jp.n_splits_q > 1 ? kCostMergeUs + kCostMergeUsPerMB * (float)jp.part_bytes_q / 1e6f : 0.f);
 }
 }  // namespace
 
@@ -1172,7 +1111,7 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     static std::mutex mu;
     static std::map<JointShape, JointPlan> cache;
     const JointShape shape{k, L_q, L_d, Hq, G};
-    const bool forced = g_force_chunk > 0 || g_force_splits_q > 0;
+    const bool forced = g_force_splits_q > 0;
     // a layer loop asks for the same shape over and over: each thread keeps its last answer (no lock)
     static thread_local bool have_last = false;
     static thread_local JointShape last_shape;
@@ -1184,34 +1123,31 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
         if (it != cache.end()) { last_shape = shape; last_plan = it->second; have_last = true; return it->second; }
     }
     JointPlan jp;
-    jp.n_tb_i = (k + kBlockM - 1) / kBlockM;
+    jp.Gp_i = causal_heads_per_tile(k, G);
+    jp.Tt_i = kBlockM / jp.Gp_i;
+    jp.n_tb_i = (k + jp.Tt_i - 1) / jp.Tt_i;
+    jp.head_blocks_i = Hq / jp.Gp_i;
+    jp.items_i = jp.head_blocks_i * jp.n_tb_i;
     jp.Gp_q = G > 128 ? 1 : G;
     jp.Tt_q = kBlockM / jp.Gp_q;
     jp.n_tb_q = (L_q + jp.Tt_q - 1) / jp.Tt_q;
     jp.head_blocks_q = Hq / jp.Gp_q;
     const int tiles_q = (L_d + L_q + kBlockN - 1) / kBlockN;
     if (forced) {
-        set_choice(jp, g_force_chunk > 0 ? g_force_chunk : jp.n_tb_i, g_force_splits_q > 0 ? g_force_splits_q : 1, L_q, L_d, Hq);
-        g_last_predicted_us = predict_us(jp, k, L_q, L_d, Hq);
+        set_choice(jp, g_force_splits_q, L_q, L_d, Hq);
+        g_last_predicted_us = predict_us(jp, k, L_q, L_d);
         return jp;
     }
-    // candidates: the causal chains whole, or cut so that the longest has 2..6 ranges; every distinct
-    // number of question ranges up to 32
     JointPlan best = jp;
     float best_us = -1.f;
-    for (int m = 1; m <= 6; ++m) {
-        const int chunk = (jp.n_tb_i + m - 1) / m;
-        if (m > 1 && chunk == (jp.n_tb_i + m - 2) / (m - 1)) continue;   // same cut as the previous candidate
-        int last_tps = -1;
-        for (int n = 1; n <= kMaxSplits && n <= tiles_q; ++n) {
-            JointPlan cand = jp;
-            set_choice(cand, chunk, n, L_q, L_d, Hq);
-            if (cand.tiles_per_split_q == last_tps) continue;
-            last_tps = cand.tiles_per_split_q;
-            if (cand.part_bytes_i > ((size_t)256 << 20)) continue;   // partials of a large problem: not worth their memory
-            const float us = predict_us(cand, k, L_q, L_d, Hq);
-            if (best_us < 0.f || us < best_us) { best_us = us; best = cand; }
-        }
+    int last_tps = -1;
+    for (int n = 1; n <= kMaxSplits && n <= tiles_q; ++n) {
+        JointPlan cand = jp;
+        set_choice(cand, n, L_q, L_d, Hq);
+        if (cand.tiles_per_split_q == last_tps) continue;
+        last_tps = cand.tiles_per_split_q;
+        const float us = predict_us(cand, k, L_q, L_d);
+        if (best_us < 0.f || us < best_us) { best_us = us; best = cand; }
     }
     g_last_predicted_us = best_us;
     std::lock_guard<std::mutex> lock(mu);
@@ -1221,11 +1157,11 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
 }
 
 #if defined(DAF_TRACE) || defined(DAF_TUNE)     // tuning builds: pin the planner's choice, read its prediction
-extern "C" void daf_dbg_joint_force(int chunk, int n_splits_q) { g_force_chunk = chunk; g_force_splits_q = n_splits_q; }
+extern "C" void daf_dbg_joint_force(int n_splits_q) { g_force_splits_q = n_splits_q; }
 extern "C" float daf_dbg_joint_predicted_us(void) { return g_last_predicted_us; }
 extern "C" void daf_dbg_joint_plan(int k, int L_q, int L_d, int Hq, int G, int* out) {
     const JointPlan jp = plan_joint(k, L_q, L_d, Hq, G);
-    out[0] = jp.chunk; out[1] = jp.n_tb_i; out[2] = jp.n_splits_q; out[3] = jp.items_i + jp.items_q;
+    out[0] = jp.Gp_i; out[1] = jp.n_tb_i; out[2] = jp.n_splits_q; out[3] = jp.items_i + jp.items_q;
 }
 #endif
 
@@ -1243,23 +1179,10 @@ static void fill_problem(SegArgs* s, int n_q, int n_kv, int Hq, int G, int Gp, i
     s->lse = lse;
 }
 
-static void fill_combine(CombineSeg* c, const SegArgs& s) {
-    const int unit_tokens = kBlockM;   // packed causal attention has one head per tile: a unit is 128 tokens
-    c->part_o = s.part_o; c->part_lse = s.part_lse;
-    c->n_q = s.n_q; c->Hq = s.Hq;
-    c->n_splits = s.chunk == 0 ? s.n_splits : 0;
-    c->unit_tokens = unit_tokens; c->chunk = s.chunk > 0 ? s.chunk : 1;
-    c->tok_first = 0;
-    if (s.chunk == 0 && s.n_splits <= 1) c->tok_first = s.n_q;                    // nothing to merge
-    if (s.chunk > 0) c->tok_first = s.chunk * unit_tokens < s.n_q ? s.chunk * unit_tokens : s.n_q;
-    c->n_rows = (s.n_q - c->tok_first) * s.Hq;
-    c->out = s.out; c->out_row_stride = s.out_row_stride; c->dst_rows = s.dst_rows; c->lse = s.lse;
-}
-
-static int launch_combine(const CombineSeg& c0, const CombineSeg& c1, cudaStream_t stream) {
-    const int rows = c0.n_rows + c1.n_rows;
-    if (rows <= 0) return DAF_OK;
-    cudaError_t e = launch_kernel(attn_combine_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, stream, c0, c1);
+static int launch_combine(const SegArgs& s, cudaStream_t stream) {
+    if (s.n_splits <= 1) return DAF_OK;
+    const CombineArgs c{s.part_o, s.part_lse, s.n_q, s.Hq, s.n_splits, s.out, s.out_row_stride, s.dst_rows, s.lse};
+    const cudaError_t e = launch_kernel(attn_combine_kernel, dim3((unsigned)((s.n_q * s.Hq + 7) / 8)), dim3(256), 0, stream, c);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
@@ -1271,6 +1194,8 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
                      cudaStream_t stream, const int32_t* q_pos) {
     if (n_q <= 0) return DAF_OK;
     const int G = Hq / Hkv;
+    // a causal problem over its own keys chooses how many heads share a tile; the question rows always pack the group
+    if (!pack_group && q_pos == nullptr && causal_off == 0) pack_group = causal_heads_per_tile(n_q, G) > 1;
     AttnPlan pl = plan_attention(n_q, n_kv, Hq, G, causal_off, pack_group, allow_split);
     const size_t need = attn_partial_bytes(n_q, Hq, pl.n_splits);
     if (need > scratch_bytes) return DAF_ERR_WORKSPACE;
@@ -1293,7 +1218,6 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     s.out_tiled = out_tiled ? 1 : 0;
     s.n_units = pl.n_tb;
     s.n_splits = pl.n_splits; s.tiles_per_split = pl.tiles_per_split;
-    s.chunk = 0; s.n_slots = 0;
     s.n_items = pl.head_blocks * pl.n_tb * pl.n_splits;
     s.part_o = reinterpret_cast<float*>(scratch);
     s.part_lse = pl.n_splits > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(scratch) +
@@ -1307,13 +1231,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     if (int rc = check_launch()) return rc;
-    if (pl.n_splits > 1) {
-        CombineSeg c0, c1;
-        fill_combine(&c0, s);
-        memset(&c1, 0, sizeof(c1));
-        return launch_combine(c0, c1, stream);
-    }
-    return DAF_OK;
+    return launch_combine(s, stream);
 }
 
 // Self-test of the bounded wait every kernel here relies on: two warps wait on a barrier that nothing ever
@@ -1337,7 +1255,7 @@ int launch_bounded_wait_selftest(DeviceStatus* status, int limit_ms, cudaStream_
     return check_launch();
 }
 
-size_t joint_partial_bytes(const JointPlan& jp) { return jp.part_bytes_q + jp.part_bytes_i; }
+size_t joint_partial_bytes(const JointPlan& jp) { return jp.part_bytes_q; }
 
 int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t* idx, const void* k_imp, const void* v_imp,
                            const void* k_fresh, const void* v_fresh,
@@ -1354,7 +1272,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     // without packed Q rows the kernel reads them in place through idx (no tensor map needed for them)
     const bool gather_q = q_imp == nullptr;
     if (gather_q && (q_fresh == nullptr || idx == nullptr)) return DAF_ERR_INVALID_ARG;
-    if (int rc = make_tmap(&tq0, gather_q ? q_question : q_imp, gather_q ? L_q : k, Hq, 1, kBlockM)) return rc;
+    if (int rc = make_tmap(&tq0, gather_q ? q_question : q_imp, gather_q ? L_q : k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
     // without packed K/V rows the producer warp reads them in place through idx as well
     const bool gather_kv = k_imp == nullptr;
     if (gather_kv && (v_imp != nullptr || k_fresh == nullptr || v_fresh == nullptr || idx == nullptr)) return DAF_ERR_INVALID_ARG;
@@ -1371,7 +1289,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     CUtensorMap to0 = tq1, to1 = tq1;
     const bool imp_tiled = dst_rows_imp == nullptr;
     if (imp_tiled)
-        if (int rc = make_tmap(&to0, out_imp, k, Hq, 1, kBlockM, out_row_stride_bytes)) return rc;
+        if (int rc = make_tmap(&to0, out_imp, k, Hq, jp.Gp_i, jp.Tt_i, out_row_stride_bytes)) return rc;
     if (int rc = make_tmap(&to1, out_question, L_q, Hq, jp.Gp_q, jp.Tt_q, out_row_stride_bytes)) return rc;
     if (int rc = set_kernel_attributes()) return rc;
 
@@ -1384,13 +1302,12 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     sq.out_tiled = 1;
     sq.n_units = jp.n_tb_q;
     sq.n_splits = jp.n_splits_q; sq.tiles_per_split = jp.tiles_per_split_q;
-    sq.chunk = 0; sq.n_slots = 0;
     sq.n_items = jp.items_q;
     sq.part_o = reinterpret_cast<float*>(sc);
     sq.part_lse = reinterpret_cast<float*>(sc + (size_t)jp.n_splits_q * L_q * Hq * kD * sizeof(float));
-    // important tokens: packed causal attention, long chains cut into balanced ranges
+    // important tokens: causal attention over the condensed sequence, keys never cut
     SegArgs& si = a.seg[0];
-    fill_problem(&si, k, k, Hq, G, 1, 0, nullptr, scale, out_imp, out_row_stride_bytes, dst_rows_imp, nullptr);
+    fill_problem(&si, k, k, Hq, G, jp.Gp_i, 0, nullptr, scale, out_imp, out_row_stride_bytes, dst_rows_imp, nullptr);
     if (gather_q) {
         si.q_src = reinterpret_cast<const __nv_bfloat16*>(q_fresh);
         si.q_idx = idx;
@@ -1405,12 +1322,8 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     }
     si.out_tiled = imp_tiled ? 1 : 0;
     si.n_units = jp.n_tb_i;
-    si.n_splits = 1; si.tiles_per_split = jp.n_tb_i;
-    si.chunk = jp.chunk; si.n_slots = jp.n_slots;
+    si.n_splits = 1; si.tiles_per_split = (k + kBlockN - 1) / kBlockN;
     si.n_items = jp.items_i;
-    const size_t rows_i = (size_t)jp.n_slots * kBlockM * Hq;
-    si.part_o = reinterpret_cast<float*>(sc + jp.part_bytes_q);
-    si.part_lse = reinterpret_cast<float*>(sc + jp.part_bytes_q + rows_i * kD * sizeof(float));
     a.joint = 1;
     a.status = status;
 
@@ -1426,10 +1339,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
         if (int rc = check_launch()) return rc;
     }
     if (!(launches & 2)) return DAF_OK;
-    CombineSeg ci, cq;
-    fill_combine(&ci, si);
-    fill_combine(&cq, sq);
-    return launch_combine(ci, cq, stream);
+    return launch_combine(sq, stream);
 }
 
 }  // namespace daf

@@ -279,6 +279,22 @@ def test_important_attention_matches_oracle(n, Hq, Hkv, qscale):
     assert np.array_equal(_f(out[0]), np.repeat(_f(v[0]), Hq // Hkv, axis=0))
 
 
+@pytest.mark.parametrize("n,Hq,Hkv", [(1, 7, 1), (19, 14, 2), (155, 7, 1), (129, 10, 2), (77, 12, 1), (300, 100, 1), (33, 129, 1)])
+def test_causal_tiles_that_hold_a_whole_group_of_heads(n, Hq, Hkv):
+    """Group sizes that do and do not divide the 128 rows of a tile, and one that does not fit it: packed rows, the last
+    token block and the rows left over (tolerances as for every attention call)."""
+    q, k, v = _normal((n, Hq, 128), 71), _normal((n, Hkv, 128), 72), _normal((n, Hkv, 128), 73)
+    p = api.make_params(n, 0, 1.0, Hq, Hkv)
+    ws = api.alloc_workspace(p)
+    out = torch.full((n + 1, Hq, 128), 5.0, dtype=torch.bfloat16, device="cuda")
+    lse = torch.zeros(Hq, n, dtype=torch.float32, device="cuda")
+    _ok(api.daf_important_attn(p, n, q.cuda(), k.cuda(), v.cuda(), out, Hq * 256, None, lse, ws), ws, "daf_important_attn")
+    ref, ref_lse = oracle.important_attn(_f(q), _f(k), _f(v), 1.0 / math.sqrt(128), return_lse=True)
+    _assert_close(out[:n], ref, f"packed heads n={n} {Hq}/{Hkv}")
+    assert torch.all(out[n] == 5.0)
+    np.testing.assert_allclose(lse.cpu().numpy().T, ref_lse, atol=2e-3, rtol=0)
+
+
 def test_important_attention_scatters_rows_through_dst_rows():
     n, Hq, Hkv = 200, 4, 2
     q, k, v = _normal((n, Hq, 128), 31), _normal((n, Hkv, 128), 32), _normal((n, Hkv, 128), 33)
