@@ -94,7 +94,7 @@ static int carve_workspace(const ResolvedParams& rp, void* workspace, size_t byt
 static int do_select(const ResolvedParams& rp, const float* scores, int32_t n_sig, const int32_t* idx_in,
                      const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                      int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack, const Workspace& ws, cudaStream_t st,
-                     bool beside_previous_kernel = false, bool rows_far = false) {
+                     bool beside_previous_kernel = false, const RowSource* far = nullptr) {
     if (scores != nullptr && n_sig < 1) return DAF_ERR_INVALID_ARG;
     if (rp.k > 0) {
         if (scores == nullptr && idx_in == nullptr) return DAF_ERR_INVALID_ARG;
@@ -110,7 +110,7 @@ static int do_select(const ResolvedParams& rp, const float* scores, int32_t n_si
         if (ptr != nullptr && !aligned16(ptr)) return DAF_ERR_ALIGNMENT;
     return launch_select(rp, scores, n_sig, idx_in, q_fresh, k_fresh, v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
                          v_pack, ws.status, ws.select_scratch, st, beside_previous_kernel,
-                         /*select_only=*/false, rows_far);
+                         /*select_only=*/false, far);
 }
 
 static int check_out(const void* out, int64_t stride_bytes, int Hq) {
@@ -308,9 +308,6 @@ int daf_full_causal_attn(const daf_params* p, int32_t n_tokens, const void* q, c
 namespace {
 // Offline cache of one layer kept in fp8 (daf_layer_fp8): expanded into kv_k / kv_v ahead of everything else.
 struct Fp8Cache { const void* k8; const void* v8; const float* k_scale; const float* v_scale; };
-// Where the gather / cache-update kernel reads the fresh rows when that is not the tensors the attention reads the
-// question rows from: device-accessible pointers to [N, heads, 128] tensors (mapped pinned host memory).
-struct RowSource { const void* q; const void* k; const void* v; };
 
 int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, int32_t n_sig, const int32_t* idx_in,
                const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
@@ -345,7 +342,7 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     if (int rc = do_select(rp, scores, n_sig, idx_in, rows ? rows->q : q_fresh, rows ? rows->k : k_fresh,
                            rows ? rows->v : v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
                            v_pack, ws, st, /*beside_previous_kernel=*/fp8 != nullptr && rp.L_d > 0,
-                           /*rows_far=*/rows != nullptr)) return rc;
+                           rows)) return rc;
     char* h = reinterpret_cast<char*>(hidden);
     // State fusion is done by the attention epilogues: each stage writes its final rows.  When both
     // stages have rows they run as one list of work items in one launch, right behind the gather
@@ -465,6 +462,35 @@ constexpr int kArenaSignalRows = 8;   // arena is sized for up to this many sign
 // them in place): measured -2 % layer time at k = 41780, +-1 % at k = 6554, +10 % at k = 922.
 constexpr int kQInPlaceMinK = 16384;
 
+// A second stream for the part of a host-buffer layer that runs beside the rest, with the events that fork from and join
+// the caller's stream.  Each host thread keeps two per device (a pipelining caller begins a layer before it ends the one
+// before), made on first use and given back when the thread ends; what they order is in the events, so a lane may be
+// used again while earlier work is still under way in it.
+struct SideLane {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    ~SideLane() {
+        if (join) cudaEventDestroy(join);
+        if (fork) cudaEventDestroy(fork);
+        if (stream) cudaStreamDestroy(stream);
+    }
+};
+SideLane* side_lane() {
+    constexpr int kDevices = 16;
+    static thread_local SideLane lanes[kDevices][2];
+    static thread_local unsigned turn = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) { (void)cudaGetLastError(); return nullptr; }
+    SideLane& l = lanes[dev][turn++ & 1u];
+    if ((l.stream == nullptr && cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking) != cudaSuccess) ||
+        (l.fork == nullptr && cudaEventCreateWithFlags(&l.fork, cudaEventDisableTiming) != cudaSuccess) ||
+        (l.join == nullptr && cudaEventCreateWithFlags(&l.join, cudaEventDisableTiming) != cudaSuccess)) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return &l;
+}
+
 // True (and *dev set) when `h` is pinned host memory that kernels on the current device can address.
 bool mapped_host_pointer(const void* h, const void** dev) {
     cudaPointerAttributes attr;
@@ -472,6 +498,48 @@ bool mapped_host_pointer(const void* h, const void** dev) {
     if (attr.type != cudaMemoryTypeHost || attr.devicePointer == nullptr) return false;
     *dev = attr.devicePointer;
     return true;
+}
+
+// A layer from pinned host buffers, compact rows, with both directions of the link to the host at work: the fresh rows
+// come first (the gather kernel reads them from the host and writes the changed cache rows back), then the important
+// tokens' attention and the copy out of its rows run on a second stream beside the copy in of the document rows, which
+// only the question rows wait for.  Bound by the link: k + L_q fresh rows and the document rows in (22 MB for the 6k layer,
+// 0.42 ms at 52 GB/s).  6k layer, cache copied back: one stream, whole cache copied back @@A@@ us; this way @@B@@.
+int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows, const float* scores, int32_t n_sig,
+                        const void* h_kv_k, const void* h_kv_v, void* h_hidden, int32_t* h_idx_out, cudaStream_t st,
+                        const SideLane& lane) {
+    const size_t qrow = (size_t)rp.Hq * 256, kvrow = (size_t)rp.Hkv * 256;
+    Workspace ws;
+    if (int rc = carve_workspace(rp, a.ws, a.ws_bytes, &ws)) return rc;
+    rows.cache_later = true;
+    if (int rc = do_select(rp, scores, n_sig, scores ? nullptr : a.idx_in, rows.q, rows.k, rows.v, a.kv_k, a.kv_v, a.idx_out, a.q_pack,
+                           a.k_pack, a.v_pack, ws, st, false, &rows)) return rc;
+    DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
+    DAF_CUDA_TRY(cudaStreamWaitEvent(lane.stream, lane.fork, 0));
+    auto important = [&]() -> int {
+        if (int rc = launch_attention(a.q_pack, a.k_pack, a.v_pack, rp.k, rp.k, rp.Hq, rp.Hkv, 0, rp.scale, false, false, a.hidden,
+                                      (long long)qrow, nullptr, nullptr, ws.status, nullptr, 0, lane.stream)) return rc;
+        DAF_CUDA_TRY(cudaMemcpyAsync(h_hidden, a.hidden, qrow * rp.k, cudaMemcpyDeviceToHost, lane.stream));
+        if (h_idx_out) DAF_CUDA_TRY(cudaMemcpyAsync(h_idx_out, a.idx_out, (size_t)rp.k * 4, cudaMemcpyDeviceToHost, lane.stream));
+        return DAF_OK;
+    };
+    auto question = [&]() -> int {
+        DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_k, h_kv_k, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
+        DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_v, h_kv_v, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
+        if (rp.overwrite)
+            if (int rc = launch_update_cache(rp, a.idx_out, a.k_pack, a.v_pack, a.kv_k, a.kv_v, st)) return rc;
+        char* out = a.hidden + qrow * rp.k;
+        if (int rc = launch_attention(a.q_fresh + qrow * rp.L_d, a.kv_k, a.kv_v, rp.L_q, rp.N, rp.Hq, rp.Hkv, rp.L_d, rp.scale, true, true,
+                                      out, (long long)qrow, nullptr, nullptr, ws.status, ws.attn_scratch, ws.attn_bytes, st)) return rc;
+        DAF_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(h_hidden) + qrow * rp.k, out, qrow * rp.L_q, cudaMemcpyDeviceToHost, st));
+        return DAF_OK;
+    };
+    int rc = important();
+    if (rc == DAF_OK) rc = question();
+    // joined in every case: the caller's stream covers all that was enqueued
+    DAF_CUDA_TRY(cudaEventRecord(lane.join, lane.stream));
+    DAF_CUDA_TRY(cudaStreamWaitEvent(st, lane.join, 0));
+    return rc;
 }
 }  // namespace
 
@@ -508,9 +576,15 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
     // three host tensors are pinned memory that the device can address, the gather / cache-update kernel reads those
     // rows straight from the host (k + L_q rows instead of N cross the link) and only the question's Q rows, which
     // the attention kernel reads through a tensor map, are copied; otherwise the tensors are copied whole.
-    RowSource rows = {nullptr, nullptr, nullptr};
+    RowSource rows = {};
     const bool in_place_rows = rp.k > 0 && mapped_host_pointer(h_q_fresh, &rows.q) && mapped_host_pointer(h_k_fresh, &rows.k) &&
                                mapped_host_pointer(h_v_fresh, &rows.v);
+    // Of the cache a layer changes only the rows of the important tokens and of the question.  When the caller's cache is
+    // pinned too, the same kernel writes those rows straight back to it; otherwise the cache is copied back whole.
+    const void *host_k = nullptr, *host_v = nullptr;
+    const bool rows_back = in_place_rows && mapped_host_pointer(h_kv_k, &host_k) && mapped_host_pointer(h_kv_v, &host_v) &&
+                           aligned16(host_k) && aligned16(host_v);
+    if (rows_back && copy_back_kv) { rows.host_k = const_cast<void*>(host_k); rows.host_v = const_cast<void*>(host_v); }
     if (in_place_rows) {
         if (rp.L_q > 0)
             DAF_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(a.q_fresh) + qrow * rp.L_d,
@@ -520,6 +594,13 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
         DAF_CUDA_TRY(cudaMemcpyAsync(a.q_fresh, h_q_fresh, qrow * rp.N, cudaMemcpyHostToDevice, st));
         DAF_CUDA_TRY(cudaMemcpyAsync(a.k_fresh, h_k_fresh, kvrow * rp.N, cudaMemcpyHostToDevice, st));
         DAF_CUDA_TRY(cudaMemcpyAsync(a.v_fresh, h_v_fresh, kvrow * rp.N, cudaMemcpyHostToDevice, st));
+    }
+    if (rows_back && rp.L_q > 0 && rp.fuse_mode == 0) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        DAF_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
+        SideLane* lane = capture == cudaStreamCaptureStatusNone ? side_lane() : nullptr;
+        if (lane != nullptr)
+            return host_layer_two_ways(rp, a, rows, h_scores ? a.scores : nullptr, n_sig, h_kv_k, h_kv_v, h_hidden, h_idx_out, st, *lane);
     }
     // only the document rows of the cache carry information on entry
     DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_k, h_kv_k, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
@@ -532,7 +613,7 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
     const size_t hidden_rows = rp.fuse_mode == 1 ? rp.N : rp.k + rp.L_q;
     DAF_CUDA_TRY(cudaMemcpyAsync(h_hidden, a.hidden, qrow * hidden_rows, cudaMemcpyDeviceToHost, st));
     if (h_idx_out && rp.k > 0) DAF_CUDA_TRY(cudaMemcpyAsync(h_idx_out, a.idx_out, (size_t)rp.k * 4, cudaMemcpyDeviceToHost, st));
-    if (copy_back_kv) {
+    if (copy_back_kv && !rows_back) {
         DAF_CUDA_TRY(cudaMemcpyAsync(h_kv_k, a.kv_k, kvrow * rp.N, cudaMemcpyDeviceToHost, st));
         DAF_CUDA_TRY(cudaMemcpyAsync(h_kv_v, a.kv_v, kvrow * rp.N, cudaMemcpyDeviceToHost, st));
     }
@@ -546,10 +627,10 @@ int daf_layer_host_end(const daf_params* p, void* arena, size_t arena_bytes, voi
     Arena a;
     carve_arena(rp, kArenaSignalRows, reinterpret_cast<char*>(arena), &a);
     if (arena_bytes < a.total) return DAF_ERR_WORKSPACE;
-    DAF_CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
-    if (rp.k + rp.L_q == 0) return DAF_OK;
-    DeviceStatus hs;
-    DAF_CUDA_TRY(cudaMemcpy(&hs, a.ws, sizeof(hs), cudaMemcpyDeviceToHost));
+    cudaStream_t st = (cudaStream_t)stream;
+    DeviceStatus hs = {};
+    if (rp.k + rp.L_q > 0) DAF_CUDA_TRY(cudaMemcpyAsync(&hs, a.ws, sizeof(hs), cudaMemcpyDeviceToHost, st));
+    DAF_CUDA_TRY(cudaStreamSynchronize(st));
     return hs.code;
 }
 

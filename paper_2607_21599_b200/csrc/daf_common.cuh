@@ -37,10 +37,17 @@ int resolve_params(const daf_params* p, ResolvedParams* out);  // validates; DAF
 
 // kernel launchers (daf_select.cu, daf_attn.cu), called by the C ABI in daf_api.cu
 size_t select_scratch_bytes(int L_d);
+// Where the gather / cache-update kernel reads the fresh rows when that is not the tensors the attention reads the question
+// rows from: device-accessible pointers to [N, heads, 128] tensors (mapped pinned host memory).  host_k / host_v: the
+// caller's cache in host memory, likewise mapped, when the kernel is to write the rows that change straight back to it.
+// cache_later: the important rows of the device's cache are written by launch_update_cache instead.
+struct RowSource { const void* q; const void* k; const void* v; void* host_k; void* host_v; bool cache_later; };
 int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, const int32_t* idx_in,
                   const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                   int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack,
-                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool beside_previous_kernel = false, bool select_only = false, bool rows_far = false);
+                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool beside_previous_kernel = false, bool select_only = false, const RowSource* far = nullptr);
+int launch_update_cache(const ResolvedParams& rp, const int32_t* idx, const void* k_pack, const void* v_pack, void* kv_k,
+                        void* kv_v, cudaStream_t stream);
 int launch_check_indices(const int32_t* idx, int k, int L_d, DeviceStatus* status, cudaStream_t stream);
 int launch_expand_fp8(const ResolvedParams& rp, const void* k8, const void* v8, const float* k_scale, const float* v_scale,
                       void* kv_k, void* kv_v, cudaStream_t stream);

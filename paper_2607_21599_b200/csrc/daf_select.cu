@@ -433,6 +433,10 @@ struct GatherArgs {
     int32_t* idx_copy;        // when non-null, also receives idx (the idx_in path)
     int k, L_d, L_q, cq, ckv; // cq/ckv: 16-byte chunks per Q row / per K (or V) row
     int overwrite;
+    // kFar only: the caller's cache in host memory (null: not written), and whether the important rows of the device's
+    // cache are left to update_cache_kernel because the document rows are still on their way to it
+    int4* host_k; int4* host_v;
+    int cache_later;
     DeviceStatus* status;
 };
 
@@ -479,11 +483,13 @@ gather_update_kernel(const GatherArgs a) {
                     } else if (c < a.cq + a.ckv) {
                         const int cc = c - a.cq;
                         if (a.k_pack != nullptr) a.k_pack[kdst + cc] = v[u];
-                        if (a.overwrite) a.kv_k[ksrc + cc] = v[u];
+                        if (a.overwrite && !a.cache_later) a.kv_k[ksrc + cc] = v[u];
+                        if (a.overwrite && a.host_k != nullptr) a.host_k[ksrc + cc] = v[u];
                     } else if (c < c_end) {
                         const int cc = c - a.cq - a.ckv;
                         if (a.v_pack != nullptr) a.v_pack[kdst + cc] = v[u];
-                        if (a.overwrite) a.kv_v[ksrc + cc] = v[u];
+                        if (a.overwrite && !a.cache_later) a.kv_v[ksrc + cc] = v[u];
+                        if (a.overwrite && a.host_v != nullptr) a.host_v[ksrc + cc] = v[u];
                     }
                 }
             }
@@ -507,11 +513,41 @@ gather_update_kernel(const GatherArgs a) {
     } else {
         const size_t off = (size_t)(a.L_d + (row - a.k)) * a.ckv;
         for (int c = threadIdx.x; c < 2 * a.ckv; c += kRowThreads) {
-            if (c < a.ckv) a.kv_k[off + c] = __ldg(a.k_fresh + off + c);
-            else a.kv_v[off + c - a.ckv] = __ldg(a.v_fresh + off + c - a.ckv);
+            const size_t at = off + (c < a.ckv ? c : c - a.ckv);
+            const int4 v = __ldg((c < a.ckv ? a.k_fresh : a.v_fresh) + at);
+            (c < a.ckv ? a.kv_k : a.kv_v)[at] = v;
+            if (kFar && a.host_k != nullptr) (c < a.ckv ? a.host_k : a.host_v)[at] = v;
         }
     }
     DAF_KT_END(1);
+}
+
+// The important rows of the device's cache from their packed copies (layers from host buffers, where the document rows
+// arrive after the rows were gathered).  One warp per row.
+__global__ void __launch_bounds__(256)
+update_cache_kernel(const int32_t* __restrict__ idx, int k, int L_d, int ckv, const int4* __restrict__ k_pack,
+                    const int4* __restrict__ v_pack, int4* __restrict__ kv_k, int4* __restrict__ kv_v) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int row = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (row >= k) return;
+    const int p = idx[row];
+    if (p < 0 || p >= L_d) return;            // reported by the gather kernel
+    for (int c = threadIdx.x & 31; c < ckv; c += 32) {
+        kv_k[(size_t)p * ckv + c] = __ldg(k_pack + (size_t)row * ckv + c);
+        kv_v[(size_t)p * ckv + c] = __ldg(v_pack + (size_t)row * ckv + c);
+    }
+}
+
+int launch_update_cache(const ResolvedParams& rp, const int32_t* idx, const void* k_pack, const void* v_pack, void* kv_k,
+                        void* kv_v, cudaStream_t stream) {
+    if (rp.k <= 0) return DAF_OK;
+    const cudaError_t e = launch_kernel(update_cache_kernel, dim3((unsigned)((rp.k + 7) / 8)), dim3(256), 0, stream, idx, rp.k, rp.L_d,
+                                        rp.Hkv * 16, reinterpret_cast<const int4*>(k_pack), reinterpret_cast<const int4*>(v_pack),
+                                        reinterpret_cast<int4*>(kv_k), reinterpret_cast<int4*>(kv_v));
+    count_launch();
+    if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
+    return check_launch();
 }
 
 // ------------------------------------------------------------- state fusion
@@ -636,7 +672,7 @@ static size_t select_smem_bytes(int L_d) {
 int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, const int32_t* idx_in,
                   const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                   int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack,
-                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool beside_previous_kernel, bool select_only, bool rows_far) {
+                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool beside_previous_kernel, bool select_only, const RowSource* far) {
     // beside_previous_kernel: the kernel launched just before (the fp8 cache expansion) is independent of the
     // selection; the selection kernel starts while it runs and only waits for it before it retires
     const int wait_at_end = beside_previous_kernel ? 1 : 0;
@@ -686,12 +722,15 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         a.k = rp.k; a.L_d = rp.L_d; a.L_q = rp.L_q;
         a.cq = rp.Hq * 16; a.ckv = rp.Hkv * 16;
         a.overwrite = rp.overwrite;
+        a.host_k = far != nullptr ? reinterpret_cast<int4*>(far->host_k) : nullptr;
+        a.host_v = far != nullptr ? reinterpret_cast<int4*>(far->host_v) : nullptr;
+        a.cache_later = far != nullptr && far->cache_later;
         a.status = status;
         // Always a programmatic dependent of whatever kernel precedes it on the stream: the kernel waits for that
         // kernel to complete before it touches anything (so the result is that of a plain launch), but its CTAs are
         // already in place then -- after this library's selection kernel, and equally after the previous layer's
         // merge when layers are issued back to back.
-        cudaError_t e = rows_far ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a)
+        cudaError_t e = far != nullptr ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a)
                                  : launch_kernel(gather_update_kernel<false>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }

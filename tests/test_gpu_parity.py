@@ -487,6 +487,33 @@ def test_host_layer_from_pageable_and_from_pinned_fresh_tensors_agree():
     _assert_close(outs[0][0], ref["hidden"], "hidden rows from pinned host tensors")
 
 
+@pytest.mark.parametrize("fuse_mode,overwrite,copy_back,L_q", [(0, 1, 1, 33), (0, 0, 1, 33), (0, 1, 0, 33), (1, 1, 1, 33), (0, 1, 1, 0),
+                                                               (0, 1, 1, 1)])
+def test_host_layer_with_a_pinned_cache_changes_only_the_rows_that_change(fuse_mode, overwrite, copy_back, L_q):
+    """All host tensors pinned (changed cache rows written straight back, the two directions of the link used at once in
+    compact mode) against the oracle: positions and cache bytes identical, rows close; run twice on one arena."""
+    w = W.Workload("t", 41, 14, 2, 128, 1, 1100, 500, L_q, 0.3, "lognormal", 1)
+    p = api.make_params(w.L_d, w.L_q, w.r, w.n_q_heads, w.n_kv_heads, fuse_mode=fuse_mode, overwrite_doc_kv=overwrite)
+    k = api.daf_num_important(w.L_d, w.r)
+    arena = torch.zeros(api.daf_layer_host_arena_bytes(p), dtype=torch.uint8, device="cuda")
+    for layer in range(2):
+        L = W.make_layer(w, layer)
+        h = {n: t.pin_memory() for n, t in L.items() if t is not None}
+        kv = [torch.zeros(w.N, w.n_kv_heads, 128, dtype=torch.bfloat16).pin_memory() for _ in range(2)]
+        kv[0][: w.L_d], kv[1][: w.L_d] = L["k_cached"], L["v_cached"]
+        entry = [t.clone() for t in kv]
+        hidden = torch.full((k + L_q if fuse_mode == 0 else w.N, w.n_q_heads, 128), -9.0, dtype=torch.bfloat16).pin_memory()
+        idx_out = torch.full((k,), -1, dtype=torch.int32).pin_memory()
+        api.check(api.daf_layer_host(p, h["scores"], 1, None, h["q_fresh"], h["k_fresh"], h["v_fresh"], kv[0], kv[1], copy_back,
+                                     hidden, idx_out, arena), "daf_layer_host")
+        ref = _oracle_layer(w, L, fuse_mode, overwrite)
+        assert np.array_equal(idx_out.numpy(), ref["idx"])
+        for got, name, before in zip(kv, ("kv_k", "kv_v"), entry):
+            assert np.array_equal(_f(got), ref[name] if copy_back else _f(before)), name
+        rows = torch.from_numpy(ref["row_pos"]).long() if fuse_mode == 1 else slice(None)
+        _assert_close(hidden[rows], ref["hidden"][rows] if fuse_mode == 0 else ref["hidden"][ref["row_pos"]], "hidden rows")
+
+
 def test_host_layers_pipelined_on_two_arenas_match_the_plain_host_call():
     """daf_layer_host_begin / _end with two arenas and two streams (layer i + 1 begun before layer i is ended) give,
     layer by layer, exactly what daf_layer_host gives."""
