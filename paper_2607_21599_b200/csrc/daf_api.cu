@@ -504,7 +504,7 @@ bool mapped_host_pointer(const void* h, const void** dev) {
 // come first (the gather kernel reads them from the host and writes the changed cache rows back), then the important
 // tokens' attention and the copy out of its rows run on a second stream beside the copy in of the document rows, which
 // only the question rows wait for.  Bound by the link: k + L_q fresh rows and the document rows in (22 MB for the 6k layer,
-// 0.42 ms at 52 GB/s).  6k layer, cache copied back: one stream, whole cache copied back @@A@@ us; this way @@B@@.
+// 0.42 ms at 52 GB/s).  6k layer, cache copied back: one stream, whole cache copied back 865 us; this way 577.
 int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows, const float* scores, int32_t n_sig,
                         const void* h_kv_k, const void* h_kv_v, void* h_hidden, int32_t* h_idx_out, cudaStream_t st,
                         const SideLane& lane) {
