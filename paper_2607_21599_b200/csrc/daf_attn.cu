@@ -22,9 +22,9 @@
 namespace daf {
 
 constexpr int kBlockM = 128;            // rows per query tile
-constexpr int kBlockN = 128;            // keys per KV tile
+constexpr int kBlockN = 128;            // tensor-memory columns of the logits: two sub-steps of 64 keys
 constexpr int kD = 128;                 // head_dim
-constexpr int kTileBytes = kBlockN * kD * 2;      // 32 KB: one Q tile, or K (or V) of 128 keys
+constexpr int kTileBytes = kBlockN * kD * 2;      // 32 KB: one Q tile, or two sub-steps of K (or V)
 constexpr int kHalfBytes = kTileBytes / 2;        // one 64-column half (128-byte rows)
 constexpr int kMaxSplits = 32;
 constexpr int kNumSMsDefault = 148;    // B200; the planners ask the device (num_sms below)
@@ -52,9 +52,9 @@ struct SegArgs {
     const int32_t* kv_idx;
     int kv_src_rows, kv_heads;
     // Work items.  A CTA owns one token block (a unit) of one head block, and one of n_splits KV ranges of
-    // tiles_per_split tiles.
+    // steps_per_split sub-steps (64 keys each).
     int head_blocks, n_units;
-    int n_splits, tiles_per_split;
+    int n_splits, steps_per_split;
     int n_items;           // head_blocks * n_units * n_splits
     float scale;        // softmax scale
     float scale_log2;   // scale * log2(e)
@@ -214,10 +214,10 @@ __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
         unit = n_units - 1 - rest % n_units;
         split = rest / n_units;
     }
-    const int tps = DAF_SEG(tiles_per_split);
+    const int steps = DAF_SEG(steps_per_split);
     a.seg_id = seg_id; a.hb = hb; a.unit = unit;
-    a.j_begin = split * tps;
-    a.j_end = a.j_begin + tps;
+    a.j_begin = split * steps;
+    a.j_end = a.j_begin + steps;
     a.item_splits = DAF_SEG(n_splits);
     a.part_row0 = (long long)split * a.n_q;
 }
@@ -438,7 +438,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     const int h0 = a.hb * a.Gp;
     const int g_kv = h0 / a.G;
     const int t0 = a.unit * a.Tt;
-    const int key_begin = a.j_begin * kBlockN;
+    const int key_begin = a.j_begin * kSubN;
     // kGatherKV: the launch has a problem whose K/V rows the producer warp fetches in place through an index (k_src
     // non-null); a form of its own, so that the plain form carries none of that code
     const __nv_bfloat16* const k_src = kGatherKV ? DAF_SEG(k_src) : nullptr;
@@ -541,7 +541,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         const int max_tok = min(a.n_q, t0 + a.Tt) - 1;
         const long long last_key = a.q_pos ? (long long)__ldg(a.q_pos + max_tok) : (long long)max_tok + a.causal_off;
         long long hi = min((long long)a.n_kv, last_key + 1);
-        hi = min(hi, (long long)a.j_end * kBlockN);
+        hi = min(hi, (long long)a.j_end * kSubN);
         if (hi > key_begin) n_t = (int)((hi - key_begin + kSubN - 1) / kSubN);
     }
     if (warp == 4 && lane == 0) {
@@ -835,7 +835,12 @@ struct CombineArgs {
     __nv_bfloat16* out; long long out_row_stride; const int32_t* dst_rows; float* lse;
 };
 
-__global__ void __launch_bounds__(256)
+// kMost: the largest number of partials a launch of this form merges.  Bound by latency: all of a row's partials and their
+// log-sum-exps are requested at once (a second round is a second trip to L2: as eight and then four by four, 24 tokens of 28
+// heads over 14k keys, 22 ranges, took 22.4 us with their attention, at once 19.8; 28 layers of 6k, 7 ranges, 747 against 726).  Two CTAs per SM are asked for so that
+// the compiler has the registers to keep them all under way.
+template <int kMost>
+__global__ void __launch_bounds__(256, 2)
 attn_combine_kernel(const CombineArgs a) {
     DAF_KT_BEGIN(2);
     pdl_wait();                // partial results come from the attention kernel launched just before
@@ -844,49 +849,30 @@ attn_combine_kernel(const CombineArgs a) {
     const int lane = threadIdx.x & 31;
     const int Hq = a.Hq, n_q = a.n_q, n_splits = a.n_splits;
     if (row >= n_q * Hq) return;
-    const int tok = row / Hq, head = row % Hq;
-    const size_t first = row, stride = (size_t)n_q * Hq;      // in rows of the partial arrays
-    const float* part_o = a.part_o;
-    const float* part_lse = a.part_lse;
-    // lane s holds the log-sum-exp of partial s (at most 32 of them), so all of them are fetched at once;
-    // the first eight partial rows are requested in the same breath, before the weights are known
-    const float4* src = reinterpret_cast<const float4*>(part_o + first * kD) + lane;
-    const float my_lse = lane < n_splits ? part_lse[first + (size_t)lane * stride] : -INFINITY;
-    float4 head_v[8];
+    const size_t stride = (size_t)n_q * Hq;      // rows from one partial to the next
+    const float* const lse_src = a.part_lse + row;
+    const float4* const src = reinterpret_cast<const float4*>(a.part_o + (size_t)row * kD) + lane;
+    const int tok = row / Hq, head = row - tok * Hq;
+    float4 v[kMost];
+    float mx, wsum = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    // lane s holds the log-sum-exp of partial s
+    const float my_lse = lane < n_splits ? __ldcs(lse_src + (size_t)lane * stride) : -INFINITY;
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-        head_v[u] = u < n_splits ? __ldcs(src + (size_t)u * stride * (kD / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float mx = my_lse;
+    for (int u = 0; u < kMost; ++u)
+        v[u] = u < n_splits ? __ldcs(src + (size_t)u * stride * (kD / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const long long drow = a.dst_rows ? (long long)a.dst_rows[tok] : (long long)tok;
+    mx = my_lse;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    const float my_w = (my_lse == -INFINITY) ? 0.f : __expf(my_lse - mx);
-    float wsum = my_w;
+    const float my_w = my_lse == -INFINITY ? 0.f : __expf(my_lse - mx);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xFFFFFFFFu, wsum, o);
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < kMost; ++u) {
         const float w = __shfl_sync(0xFFFFFFFFu, my_w, u);     // zero for u >= n_splits
-        acc.x += w * head_v[u].x; acc.y += w * head_v[u].y; acc.z += w * head_v[u].z; acc.w += w * head_v[u].w;
-    }
-    int s = 8;
-    for (; s + 4 <= n_splits; s += 4) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldcs(src + (size_t)(s + u) * stride * (kD / 4));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float w = __shfl_sync(0xFFFFFFFFu, my_w, s + u);
-            acc.x += w * v[u].x; acc.y += w * v[u].y; acc.z += w * v[u].z; acc.w += w * v[u].w;
-        }
-    }
-    for (; s < n_splits; ++s) {
-        const float4 v = __ldcs(src + (size_t)s * stride * (kD / 4));
-        const float w = __shfl_sync(0xFFFFFFFFu, my_w, s);
-        acc.x += w * v.x; acc.y += w * v.y; acc.z += w * v.z; acc.w += w * v.w;
+        wsum += w;
+        acc.x += w * v[u].x; acc.y += w * v[u].y; acc.z += w * v[u].z; acc.w += w * v[u].w;
     }
     const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-    const long long drow = a.dst_rows ? (long long)a.dst_rows[tok] : (long long)tok;
     uint2 w2;
     w2.x = pack_bf16(acc.x * inv, acc.y * inv);
     w2.y = pack_bf16(acc.z * inv, acc.w * inv);
@@ -1007,9 +993,39 @@ static int causal_heads_per_tile(int n, int G) {
     return causal_substeps(n, G, G) <= causal_substeps(n, G, 1) ? G : 1;
 }
 
+// Into how many sub-steps per range the keys of the question rows are cut when they have the GPU to themselves: `total`
+// sub-steps, `ctas` = token blocks x head blocks.  The ranges have to fill the CTA slots (two per SM), but each costs its
+// set-up, and the partial rows (`mb` megabytes per range) a merge; the last range takes what is left over, and a few short
+// items may follow others in a slot.  Constants measured by forced plans, question rows on their own (2k to 32k
+// keys): a sub-step takes 0.82 us in a CTA alone on its SM and 1.03 beside another.  64 tokens of 28 heads on 4 over 32k
+// keys: 18 ranges of 15 x 128 keys 42.4 us, 19 of 14 x 128 40.1; 79 tokens of 40 heads on 8 over 2181: 9 ranges (as many as
+// there are slots for) 18.4, 6 ranges 16.5.
+static int question_steps_per_split(int total, int ctas, float mb) {
+    constexpr float kItemUs = 4.4f, kAloneUs = 0.82f, kPairUs = 1.03f, kMergeUs = 4.5f, kMergeUsPerMB = 0.25f;
+    const int sms = num_sms(), slots = 2 * sms;
+    float best_us = 0.f;
+    int best = total;
+    for (int n = 1; n <= kMaxSplits && n <= total; ++n) {
+        const int even = (total + n - 1) / n;
+        for (int j = 0; j < 8; ++j) {
+            const int steps = even + j * (even / 32 + 1);
+            if ((total + steps - 1) / steps != n) break;
+            const int rest = total - (n - 1) * steps, full = ctas * (rest == steps ? n : n - 1), items = ctas * n;
+            float us;
+            if (items <= sms) us = kItemUs + kAloneUs * (float)steps;
+            else if (items <= slots) us = kItemUs + kPairUs * (float)steps;
+            else if (full <= slots && 2 * (slots - full) >= items - full)     // the short items fit in behind one another
+                us = fmaxf(kItemUs + kPairUs * (float)steps, 2.f * (kItemUs + kPairUs * (float)rest));
+            else us = (float)((items + slots - 1) / slots) * (kItemUs + kPairUs * (float)steps);
+            if (n > 1) us += kMergeUs + kMergeUsPerMB * mb * (float)n;
+            if (best_us == 0.f || us < best_us) { best_us = us; best = steps; }
+        }
+    }
+    return best;
+}
+
 // How a single problem is cut into CTAs: one per (head block, token block), and for the question rows,
 // where there are few query tiles and a long KV axis, also per range of the KV axis.
-
 AttnPlan plan_attention(int n_q, int n_kv, int Hq, int G, int causal_off, bool pack_group, bool allow_split) {
     AttnPlan pl;
     pl.Gp = pack_group ? G : 1;
@@ -1019,19 +1035,18 @@ AttnPlan plan_attention(int n_q, int n_kv, int Hq, int G, int causal_off, bool p
     pl.head_blocks = Hq / pl.Gp;
     long long kv_hi = (long long)n_q - 1 + causal_off + 1;
     if (kv_hi > n_kv) kv_hi = n_kv;
-    const int total_tiles = kv_hi > 0 ? (int)((kv_hi + kBlockN - 1) / kBlockN) : 0;
+    const int total = kv_hi > 0 ? (int)((kv_hi + kSubN - 1) / kSubN) : 0;
     pl.n_splits = 1;
-    pl.tiles_per_split = total_tiles > 0 ? total_tiles : 1;
-    if (allow_split && total_tiles > 1) {
+    pl.steps_per_split = total > 0 ? total : 1;
+    if (allow_split && total > 1) {
+        // a loop over layers or questions asks for the same shape over and over: each thread keeps its last answer
+        struct Last { int total, ctas, n_q, Hq, steps; };
+        static thread_local Last last = {0, 0, 0, 0, 0};
         const int ctas = pl.n_tb * pl.head_blocks;
-        const int slots = num_sms() * 2;
-        int want = ctas > 0 ? slots / ctas : 1;
-        if (want > kMaxSplits) want = kMaxSplits;
-        if (want > total_tiles) want = total_tiles;
-        if (want > 1) {
-            pl.tiles_per_split = (total_tiles + want - 1) / want;
-            pl.n_splits = (total_tiles + pl.tiles_per_split - 1) / pl.tiles_per_split;
-        }
+        if (last.total != total || last.ctas != ctas || last.n_q != n_q || last.Hq != Hq)
+            last = Last{total, ctas, n_q, Hq, question_steps_per_split(total, ctas, (float)n_q * (float)Hq * 516e-6f)};
+        pl.steps_per_split = last.steps;
+        pl.n_splits = (total + pl.steps_per_split - 1) / pl.steps_per_split;
     }
     return pl;
 }
@@ -1068,10 +1083,11 @@ bool operator<(const JointShape& a, const JointShape& b) {
 
 // Fills the fields of `jp` that follow from n_splits_q.
 void set_choice(JointPlan& jp, int n_splits_q, int L_q, int L_d, int Hq) {
-    const int tiles_q = (L_d + L_q + kBlockN - 1) / kBlockN;
+    const int steps_q = (L_d + L_q + kSubN - 1) / kSubN;
     if (n_splits_q < 1) n_splits_q = 1;
-    jp.tiles_per_split_q = (tiles_q + n_splits_q - 1) / n_splits_q;
-    jp.n_splits_q = (tiles_q + jp.tiles_per_split_q - 1) / jp.tiles_per_split_q;
+    jp.steps_per_split_q = (steps_q + n_splits_q - 1) / n_splits_q;
+    if (jp.steps_per_split_q >= 8) jp.steps_per_split_q += jp.steps_per_split_q & 1;    // whole 128 keys: 32k 415 us, 419 with odd cuts
+    jp.n_splits_q = (steps_q + jp.steps_per_split_q - 1) / jp.steps_per_split_q;
     jp.items_q = jp.head_blocks_q * jp.n_tb_q * jp.n_splits_q;
     jp.part_bytes_q = attn_partial_bytes(L_q, Hq, jp.n_splits_q);
 }
@@ -1095,8 +1111,8 @@ float predict_us(const JointPlan& jp, int k, int L_q, int L_d) {
     for (int s = 0; s < jp.n_splits_q; ++s)
         for (int u = jp.n_tb_q - 1; u >= 0; --u) {
             const int last_tok = (u + 1) * jp.Tt_q < L_q ? (u + 1) * jp.Tt_q : L_q;
-            const int begin = s * jp.tiles_per_split_q * kBlockN;
-            int end = begin + jp.tiles_per_split_q * kBlockN;
+            const int begin = s * jp.steps_per_split_q * kSubN;
+            int end = begin + jp.steps_per_split_q * kSubN;
             if (end > L_d + last_tok) end = L_d + last_tok;
             if (end > begin) run(jp.head_blocks_q, (end - begin + kSubN - 1) / kSubN);
         }
@@ -1132,7 +1148,7 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     jp.Tt_q = kBlockM / jp.Gp_q;
     jp.n_tb_q = (L_q + jp.Tt_q - 1) / jp.Tt_q;
     jp.head_blocks_q = Hq / jp.Gp_q;
-    const int tiles_q = (L_d + L_q + kBlockN - 1) / kBlockN;
+    const int steps_q = (L_d + L_q + kSubN - 1) / kSubN;
     if (forced) {
         set_choice(jp, g_force_splits_q, L_q, L_d, Hq);
         g_last_predicted_us = predict_us(jp, k, L_q, L_d);
@@ -1140,12 +1156,12 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     }
     JointPlan best = jp;
     float best_us = -1.f;
-    int last_tps = -1;
-    for (int n = 1; n <= kMaxSplits && n <= tiles_q; ++n) {
+    int last_steps = -1;
+    for (int n = 1; n <= kMaxSplits && n <= steps_q; ++n) {
         JointPlan cand = jp;
         set_choice(cand, n, L_q, L_d, Hq);
-        if (cand.tiles_per_split_q == last_tps) continue;
-        last_tps = cand.tiles_per_split_q;
+        if (cand.steps_per_split_q == last_steps) continue;
+        last_steps = cand.steps_per_split_q;
         const float us = predict_us(cand, k, L_q, L_d);
         if (best_us < 0.f || us < best_us) { best_us = us; best = cand; }
     }
@@ -1182,7 +1198,14 @@ static void fill_problem(SegArgs* s, int n_q, int n_kv, int Hq, int G, int Gp, i
 static int launch_combine(const SegArgs& s, cudaStream_t stream) {
     if (s.n_splits <= 1) return DAF_OK;
     const CombineArgs c{s.part_o, s.part_lse, s.n_q, s.Hq, s.n_splits, s.out, s.out_row_stride, s.dst_rows, s.lse};
-    const cudaError_t e = launch_kernel(attn_combine_kernel, dim3((unsigned)((s.n_q * s.Hq + 7) / 8)), dim3(256), 0, stream, c);
+    const dim3 grid((unsigned)((s.n_q * s.Hq + 7) / 8));
+    auto* kernel = s.n_splits <= 4    ? attn_combine_kernel<4>
+                   : s.n_splits <= 8  ? attn_combine_kernel<8>
+                   : s.n_splits <= 12 ? attn_combine_kernel<12>
+                   : s.n_splits <= 16 ? attn_combine_kernel<16>
+                   : s.n_splits <= 24 ? attn_combine_kernel<24>
+                                      : attn_combine_kernel<kMaxSplits>;
+    const cudaError_t e = launch_kernel(kernel, grid, dim3(256), 0, stream, c);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
@@ -1191,12 +1214,12 @@ static int launch_combine(const SegArgs& s, cudaStream_t stream) {
 int launch_attention(const void* q, const void* k, const void* v, int n_q, int n_kv, int Hq, int Hkv, int causal_off,
                      float scale, bool pack_group, bool allow_split, void* out, long long out_row_stride_bytes,
                      const int32_t* dst_rows, float* lse, DeviceStatus* status, void* scratch, size_t scratch_bytes,
-                     cudaStream_t stream, const int32_t* q_pos) {
+                     cudaStream_t stream, const int32_t* q_pos, const AttnPlan* plan) {
     if (n_q <= 0) return DAF_OK;
     const int G = Hq / Hkv;
     // a causal problem over its own keys chooses how many heads share a tile; the question rows always pack the group
     if (!pack_group && q_pos == nullptr && causal_off == 0) pack_group = causal_heads_per_tile(n_q, G) > 1;
-    AttnPlan pl = plan_attention(n_q, n_kv, Hq, G, causal_off, pack_group, allow_split);
+    const AttnPlan pl = plan != nullptr ? *plan : plan_attention(n_q, n_kv, Hq, G, causal_off, pack_group, allow_split);
     const size_t need = attn_partial_bytes(n_q, Hq, pl.n_splits);
     if (need > scratch_bytes) return DAF_ERR_WORKSPACE;
 
@@ -1217,7 +1240,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     fill_problem(&s, n_q, n_kv, Hq, G, pl.Gp, causal_off, q_pos, scale, out, out_row_stride_bytes, dst_rows, lse);
     s.out_tiled = out_tiled ? 1 : 0;
     s.n_units = pl.n_tb;
-    s.n_splits = pl.n_splits; s.tiles_per_split = pl.tiles_per_split;
+    s.n_splits = pl.n_splits; s.steps_per_split = pl.steps_per_split;
     s.n_items = pl.head_blocks * pl.n_tb * pl.n_splits;
     s.part_o = reinterpret_cast<float*>(scratch);
     s.part_lse = pl.n_splits > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(scratch) +
@@ -1301,7 +1324,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     fill_problem(&sq, L_q, N, Hq, G, jp.Gp_q, L_d, nullptr, scale, out_question, out_row_stride_bytes, nullptr, nullptr);
     sq.out_tiled = 1;
     sq.n_units = jp.n_tb_q;
-    sq.n_splits = jp.n_splits_q; sq.tiles_per_split = jp.tiles_per_split_q;
+    sq.n_splits = jp.n_splits_q; sq.steps_per_split = jp.steps_per_split_q;
     sq.n_items = jp.items_q;
     sq.part_o = reinterpret_cast<float*>(sc);
     sq.part_lse = reinterpret_cast<float*>(sc + (size_t)jp.n_splits_q * L_q * Hq * kD * sizeof(float));
@@ -1322,7 +1345,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     }
     si.out_tiled = imp_tiled ? 1 : 0;
     si.n_units = jp.n_tb_i;
-    si.n_splits = 1; si.tiles_per_split = (k + kBlockN - 1) / kBlockN;
+    si.n_splits = 1; si.steps_per_split = (k + kSubN - 1) / kSubN;
     si.n_items = jp.items_i;
     a.joint = 1;
     a.status = status;
@@ -1399,10 +1422,19 @@ extern "C" int daf_qd_attn_static(const daf_params* p, const void* q_question, c
     if (!aligned16(q_question) || !aligned16(kv_k) || !aligned16(kv_v) || !aligned16(out) ||
         out_row_stride_bytes % 16 != 0) return DAF_ERR_ALIGNMENT;
     if (out_row_stride_bytes < (int64_t)rp.Hq * 256) return DAF_ERR_INVALID_ARG;
-    // the fixed array must hold the status word and this problem's split-KV partials
-    const AttnPlan pl = plan_attention(rp.L_q, rp.N, rp.Hq, rp.G, rp.L_d, true, true);
-    const size_t need = kStatusBytes + attn_partial_bytes(rp.L_q, rp.Hq, pl.n_splits);
-    if (need > kStaticScratchBytes) return DAF_ERR_WORKSPACE;   // problem too large for the fixed scratch
+    // The problems served are those whose scratch fits with as many ranges of 128 keys as there are CTA slots for; within
+    // those the planned number of ranges is used, or as many as fit.
+    AttnPlan pl = plan_attention(rp.L_q, rp.N, rp.Hq, rp.G, rp.L_d, true, true);
+    const int tiles = (rp.N + 127) / 128, ctas = pl.n_tb * pl.head_blocks;
+    int want = 2 * num_sms() / ctas;
+    if (want > kMaxSplits) want = kMaxSplits;
+    if (want > tiles) want = tiles;
+    const int per = want > 1 ? (tiles + want - 1) / want : tiles;
+    if (kStatusBytes + attn_partial_bytes(rp.L_q, rp.Hq, (tiles + per - 1) / per) > kStaticScratchBytes) return DAF_ERR_WORKSPACE;
+    while (pl.n_splits > 1 && kStatusBytes + attn_partial_bytes(rp.L_q, rp.Hq, pl.n_splits) > kStaticScratchBytes) {
+        ++pl.steps_per_split;
+        pl.n_splits = ((rp.N + kSubN - 1) / kSubN + pl.steps_per_split - 1) / pl.steps_per_split;
+    }
     void* base = nullptr;
     if (int rc = static_scratch_address(&base)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
@@ -1411,7 +1443,7 @@ extern "C" int daf_qd_attn_static(const daf_params* p, const void* q_question, c
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return launch_attention(q_question, kv_k, kv_v, rp.L_q, rp.N, rp.Hq, rp.Hkv, rp.L_d, rp.scale, true, true, out,
                             out_row_stride_bytes, dst_rows, lse, reinterpret_cast<DeviceStatus*>(base),
-                            reinterpret_cast<char*>(base) + kStatusBytes, kStaticScratchBytes - kStatusBytes, st);
+                            reinterpret_cast<char*>(base) + kStatusBytes, kStaticScratchBytes - kStatusBytes, st, nullptr, &pl);
 }
 
 // Status of the calls made through daf_qd_attn_static on the current device since the last poll: the

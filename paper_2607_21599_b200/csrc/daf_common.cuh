@@ -58,17 +58,17 @@ int launch_fuse(const ResolvedParams& rp, const int32_t* idx, const void* o_imp,
                 int32_t* row_pos_out, cudaStream_t stream);
 int launch_deviation_scores(const ResolvedParams& rp, const void* k_fresh, const void* v_fresh, const void* k_cached,
                             const void* v_cached, float* scores, cudaStream_t stream);
-struct AttnPlan { int Gp, Tt, n_tb, head_blocks, n_splits, tiles_per_split; };
+struct AttnPlan { int Gp, Tt, n_tb, head_blocks, n_splits, steps_per_split; };
 AttnPlan plan_attention(int n_q, int n_kv, int Hq, int G, int causal_off, bool pack_group, bool allow_split);
 size_t attn_partial_bytes(int n_q, int Hq, int n_splits);
 int launch_attention(const void* q, const void* k, const void* v, int n_q, int n_kv, int Hq, int Hkv, int causal_off,
                      float scale, bool pack_group, bool allow_split, void* out, long long out_row_stride_bytes,
                      const int32_t* dst_rows, float* lse, DeviceStatus* status, void* scratch, size_t scratch_bytes,
-                     cudaStream_t stream, const int32_t* q_pos = nullptr);
+                     cudaStream_t stream, const int32_t* q_pos = nullptr, const AttnPlan* plan = nullptr);   // plan: null = planned here
 // Steps 2 and 3 of a layer from one list of work items (one attention launch and one merge launch).
 struct JointPlan {
     int Gp_i, Tt_i, n_tb_i, head_blocks_i, items_i;                       // important-token stage
-    int Gp_q, Tt_q, n_tb_q, head_blocks_q, n_splits_q, tiles_per_split_q, items_q;   // question stage
+    int Gp_q, Tt_q, n_tb_q, head_blocks_q, n_splits_q, steps_per_split_q, items_q;   // question stage
     size_t part_bytes_q;        // partial results of the question ranges
 };
 JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G);

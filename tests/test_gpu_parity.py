@@ -361,6 +361,23 @@ def test_question_attention_matches_oracle(L_d, L_q, Hq, Hkv, qscale):
     np.testing.assert_allclose(lse.cpu().numpy().T, ref_lse, atol=2e-3, rtol=0)
 
 
+@pytest.mark.parametrize("L_d,L_q,Hq,Hkv", [(130, 5, 4, 4), (450, 16, 7, 1), (700, 20, 14, 2), (900, 9, 7, 1),
+                                            (1500, 16, 8, 2), (9000, 3, 4, 1)])
+def test_question_attention_over_few_and_many_ranges(L_d, L_q, Hq, Hkv):
+    """Every form of the merge (8, 12, 15, 24 and 29 ranges, and none) and ranges that are not whole 128 keys."""
+    N = L_d + L_q
+    q, k, v = _normal((L_q, Hq, 128), 44), _normal((N, Hkv, 128), 45), _normal((N, Hkv, 128), 46)
+    p = api.make_params(L_d, L_q, 0.1, Hq, Hkv)
+    ws = api.alloc_workspace(p)
+    out = torch.full((L_q + 1, Hq, 128), 5.0, dtype=torch.bfloat16, device="cuda")
+    lse = torch.zeros(Hq, L_q, dtype=torch.float32, device="cuda")
+    _ok(api.daf_qd_attn(p, q.cuda(), k.cuda(), v.cuda(), out, Hq * 256, None, lse, ws), ws, "daf_qd_attn")
+    ref, ref_lse = oracle.qd_attn(_f(q), _f(k), _f(v), L_d, 1.0 / math.sqrt(128), return_lse=True)
+    _assert_close(out[:L_q], ref, f"question attention L_d={L_d} L_q={L_q}")
+    assert torch.all(out[L_q] == 5.0)
+    np.testing.assert_allclose(lse.cpu().numpy().T, ref_lse, atol=2e-3, rtol=0)
+
+
 @pytest.mark.parametrize("n,Hq,Hkv", [(1056, 28, 4), (513, 8, 8)])
 def test_full_causal_attention_matches_oracle(n, Hq, Hkv):
     q, k, v = _normal((n, Hq, 128), 51), _normal((n, Hkv, 128), 52), _normal((n, Hkv, 128), 53)
