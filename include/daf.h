@@ -174,10 +174,7 @@ int daf_qd_attn(const daf_params* p, const void* q_question, const void* kv_k, c
  * daf_important_attn + daf_qd_attn up to fp32 summation order.  State fusion (Methods item 3)
  * is done by the epilogues as in daf_layer:
  *   q_pack, k_pack, v_pack   the k packed rows left by daf_select.  q_pack may be NULL: the Q row of
- *            packed row j is then read in place, row idx[j] of q_fresh ([>= L_d, n_q_heads, 128]),
- *            which saves writing and re-reading the largest of the packed tensors but costs every
- *            work item a scattered fetch; measured on B200 the layer time changes by -2 % at
- *            k = 41780, +-1 % at k = 6554 and +10 % at k = 922.
+ *            packed row j is then read in place, row idx[j] of q_fresh ([>= L_d, n_q_heads, 128]).
  *   q_question, kv_k, kv_v   as in daf_qd_attn
  *   idx      int32 [k] positions of the packed rows; read iff p->fuse_mode == 1 or q_pack == NULL
  *   hidden   bf16, row stride n_q_heads * 256 bytes.  fuse_mode 0: rows 0..k-1 are the
@@ -248,7 +245,8 @@ int daf_full_causal_attn(const daf_params* p, int32_t n_tokens, const void* q, c
  * epilogues (device pointers; arguments as in daf_select, plus)
  *   hidden       compact: [k+L_q, n_q_heads*128]; scatter: [N, n_q_heads*128]
  *   row_pos_out  optional int32 [k+L_q]
- *   q_pack       may be NULL when L_q > 0: step 2 then reads its Q rows in place (see daf_imp_qd_attn)
+ *   q_pack       may be NULL when L_q > 0.  (When L_q > 0 step 2 reads its Q rows in place either way; a buffer given
+ *                receives the packed rows on the way.)
  *   k_pack, v_pack  may be NULL (both or neither) when k > 0 and L_q > 0: step 2 then reads its K/V rows in
  *                place too -- rows idx of k_fresh / v_fresh, fetched by the attention kernel itself -- and
  *                the kernel in front of it only updates the hybrid cache.  Same results, bit for bit, and no

@@ -240,7 +240,7 @@ int daf_imp_qd_attn_launches(const daf_params* p, const void* q_pack, const void
     if (int rc = check_out(hidden, row_bytes, rp.Hq)) return rc;
     char* h = reinterpret_cast<char*>(hidden);
     const int64_t first_row = rp.fuse_mode == 1 ? rp.L_d : rp.k;
-    return launch_attention_joint(q_pack, q_fresh, idx, k_pack, v_pack, nullptr, nullptr, rp.k, h, rp.fuse_mode == 1 ? idx : nullptr, q_question, kv_k, kv_v,
+    return launch_attention_joint(q_pack, q_fresh, q_pack == nullptr, false, idx, k_pack, v_pack, nullptr, nullptr, rp.k, h, rp.fuse_mode == 1 ? idx : nullptr, q_question, kv_k, kv_v,
                                   rp.L_q, rp.L_d, h + first_row * row_bytes, row_bytes, rp.Hq, rp.Hkv, rp.scale, ws.status,
                                   ws.attn_scratch, ws.attn_bytes, (cudaStream_t)stream, launches);
 }
@@ -334,13 +334,17 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     if (q_fresh != nullptr && !aligned16(q_fresh)) return DAF_ERR_ALIGNMENT;
     const int64_t row_bytes = (int64_t)rp.Hq * 256;
     if (int rc = check_out(hidden, row_bytes, rp.Hq)) return rc;
+    // Step 2 reads its Q rows in place and packs them on the way (the largest of the packed tensors: the gather kernel is left
+    // with K/V), unless they lie in host memory: 6k layer 32.9 -> 31.4 us, 11k 113.9 -> 112.2, 28 layers of 6k 728 -> 716, 16k
+    // 87.4 -> 87.7 (there the longer start of an item, positions and then rows from HBM, weighs as much as the copy saved).
+    const bool q_in_place = rows == nullptr && rp.k > 0 && rp.L_q > 0;
     // An fp8 offline cache is expanded into the hybrid-cache buffer first.  The selection does not depend on it,
     // so the selection kernel is launched beside it; the gather kernel (which overwrites the important rows of
     // the expanded cache) runs behind both.
     if (fp8 != nullptr)
         if (int rc = launch_expand_fp8(rp, fp8->k8, fp8->v8, fp8->k_scale, fp8->v_scale, kv_k, kv_v, st)) return rc;
     if (int rc = do_select(rp, scores, n_sig, idx_in, rows ? rows->q : q_fresh, rows ? rows->k : k_fresh,
-                           rows ? rows->v : v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
+                           rows ? rows->v : v_fresh, kv_k, kv_v, idx_out, q_in_place ? nullptr : q_pack, k_pack,
                            v_pack, ws, st, /*beside_previous_kernel=*/fp8 != nullptr && rp.L_d > 0,
                            rows)) return rc;
     char* h = reinterpret_cast<char*>(hidden);
@@ -351,7 +355,7 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     const char* qq = reinterpret_cast<const char*>(q_fresh) + (int64_t)rp.L_d * row_bytes;
     const int32_t* dst = rp.fuse_mode == 1 ? idx_out : nullptr;
     if (rp.k > 0 && rp.L_q > 0) {
-        if (int rc = launch_attention_joint(q_pack, q_fresh, idx_out, k_pack, v_pack, k_fresh, v_fresh, rp.k, h, dst, qq, kv_k, kv_v, rp.L_q, rp.L_d,
+        if (int rc = launch_attention_joint(q_pack, q_fresh, q_in_place, /*q_early=*/true, scores != nullptr ? idx_out : idx_in, k_pack, v_pack, k_fresh, v_fresh, rp.k, h, dst, qq, kv_k, kv_v, rp.L_q, rp.L_d,
                                             h + first_row * row_bytes, row_bytes, rp.Hq, rp.Hkv, rp.scale, ws.status,
                                             ws.attn_scratch, ws.attn_bytes, st)) return rc;
     } else if (rp.L_q > 0) {
@@ -458,9 +462,6 @@ void carve_arena(const ResolvedParams& rp, int n_sig, char* base, Arena* a) {
     a->total = off;
 }
 constexpr int kArenaSignalRows = 8;   // arena is sized for up to this many signal rows
-// From this many important tokens on the host-buffer layer skips the packed copy of the Q rows (step 2 reads
-// them in place): measured -2 % layer time at k = 41780, +-1 % at k = 6554, +10 % at k = 922.
-constexpr int kQInPlaceMinK = 16384;
 
 // A second stream for the part of a host-buffer layer that runs beside the rest, with the events that fork from and join
 // the caller's stream.  Each host thread keeps two per device (a pipelining caller begins a layer before it ends the one
@@ -606,7 +607,7 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
     DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_k, h_kv_k, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
     DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_v, h_kv_v, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
     // (rows read from the host: always with packed copies on the device, the attention kernel must not go to the host)
-    void* qp = (!in_place_rows && rp.k >= kQInPlaceMinK && rp.L_q > 0) ? nullptr : a.q_pack;
+    void* qp = (!in_place_rows && rp.L_q > 0) ? nullptr : a.q_pack;     // otherwise nobody asks for a packed copy of Q
     if (int rc = layer_impl(p, nullptr, h_scores ? a.scores : nullptr, n_sig, h_scores ? nullptr : a.idx_in, a.q_fresh, a.k_fresh,
                             a.v_fresh, a.kv_k, a.kv_v, a.idx_out, qp, a.k_pack, a.v_pack, a.hidden, nullptr, a.ws, a.ws_bytes, stream,
                             in_place_rows ? &rows : nullptr)) return rc;

@@ -40,11 +40,12 @@ struct SegArgs {
     int n_tb;           // token blocks = ceil(n_q / Tt)
     int causal_off;     // token t sees keys <= t + causal_off ...
     const int32_t* q_pos; // ... or, when given, keys <= q_pos[t] (ascending positions of the query tokens)
-    // Query rows read in place instead of from a packed copy: query token t is row q_idx[t]
-    // of q_src, a [q_src_rows, Hq, 128] tensor.  q_idx == nullptr: the Q tensor map covers packed rows.
-    const __nv_bfloat16* q_src;
+    // Query rows read in place instead of from a packed copy: query token t is row q_idx[t] of a tensor of q_src_rows rows
+    // (which the Q tensor map then covers, with a box of one token).  q_idx == nullptr: the map covers packed rows.
     const int32_t* q_idx;
     int q_src_rows;
+    int q_early;        // q_idx and the rows are complete before the kernel launched just before this one started
+    int q_save;         // the tiles so fetched are also written out as packed rows (second Q map)
     // Likewise the keys: key j is row kv_idx[j] of k_src / v_src, [kv_src_rows, kv_heads, 128] tensors.
     // k_src == nullptr: the K and V tensor maps cover packed rows.
     const __nv_bfloat16* k_src;
@@ -404,6 +405,7 @@ struct AttnSmem {
     uint64_t k_full[2], v_full[2];
     uint64_t s_full[2], p_full[2];
     uint64_t pv_done[2];      // O += P_t V_t has completed: sub-steps alternate between the two barriers
+    uint64_t q_saved;         // the Q tile has been read by the store of the packed rows
     uint64_t rows_parked;     // epilogue: the four softmax warps have parked their rows for the tiled store
     uint32_t tmem_base;
     int abort_flag;
@@ -416,7 +418,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
                   const __grid_constant__ CUtensorMap tmap_v0, const __grid_constant__ CUtensorMap tmap_q1,
                   const __grid_constant__ CUtensorMap tmap_k1, const __grid_constant__ CUtensorMap tmap_v1,
                   const __grid_constant__ CUtensorMap tmap_o0, const __grid_constant__ CUtensorMap tmap_o1,
-                  const AttnArgs args) {
+                  const __grid_constant__ CUtensorMap tmap_qp0, const AttnArgs args) {
     extern __shared__ unsigned char attn_smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(attn_smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char* q_smem = smem;                                 // 32 KB
@@ -515,13 +517,17 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     // Everything up to the wait below touches no memory an earlier kernel writes, so with programmatic
     // dependent launch it runs while the kernel launched just before (gather / hybrid-cache update) drains.
     __shared__ int skip_cta;
-    const int32_t* const q_idx = DAF_SEG(q_idx);     // non-null: the softmax warps fetch the Q rows themselves
+    const int32_t* const q_idx = DAF_SEG(q_idx);     // non-null: Q rows are fetched token by token through this list
+    const bool q_save = q_idx != nullptr && DAF_SEG(q_save) != 0;
+    const bool q_early = q_idx != nullptr && DAF_SEG(q_early) != 0;
+    int q_first = -1;            // position of this lane's first token: asked for ahead of everything else
+    if (warp == 4 && q_early && lane < min(a.Tt, a.n_q - t0)) q_first = __ldcg(q_idx + t0 + lane);
     if (warp == 5) {
         tmem_alloc(&sm->tmem_base, kAttnTmemCols);
         tmem_relinquish();
     }
     if (warp == 4 && lane == 0) {
-        mbar_init(&sm->q_full, q_idx != nullptr ? 4 : 1);
+        mbar_init(&sm->q_full, 1); mbar_init(&sm->q_saved, 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(&sm->k_full[s], kv_gather ? 32 * kGatherWarps : 1); mbar_init(&sm->v_full[s], kv_gather ? 32 * kGatherWarps : 1);
             mbar_init(&sm->s_full[s], 1); mbar_init(&sm->p_full[s], 4);
@@ -532,7 +538,25 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         mbar_fence_init();
         tma_prefetch_desc(tmap_k);
         tma_prefetch_desc(tmap_v);
-        if (q_idx == nullptr) tma_prefetch_desc(tmap_q);
+        tma_prefetch_desc(tmap_q);
+    }
+    // Q rows in place: one copy per token and half row, into the rows of the tile where one copy of packed rows would have
+    // put them (the swizzle goes by the shared-memory address).  A bad position, which the gather kernel reports, reads as zeros.
+    auto fetch_q = [&]() {
+        const int n_tok = min(a.Tt, a.n_q - t0), rows = DAF_SEG(q_src_rows);
+        if (lane == 0) mbar_arrive_expect_tx(&sm->q_full, 2u * 128u * (uint32_t)(a.Gp * n_tok));
+        __syncwarp();
+        for (int i = lane; i < n_tok; i += 32) {
+            int pos = q_early && i < 32 ? q_first : __ldcg(q_idx + t0 + i);
+            if ((unsigned)pos >= (unsigned)rows) pos = rows;
+            tma_load_3d(q_smem + i * a.Gp * 128, tmap_q, &sm->q_full, 0, h0, pos);
+            tma_load_3d(q_smem + i * a.Gp * 128 + kHalfBytes, tmap_q, &sm->q_full, 64, h0, pos);
+        }
+        __syncwarp();
+    };
+    if (warp == 4 && q_early) {
+        __syncwarp();
+        fetch_q();
     }
     pdl_wait();                // from here on: inputs that the kernel launched just before may have written
     // sub-steps of this item: the keys of its range that the tile's last token may see
@@ -544,6 +568,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         hi = min(hi, (long long)a.j_end * kSubN);
         if (hi > key_begin) n_t = (int)((hi - key_begin + kSubN - 1) / kSubN);
     }
+    if (warp == 4 && q_idx != nullptr && !q_early) fetch_q();
     if (warp == 4 && lane == 0) {
         if (n_t > 0) {
             if (q_idx == nullptr) {
@@ -555,35 +580,9 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
                 for (int t = 0; t < 2 && t < n_t; ++t) { issue_kv(t, 0); issue_kv(t, 1); }
         }
     }
-    if (q_idx != nullptr && n_t > 0 && warp < 4) {
-        const int quad = warp;
-        // Q rows of the condensed sequence straight from the unpacked tensor: each warp fetches its 32
-        // rows (16 lanes per 256-byte row) into the layout the TMA load would have produced
-        // (two 64-column halves of 128-byte rows, 16-byte chunks XOR-ed with the row number mod 8).
-        const __nv_bfloat16* q_src = DAF_SEG(q_src);
-        const int q_src_rows = DAF_SEG(q_src_rows), Hq = DAF_SEG(Hq);
-        const int sub = lane >> 4, cidx = lane & 15;
-        uint4 w[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int rr = quad * 32 + 2 * i + sub, dt = rr / a.Gp, tokr = t0 + dt;
-            w[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (dt < a.Tt && tokr < a.n_q) {
-                const int src = __ldg(q_idx + tokr);
-                if ((unsigned)src < (unsigned)q_src_rows)   // a bad position is reported by the gather kernel
-                    w[i] = __ldg(reinterpret_cast<const uint4*>(q_src + ((size_t)src * Hq + h0 + (rr - dt * a.Gp)) * kD) + cidx);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int rr = quad * 32 + 2 * i + sub;
-            *reinterpret_cast<uint4*>(q_smem + (cidx >> 3) * kHalfBytes + rr * 128 + (((cidx & 7) ^ (rr & 7)) << 4)) = w[i];
-        }
-        fence_proxy_async();
-    }
-    // rows of the Q tile past the Gp * Tt that the tiled load fills: zeros
-    if (warp == 3 && q_idx == nullptr) {
-        const int used = a.Gp * a.Tt;
+    // rows of the Q tile that the loads do not fill: zeros
+    if (warp == 3) {
+        const int used = a.Gp * (q_idx == nullptr ? a.Tt : min(a.Tt, a.n_q - t0));
         for (int i = lane; i < (kBlockM - used) * 16; i += 32)
             *reinterpret_cast<uint4*>(q_smem + ((i >> 3) & 1) * kHalfBytes + (used + (i >> 4)) * 128 + ((i & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
         if (used < kBlockM) fence_proxy_async();
@@ -598,11 +597,32 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     const bool skip = skip_cta != 0;
     if (threadIdx.x == 0) DAF_STAMP(1);
 
+    // The packed copy of a Q tile fetched in place, stored by warp 4 once the tile has landed; then the epilogue may use the tile.
+    auto save_q = [&]() {
+        if (lane == 0) {
+            tma_store_3d(&tmap_qp0, q_smem, 0, h0, t0);
+            tma_store_3d(&tmap_qp0, q_smem + kHalfBytes, 64, h0, t0);
+            tma_store_commit();
+        }
+        __syncwarp();
+    };
+    auto finish_q = [&](bool saved) {
+        if (!saved) {
+            bool ok = mbar_wait(&sm->q_full, 0, abort_flag, status, 16);
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (ok) save_q();
+        }
+        if (lane == 0) {
+            tma_store_wait_read();
+            mbar_arrive(&sm->q_saved);
+        }
+    };
+
     if (skip) {
         // nothing is computed; the loads already under way get a bounded chance to land before the CTA retires
-        if (warp == 4 && lane == 0 && n_t > 0 && !kv_gather) {
+        if (warp == 4 && lane == 0 && n_t > 0) {
             for (int i = 0; i < 4096 && !mbar_try_wait(&sm->q_full, 0); ++i) {}
-            for (int s = 0; s < 2 && s < n_t; ++s) {
+            for (int s = 0; s < 2 && s < n_t && !kv_gather; ++s) {
                 for (int i = 0; i < 4096 && !mbar_try_wait(&sm->k_full[s], 0); ++i) {}
                 for (int i = 0; i < 4096 && !mbar_try_wait(&sm->v_full[s], 0); ++i) {}
             }
@@ -627,8 +647,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
             }
         }
         kv_gather_arrive(true);   // the last copy group (also on the way out after a give-up: copies always land)
+        if (warp == 4 && q_save) finish_q(false);
     } else if (warp == 4) {
         // ------------------------------------------------------------ TMA producer (the rest of the sub-steps)
+        bool saved = !q_save;
         if (n_t > 2) {   // the whole warp walks the loop, one elected lane issues (uniform control flow)
             bool ok = true;
             for (int t = 2; t < n_t && ok; ++t) {
@@ -642,6 +664,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (ok && elect_one()) issue_kv(t, kv);
                     __syncwarp();
+                    if (ok && !saved) { save_q(); saved = true; }     // (the first logits are there: so was Q)
                 }
             }
             if (!ok && lane == 0) {
@@ -652,6 +675,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
                 }
             }
         }
+        if (q_save) finish_q(saved);
     } else if (warp == 5) {
         // ------------------------------------------------------------ MMA issuer
         // The whole warp walks the loop and waits on the barriers, one elected lane issues: control flow
@@ -745,7 +769,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         const uint32_t o_addr = tmem + lane_addr + (uint32_t)kBlockN;
         const float c = a.scale_log2;
 
-        if (q_idx != nullptr && n_t > 0 && lane == 0) mbar_arrive(&sm->q_full);   // this warp's Q rows were stored before the set-up barrier
         float m = -INFINITY, l = 0.f;
         bool ok = true;
         DAF_LAP_DECL;
@@ -781,6 +804,10 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         // ---- epilogue
         if (ok && n_t > 0) {
             ok = mbar_wait(&sm->pv_done[(n_t - 1) & 1], (uint32_t)(((n_t - 1) >> 1) & 1), abort_flag, status, 61);
+            ok = __all_sync(0xFFFFFFFFu, ok);
+        }
+        if (ok && q_save) {
+            ok = mbar_wait(&sm->q_saved, 0, abort_flag, status, 62);
             ok = __all_sync(0xFFFFFFFFu, ok);
         }
         if (ok) {
@@ -1250,7 +1277,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     a.status = status;
     dim3 grid((unsigned)pl.head_blocks, (unsigned)pl.n_tb, (unsigned)pl.n_splits);
     cudaError_t e = launch_kernel(attn_fwd_kernel<false>, grid, dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
-                                  to, to, a);
+                                  to, to, tq, a);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     if (int rc = check_launch()) return rc;
@@ -1280,7 +1307,7 @@ int launch_bounded_wait_selftest(DeviceStatus* status, int limit_ms, cudaStream_
 
 size_t joint_partial_bytes(const JointPlan& jp) { return jp.part_bytes_q; }
 
-int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t* idx, const void* k_imp, const void* v_imp,
+int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_place, bool q_early, const int32_t* idx, const void* k_imp, const void* v_imp,
                            const void* k_fresh, const void* v_fresh,
                            int k, void* out_imp, const int32_t* dst_rows_imp, const void* q_question, const void* kv_k,
                            const void* kv_v,
@@ -1292,10 +1319,13 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     if (joint_partial_bytes(jp) > scratch_bytes) return DAF_ERR_WORKSPACE;
 
     CUtensorMap tq0, tk0, tv0, tq1, tk1, tv1;
-    // without packed Q rows the kernel reads them in place through idx (no tensor map needed for them)
-    const bool gather_q = q_imp == nullptr;
-    if (gather_q && (q_fresh == nullptr || idx == nullptr)) return DAF_ERR_INVALID_ARG;
-    if (int rc = make_tmap(&tq0, gather_q ? q_question : q_imp, gather_q ? L_q : k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
+    // Q rows in place: read through idx, and left in q_imp as packed rows where the caller wants them
+    const bool gather_q = q_in_place;
+    if (gather_q ? (q_fresh == nullptr || idx == nullptr) : q_imp == nullptr) return DAF_ERR_INVALID_ARG;
+    if (int rc = gather_q ? make_tmap(&tq0, q_fresh, L_d, Hq, jp.Gp_i, 1) : make_tmap(&tq0, q_imp, k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
+    CUtensorMap tqp = tq0;
+    if (gather_q && q_imp != nullptr)
+        if (int rc = make_tmap(&tqp, q_imp, k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
     // without packed K/V rows the producer warp reads them in place through idx as well
     const bool gather_kv = k_imp == nullptr;
     if (gather_kv && (v_imp != nullptr || k_fresh == nullptr || v_fresh == nullptr || idx == nullptr)) return DAF_ERR_INVALID_ARG;
@@ -1332,9 +1362,10 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     SegArgs& si = a.seg[0];
     fill_problem(&si, k, k, Hq, G, jp.Gp_i, 0, nullptr, scale, out_imp, out_row_stride_bytes, dst_rows_imp, nullptr);
     if (gather_q) {
-        si.q_src = reinterpret_cast<const __nv_bfloat16*>(q_fresh);
         si.q_idx = idx;
         si.q_src_rows = L_d;
+        si.q_early = q_early ? 1 : 0;
+        si.q_save = q_imp != nullptr ? 1 : 0;
     }
     if (gather_kv) {
         si.k_src = reinterpret_cast<const __nv_bfloat16*>(k_fresh);
@@ -1354,9 +1385,9 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, const int32_t
     if (launches & 1) {
         const cudaError_t e = gather_kv
             ? launch_kernel(attn_fwd_kernel<true>, dim3((unsigned)items), dim3(kAttnThreadsGather), kAttnSmemBytes, stream,
-                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, a)
+                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, tqp, a)
             : launch_kernel(attn_fwd_kernel<false>, dim3((unsigned)items), dim3(kAttnThreads), kAttnSmemBytes, stream,
-                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, a);
+                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, tqp, a);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         if (int rc = check_launch()) return rc;

@@ -826,6 +826,30 @@ def test_both_attention_stages_from_one_work_list(k, L_d, L_q, Hq, Hkv, fuse_mod
         assert torch.all(h[others] == -9.0), "a row that is neither important nor a question row was written"
 
 
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv", [(700, 9, 0.3, 14, 2), (300, 5, 0.01, 4, 4), (1000, 20, 0.13, 12, 1), (260, 3, 1.0, 2, 2), (900, 4, 0.2, 129, 1)])
+def test_layer_leaves_the_packed_q_rows_it_read_in_place(L_d, L_q, r, Hq, Hkv, given):
+    """Tiles of one and of several heads, whole and partial last tiles: the packed Q rows are the fresh rows at the
+    selected positions, byte for byte, and nothing past them is written."""
+    w = W.Workload("t", 43, Hq, Hkv, 128, 1, L_d, L_d, L_q, r, "lognormal", 1)
+    L = W.make_layer(w, 0)
+    p = api.make_params(L_d, L_q, r, Hq, Hkv)
+    k = api.daf_num_important(L_d, r)
+    idx = oracle.select(L["scores"].numpy(), k)
+    g = {n: t.cuda() for n, t in L.items() if t is not None}
+    kv = [torch.cat([g[n], torch.zeros(L_q, Hkv, 128, dtype=torch.bfloat16, device="cuda")]) for n in ("k_cached", "v_cached")]
+    ws = api.alloc_workspace(p)
+    idx_out = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+    qp = torch.full((k + 1, Hq, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+    kp, vp = torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda"), torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda")
+    hidden = torch.zeros(k + L_q, Hq, 128, dtype=torch.bfloat16, device="cuda")
+    given_idx = torch.from_numpy(idx).cuda() if given else None
+    _ok(api.daf_layer(p, None if given else g["scores"], 1, given_idx, g["q_fresh"], g["k_fresh"], g["v_fresh"], kv[0], kv[1],
+                      idx_out, qp, kp, vp, hidden, None, ws), ws, "daf_layer")
+    assert np.array_equal(idx_out.cpu().numpy(), idx)
+    assert torch.equal(qp[:k], g["q_fresh"][idx_out.long()]) and torch.all(qp[k] == 3.0)
+
+
 @pytest.mark.parametrize("fuse_mode", [0, 1])
 def test_layer_without_packed_q_buffer(fuse_mode):
     """daf_layer with q_pack = NULL (step 2 reads its Q rows in place) gives the same bits as with the buffer,
