@@ -94,7 +94,7 @@ static int carve_workspace(const ResolvedParams& rp, void* workspace, size_t byt
 static int do_select(const ResolvedParams& rp, const float* scores, int32_t n_sig, const int32_t* idx_in,
                      const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                      int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack, const Workspace& ws, cudaStream_t st,
-                     bool beside_previous_kernel = false, const RowSource* far = nullptr) {
+                     const Fp8Cache* fp8 = nullptr, const RowSource* far = nullptr) {
     if (scores != nullptr && n_sig < 1) return DAF_ERR_INVALID_ARG;
     if (rp.k > 0) {
         if (scores == nullptr && idx_in == nullptr) return DAF_ERR_INVALID_ARG;
@@ -109,7 +109,7 @@ static int do_select(const ResolvedParams& rp, const float* scores, int32_t n_si
     for (const void* ptr : ptrs)
         if (ptr != nullptr && !aligned16(ptr)) return DAF_ERR_ALIGNMENT;
     return launch_select(rp, scores, n_sig, idx_in, q_fresh, k_fresh, v_fresh, kv_k, kv_v, idx_out, q_pack, k_pack,
-                         v_pack, ws.status, ws.select_scratch, st, beside_previous_kernel,
+                         v_pack, ws.status, ws.select_scratch, st, fp8,
                          /*select_only=*/false, far);
 }
 
@@ -306,9 +306,6 @@ int daf_full_causal_attn(const daf_params* p, int32_t n_tokens, const void* q, c
 }  // extern "C"
 
 namespace {
-// Offline cache of one layer kept in fp8 (daf_layer_fp8): expanded into kv_k / kv_v ahead of everything else.
-struct Fp8Cache { const void* k8; const void* v8; const float* k_scale; const float* v_scale; };
-
 int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, int32_t n_sig, const int32_t* idx_in,
                const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack,
@@ -338,14 +335,9 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     // with K/V), unless they lie in host memory: 6k layer 32.9 -> 31.4 us, 11k 113.9 -> 112.2, 28 layers of 6k 728 -> 716, 16k
     // 87.4 -> 87.7 (there the longer start of an item, positions and then rows from HBM, weighs as much as the copy saved).
     const bool q_in_place = rows == nullptr && rp.k > 0 && rp.L_q > 0;
-    // An fp8 offline cache is expanded into the hybrid-cache buffer first.  The selection does not depend on it,
-    // so the selection kernel is launched beside it; the gather kernel (which overwrites the important rows of
-    // the expanded cache) runs behind both.
-    if (fp8 != nullptr)
-        if (int rc = launch_expand_fp8(rp, fp8->k8, fp8->v8, fp8->k_scale, fp8->v_scale, kv_k, kv_v, st)) return rc;
     if (int rc = do_select(rp, scores, n_sig, idx_in, rows ? rows->q : q_fresh, rows ? rows->k : k_fresh,
                            rows ? rows->v : v_fresh, kv_k, kv_v, idx_out, q_in_place ? nullptr : q_pack, k_pack,
-                           v_pack, ws, st, /*beside_previous_kernel=*/fp8 != nullptr && rp.L_d > 0,
+                           v_pack, ws, st, rp.L_d > 0 ? fp8 : nullptr,
                            rows)) return rc;
     char* h = reinterpret_cast<char*>(hidden);
     // State fusion is done by the attention epilogues: each stage writes its final rows.  When both
@@ -407,7 +399,7 @@ int daf_select_topk(const daf_params* p, const float* scores, int32_t n_sig, int
     ResolvedParams sel = rp;
     sel.L_q = 0;
     return launch_select(sel, scores, n_sig, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, idx_out, nullptr, nullptr,
-                         nullptr, ws.status, ws.select_scratch, (cudaStream_t)stream, false, /*select_only=*/true);
+                         nullptr, ws.status, ws.select_scratch, (cudaStream_t)stream, nullptr, /*select_only=*/true);
 }
 
 int daf_check_indices(const daf_params* p, int32_t k, const int32_t* idx, void* workspace, size_t workspace_bytes_,
@@ -429,7 +421,7 @@ int daf_expand_fp8_cache(const daf_params* p, const void* k_cached_fp8, const vo
     if (rp.L_d == 0) return DAF_OK;
     if (!k_cached_fp8 || !v_cached_fp8 || !kv_k || !kv_v) return DAF_ERR_INVALID_ARG;
     if (!aligned16(k_cached_fp8) || !aligned16(v_cached_fp8) || !aligned16(kv_k) || !aligned16(kv_v)) return DAF_ERR_ALIGNMENT;
-    return launch_expand_fp8(rp, k_cached_fp8, v_cached_fp8, k_scale, v_scale, kv_k, kv_v, (cudaStream_t)stream);
+    return launch_expand_fp8(rp, Fp8Cache{k_cached_fp8, v_cached_fp8, k_scale, v_scale}, kv_k, kv_v, (cudaStream_t)stream, false);
 }
 
 // ---- host-buffer form
@@ -514,7 +506,7 @@ int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows
     if (int rc = carve_workspace(rp, a.ws, a.ws_bytes, &ws)) return rc;
     rows.cache_later = true;
     if (int rc = do_select(rp, scores, n_sig, scores ? nullptr : a.idx_in, rows.q, rows.k, rows.v, a.kv_k, a.kv_v, a.idx_out, a.q_pack,
-                           a.k_pack, a.v_pack, ws, st, false, &rows)) return rc;
+                           a.k_pack, a.v_pack, ws, st, nullptr, &rows)) return rc;
     DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
     DAF_CUDA_TRY(cudaStreamWaitEvent(lane.stream, lane.fork, 0));
     auto important = [&]() -> int {

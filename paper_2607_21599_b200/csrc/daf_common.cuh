@@ -37,6 +37,8 @@ int resolve_params(const daf_params* p, ResolvedParams* out);  // validates; DAF
 
 // kernel launchers (daf_select.cu, daf_attn.cu), called by the C ABI in daf_api.cu
 size_t select_scratch_bytes(int L_d);
+// Offline cache of one layer kept in fp8: expanded into kv_k / kv_v ahead of the gather.
+struct Fp8Cache { const void* k8; const void* v8; const float* k_scale; const float* v_scale; };
 // Where the gather / cache-update kernel reads the fresh rows when that is not the tensors the attention reads the question
 // rows from: device-accessible pointers to [N, heads, 128] tensors (mapped pinned host memory).  host_k / host_v: the
 // caller's cache in host memory, likewise mapped, when the kernel is to write the rows that change straight back to it.
@@ -45,12 +47,11 @@ struct RowSource { const void* q; const void* k; const void* v; void* host_k; vo
 int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, const int32_t* idx_in,
                   const void* q_fresh, const void* k_fresh, const void* v_fresh, void* kv_k, void* kv_v,
                   int32_t* idx_out, void* q_pack, void* k_pack, void* v_pack,
-                  DeviceStatus* status, void* scratch, cudaStream_t stream, bool beside_previous_kernel = false, bool select_only = false, const RowSource* far = nullptr);
+                  DeviceStatus* status, void* scratch, cudaStream_t stream, const Fp8Cache* fp8 = nullptr, bool select_only = false, const RowSource* far = nullptr);
 int launch_update_cache(const ResolvedParams& rp, const int32_t* idx, const void* k_pack, const void* v_pack, void* kv_k,
                         void* kv_v, cudaStream_t stream);
 int launch_check_indices(const int32_t* idx, int k, int L_d, DeviceStatus* status, cudaStream_t stream);
-int launch_expand_fp8(const ResolvedParams& rp, const void* k8, const void* v8, const float* k_scale, const float* v_scale,
-                      void* kv_k, void* kv_v, cudaStream_t stream);
+int launch_expand_fp8(const ResolvedParams& rp, const Fp8Cache& c, void* kv_k, void* kv_v, cudaStream_t stream, bool beside_selection);
 constexpr int kMaxSignalLayersHost = 8;
 int launch_deviation_sum(const ResolvedParams& rp, int n_sig, const void* const* k_fresh, const void* const* v_fresh,
                          const void* const* k_cached, const void* const* v_cached, float* sums, cudaStream_t stream);
