@@ -28,7 +28,7 @@ DAF_KT_READER(daf_dbg_kt_select)
 // the threshold are broken by position (lower first), so the result is unique.
 
 constexpr int kSelCluster = 8;
-constexpr int kSelThreads = 512;
+constexpr int kSelThreads = 1024;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelSmemKeysPerCta = 40960;   // slice kept in shared memory up to this size, in global scratch beyond
 
@@ -67,8 +67,6 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     DAF_KT_BEGIN(0);
-    pdl_wait();
-    pdl_launch_dependents();   // the gather kernel may start launching; it waits for this grid before reading idx
     extern __shared__ __align__(16) unsigned char sel_smem[];
     SelShared* sh = reinterpret_cast<SelShared*>(sel_smem);
     uint32_t* skeys = reinterpret_cast<uint32_t*>(sel_smem + sizeof(SelShared));
@@ -81,17 +79,52 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     const bool in_smem = per_cta <= kSelSmemKeysPerCta;
     uint32_t* keys = in_smem ? skeys : (gkeys + lo_cta);
     auto at = [&](int i) { return in_smem ? padded(i) : i; };   // padded layout in shared memory only
-
-    // aggregate the signal rows in ascending row order (fp32 adds, no fusing) and build keys
-    for (int i = tid; i < n_loc; i += kSelThreads) {
-        const int g = lo_cta + i;
-        float acc = scores[g];
-        for (int l = 1; l < n_sig; ++l) acc = add_rn_keep_subnormals(acc, scores[(size_t)l * L_d + g]);
-        keys[at(i)] = score_key(acc);
-    }
     if (tid < 256) { sh->hist[0][tid] = 0u; sh->hist[1][tid] = 0u; }
     if (tid == 0) { sh->pick[0] = 0u; sh->pick[1] = (uint32_t)k; sh->pick[2] = 0u; }
     __syncthreads();
+    pdl_wait();
+    pdl_launch_dependents();   // the gather kernel may start launching; it waits for this grid before reading idx
+
+    // one more key in a bin; a warp whose keys all fall in one bin adds once, otherwise every thread adds for itself
+    auto count = [&](uint32_t* hist, bool in, uint32_t bin) {
+        const uint32_t active = __ballot_sync(0xFFFFFFFFu, in);
+        if (active == 0u) return;
+        const uint32_t lead_bin = __shfl_sync(0xFFFFFFFFu, bin, __ffs(active) - 1);
+        const uint32_t same = __ballot_sync(0xFFFFFFFFu, in && bin == lead_bin);
+        if (same == active) {
+            if (lane == __ffs(active) - 1) atomicAdd(&hist[lead_bin], (uint32_t)__popc(active));
+        } else if (in) {
+            atomicAdd(&hist[bin], 1u);
+        }
+    };
+    // aggregate the signal rows in ascending row order (fp32 adds, no fusing), build keys and count their top byte
+    // (four loads in flight per thread: one per trip would serialise on memory latency)
+    for (int base = 0; base < n_loc; base += 4 * kSelThreads) {
+        float acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = base + u * kSelThreads + tid;
+            acc[u] = i < n_loc ? scores[lo_cta + i] : 0.f;
+        }
+        for (int l = 1; l < n_sig; ++l) {
+            float nxt[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = base + u * kSelThreads + tid;
+                nxt[u] = i < n_loc ? scores[(size_t)l * L_d + lo_cta + i] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[u] = add_rn_keep_subnormals(acc[u], nxt[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = base + u * kSelThreads + tid;
+            if (base + u * kSelThreads >= n_loc) break;       // uniform across the CTA
+            const uint32_t key = score_key(acc[u]);
+            if (i < n_loc) keys[at(i)] = key;
+            count(sh->hist[0], i < n_loc, key >> 24);
+        }
+    }
 
     // Radix selection from the top byte down.  It stops as soon as every key left in the chosen bin is taken
     // (with distinct scores usually after three passes): the comparisons below then look only at the bits
@@ -100,24 +133,11 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     int pass = 0;
     for (int shift = 24; shift >= 0; shift -= 8, ++pass) {
         uint32_t* hist = sh->hist[pass & 1];
-        const int n_round = (n_loc + 31) / 32 * 32;
-        for (int i = tid; i < n_round; i += kSelThreads) {
-            bool in = false;
-            uint32_t bin = 0u;
-            if (i < n_loc) {
-                const uint32_t key = keys[at(i)];
-                in = (key & mask) == prefix;
-                bin = (key >> shift) & 0xFFu;
-            }
-            // a warp whose keys all fall in one bin adds once; otherwise every thread adds for itself
-            const uint32_t active = __ballot_sync(0xFFFFFFFFu, in);
-            if (active == 0u) continue;
-            const uint32_t lead_bin = __shfl_sync(0xFFFFFFFFu, bin, __ffs(active) - 1);
-            const uint32_t same = __ballot_sync(0xFFFFFFFFu, in && bin == lead_bin);
-            if (same == active) {
-                if (lane == __ffs(active) - 1) atomicAdd(&hist[lead_bin], (uint32_t)__popc(active));
-            } else if (in) {
-                atomicAdd(&hist[bin], 1u);
+        if (pass > 0) {
+            for (int base = 0; base < n_loc; base += kSelThreads) {
+                const int i = base + tid;
+                const uint32_t key = i < n_loc ? keys[at(i)] : 0u;
+                count(hist, i < n_loc && (key & mask) == prefix, (key >> shift) & 0xFFu);
             }
         }
         cluster.sync();   // every CTA's histogram of this pass is complete
@@ -646,8 +666,10 @@ deviation_sum_kernel(const SignalLayers layers, int L_d, int chunks_per_row, flo
 }
 
 // ----------------------------------------------------------------- host side
-// Measured on B200 (selection alone): one CTA 4.9 / 5.3 / 8.1 us at 6K / 8K / 16K tokens, the cluster of eight
-// 7.0 / 5.8 / 7.6 us: one CTA up to 8K tokens, the cluster beyond.
+// Measured (selection alone, back to back in a graph, lognormal scores): one CTA 5.6 / 6.4 us at 6K / 8K tokens, the cluster
+// of eight 6.7 / 7.1 there and 7.3 / 8.1 / 10.1 / 22.1 at 11K / 16K / 32K / 136K: one CTA up to 8K tokens, the cluster beyond.
+// (The cluster with 512 threads a CTA, one load in flight each and a pass of its own for the first histogram: 7.5 / 8.7 /
+// 12.1 / 32.0.  Digits of 12 bits, whose histograms are 16 times as much to exchange: 12.0 / 14.4 / 11.9 / 22.0.)
 static int g_sel1_max_keys = 8192;
 #ifdef DAF_TRACE
 extern "C" void daf_dbg_sel1_max_keys(int n) { g_sel1_max_keys = n < kSel1MaxKeys ? n : kSel1MaxKeys; }
