@@ -493,23 +493,40 @@ bool mapped_host_pointer(const void* h, const void** dev) {
     return true;
 }
 
-// A layer from pinned host buffers, compact rows, with both directions of the link to the host at work: the fresh rows
-// come first (the gather kernel reads them from the host and writes the changed cache rows back), then the important
-// tokens' attention and the copy out of its rows run on a second stream beside the copy in of the document rows, which
-// only the question rows wait for.  Bound by the link: k + L_q fresh rows and the document rows in (22 MB for the 6k layer,
-// 0.42 ms at 52 GB/s).  6k layer, cache copied back: one stream, whole cache copied back 865 us; this way 577.
+// A layer from pinned host buffers, compact rows, with both directions of the link to the host at work.  On the caller's
+// stream the gather kernel reads the fresh rows from the host and writes the changed cache rows back, then the rest of the
+// cache is copied in and the question rows follow; on a second stream the question's Q rows and the first part of the
+// cache are copied in beside the gather kernel, then the important tokens' attention runs and its rows are copied out.
+// Bound by the link: k + L_q fresh rows and the document rows in (22 MB for the 6k layer, 0.42 ms at 53 GB/s).  6k layer,
+// cache copied back: one stream, whole cache back 865 us; both directions, cache behind the gather 571; this way 531.
 int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows, const float* scores, int32_t n_sig,
-                        const void* h_kv_k, const void* h_kv_v, void* h_hidden, int32_t* h_idx_out, cudaStream_t st,
+                        const void* h_q_question, const void* h_kv_k, const void* h_kv_v, void* h_hidden, int32_t* h_idx_out, cudaStream_t st,
                         const SideLane& lane) {
     const size_t qrow = (size_t)rp.Hq * 256, kvrow = (size_t)rp.Hkv * 256;
     Workspace ws;
     if (int rc = carve_workspace(rp, a.ws, a.ws_bytes, &ws)) return rc;
     rows.cache_later = true;
-    if (int rc = do_select(rp, scores, n_sig, scores ? nullptr : a.idx_in, rows.q, rows.k, rows.v, a.kv_k, a.kv_v, a.idx_out, a.q_pack,
-                           a.k_pack, a.v_pack, ws, st, nullptr, &rows)) return rc;
+    // The gather kernel's reads leave some of the link idle (45 GB/s of 53), so part of the cache is copied beside it; the rest
+    // follows it, as much as keeps the link busy while the important rows are copied out.
+    const size_t cache = kvrow * rp.L_d, out_bytes = qrow * rp.k;
+    const size_t early = 2 * cache > out_bytes ? (2 * cache - out_bytes) / kvrow * kvrow : 0;   // bytes of K, then of V
+    auto copy_cache = [&](size_t from, size_t to, cudaStream_t s) -> int {
+        const size_t k0 = from < cache ? from : cache, k1 = to < cache ? to : cache;
+        const size_t v0 = from > cache ? from - cache : 0, v1 = to > cache ? to - cache : 0;
+        if (k1 > k0) DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_k + k0, reinterpret_cast<const char*>(h_kv_k) + k0, k1 - k0, cudaMemcpyHostToDevice, s));
+        if (v1 > v0) DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_v + v0, reinterpret_cast<const char*>(h_kv_v) + v0, v1 - v0, cudaMemcpyHostToDevice, s));
+        return DAF_OK;
+    };
     DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
     DAF_CUDA_TRY(cudaStreamWaitEvent(lane.stream, lane.fork, 0));
     auto important = [&]() -> int {
+        DAF_CUDA_TRY(cudaMemcpyAsync(a.q_fresh + qrow * rp.L_d, h_q_question, qrow * rp.L_q, cudaMemcpyHostToDevice, lane.stream));
+        if (int rc = copy_cache(0, early, lane.stream)) return rc;
+        DAF_CUDA_TRY(cudaEventRecord(lane.join, lane.stream));
+        if (int rc = do_select(rp, scores, n_sig, scores ? nullptr : a.idx_in, rows.q, rows.k, rows.v, a.kv_k, a.kv_v, a.idx_out, a.q_pack,
+                               a.k_pack, a.v_pack, ws, st, nullptr, &rows)) return rc;
+        DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
+        DAF_CUDA_TRY(cudaStreamWaitEvent(lane.stream, lane.fork, 0));
         if (int rc = launch_attention(a.q_pack, a.k_pack, a.v_pack, rp.k, rp.k, rp.Hq, rp.Hkv, 0, rp.scale, false, false, a.hidden,
                                       (long long)qrow, nullptr, nullptr, ws.status, nullptr, 0, lane.stream)) return rc;
         DAF_CUDA_TRY(cudaMemcpyAsync(h_hidden, a.hidden, qrow * rp.k, cudaMemcpyDeviceToHost, lane.stream));
@@ -517,8 +534,8 @@ int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows
         return DAF_OK;
     };
     auto question = [&]() -> int {
-        DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_k, h_kv_k, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
-        DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_v, h_kv_v, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
+        if (int rc = copy_cache(early, 2 * cache, st)) return rc;
+        DAF_CUDA_TRY(cudaStreamWaitEvent(st, lane.join, 0));
         if (rp.overwrite)
             if (int rc = launch_update_cache(rp, a.idx_out, a.k_pack, a.v_pack, a.kv_k, a.kv_v, st)) return rc;
         char* out = a.hidden + qrow * rp.k;
@@ -578,6 +595,14 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
     const bool rows_back = in_place_rows && mapped_host_pointer(h_kv_k, &host_k) && mapped_host_pointer(h_kv_v, &host_v) &&
                            aligned16(host_k) && aligned16(host_v);
     if (rows_back && copy_back_kv) { rows.host_k = const_cast<void*>(host_k); rows.host_v = const_cast<void*>(host_v); }
+    if (rows_back && rp.L_q > 0 && rp.fuse_mode == 0) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        DAF_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
+        SideLane* lane = capture == cudaStreamCaptureStatusNone ? side_lane() : nullptr;
+        if (lane != nullptr)
+            return host_layer_two_ways(rp, a, rows, h_scores ? a.scores : nullptr, n_sig,
+                                       reinterpret_cast<const char*>(h_q_fresh) + qrow * rp.L_d, h_kv_k, h_kv_v, h_hidden, h_idx_out, st, *lane);
+    }
     if (in_place_rows) {
         if (rp.L_q > 0)
             DAF_CUDA_TRY(cudaMemcpyAsync(reinterpret_cast<char*>(a.q_fresh) + qrow * rp.L_d,
@@ -587,13 +612,6 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
         DAF_CUDA_TRY(cudaMemcpyAsync(a.q_fresh, h_q_fresh, qrow * rp.N, cudaMemcpyHostToDevice, st));
         DAF_CUDA_TRY(cudaMemcpyAsync(a.k_fresh, h_k_fresh, kvrow * rp.N, cudaMemcpyHostToDevice, st));
         DAF_CUDA_TRY(cudaMemcpyAsync(a.v_fresh, h_v_fresh, kvrow * rp.N, cudaMemcpyHostToDevice, st));
-    }
-    if (rows_back && rp.L_q > 0 && rp.fuse_mode == 0) {
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        DAF_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
-        SideLane* lane = capture == cudaStreamCaptureStatusNone ? side_lane() : nullptr;
-        if (lane != nullptr)
-            return host_layer_two_ways(rp, a, rows, h_scores ? a.scores : nullptr, n_sig, h_kv_k, h_kv_v, h_hidden, h_idx_out, st, *lane);
     }
     // only the document rows of the cache carry information on entry
     DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_k, h_kv_k, kvrow * rp.L_d, cudaMemcpyHostToDevice, st));
