@@ -462,6 +462,7 @@ constexpr int kArenaSignalRows = 8;   // arena is sized for up to this many sign
 struct SideLane {
     cudaStream_t stream = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
+    bool other_busy = false;       // the thread's other lane still has work under way: another layer is on the link
     ~SideLane() {
         if (join) cudaEventDestroy(join);
         if (fork) cudaEventDestroy(fork);
@@ -474,13 +475,16 @@ SideLane* side_lane() {
     static thread_local unsigned turn = 0;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) { (void)cudaGetLastError(); return nullptr; }
-    SideLane& l = lanes[dev][turn++ & 1u];
+    SideLane& l = lanes[dev][turn & 1u];
+    const SideLane& other = lanes[dev][++turn & 1u];
     if ((l.stream == nullptr && cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking) != cudaSuccess) ||
         (l.fork == nullptr && cudaEventCreateWithFlags(&l.fork, cudaEventDisableTiming) != cudaSuccess) ||
         (l.join == nullptr && cudaEventCreateWithFlags(&l.join, cudaEventDisableTiming) != cudaSuccess)) {
         (void)cudaGetLastError();
         return nullptr;
     }
+    l.other_busy = other.stream != nullptr && cudaStreamQuery(other.stream) == cudaErrorNotReady;
+    (void)cudaGetLastError();
     return &l;
 }
 
@@ -507,9 +511,10 @@ int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows
     if (int rc = carve_workspace(rp, a.ws, a.ws_bytes, &ws)) return rc;
     rows.cache_later = true;
     // The gather kernel's reads leave some of the link idle (45 GB/s of 53), so part of the cache is copied beside it; the rest
-    // follows it, as much as keeps the link busy while the important rows are copied out.
+    // follows it, as much as keeps the link busy while the important rows are copied out.  (Not when another layer is on the
+    // link already, which then is better served one after the other: 32k layers, two at a time, 2.61 and 2.67 ms.)
     const size_t cache = kvrow * rp.L_d, out_bytes = qrow * rp.k;
-    const size_t early = 2 * cache > out_bytes ? (2 * cache - out_bytes) / kvrow * kvrow : 0;   // bytes of K, then of V
+    const size_t early = !lane.other_busy && 2 * cache > out_bytes ? (2 * cache - out_bytes) / kvrow * kvrow : 0;   // bytes of K, then of V
     auto copy_cache = [&](size_t from, size_t to, cudaStream_t s) -> int {
         const size_t k0 = from < cache ? from : cache, k1 = to < cache ? to : cache;
         const size_t v0 = from > cache ? from - cache : 0, v1 = to > cache ? to - cache : 0;
@@ -517,12 +522,15 @@ int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows
         if (v1 > v0) DAF_CUDA_TRY(cudaMemcpyAsync(a.kv_v + v0, reinterpret_cast<const char*>(h_kv_v) + v0, v1 - v0, cudaMemcpyHostToDevice, s));
         return DAF_OK;
     };
-    DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
-    DAF_CUDA_TRY(cudaStreamWaitEvent(lane.stream, lane.fork, 0));
     auto important = [&]() -> int {
-        DAF_CUDA_TRY(cudaMemcpyAsync(a.q_fresh + qrow * rp.L_d, h_q_question, qrow * rp.L_q, cudaMemcpyHostToDevice, lane.stream));
-        if (int rc = copy_cache(0, early, lane.stream)) return rc;
-        DAF_CUDA_TRY(cudaEventRecord(lane.join, lane.stream));
+        cudaStream_t first = lane.other_busy ? st : lane.stream;
+        if (!lane.other_busy) {
+            DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
+            DAF_CUDA_TRY(cudaStreamWaitEvent(lane.stream, lane.fork, 0));
+        }
+        DAF_CUDA_TRY(cudaMemcpyAsync(a.q_fresh + qrow * rp.L_d, h_q_question, qrow * rp.L_q, cudaMemcpyHostToDevice, first));
+        if (int rc = copy_cache(0, early, first)) return rc;
+        if (!lane.other_busy) DAF_CUDA_TRY(cudaEventRecord(lane.join, lane.stream));
         if (int rc = do_select(rp, scores, n_sig, scores ? nullptr : a.idx_in, rows.q, rows.k, rows.v, a.kv_k, a.kv_v, a.idx_out, a.q_pack,
                                a.k_pack, a.v_pack, ws, st, nullptr, &rows)) return rc;
         DAF_CUDA_TRY(cudaEventRecord(lane.fork, st));
@@ -535,7 +543,7 @@ int host_layer_two_ways(const ResolvedParams& rp, const Arena& a, RowSource rows
     };
     auto question = [&]() -> int {
         if (int rc = copy_cache(early, 2 * cache, st)) return rc;
-        DAF_CUDA_TRY(cudaStreamWaitEvent(st, lane.join, 0));
+        if (!lane.other_busy) DAF_CUDA_TRY(cudaStreamWaitEvent(st, lane.join, 0));
         if (rp.overwrite)
             if (int rc = launch_update_cache(rp, a.idx_out, a.k_pack, a.v_pack, a.kv_k, a.kv_v, st)) return rc;
         char* out = a.hidden + qrow * rp.k;
