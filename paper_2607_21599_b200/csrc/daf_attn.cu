@@ -67,11 +67,10 @@ struct SegArgs {
     float* part_lse;    // [n_splits][n_q][Hq]
 };
 
-// A launch runs one problem on a 3-D grid (head block, unit, split), or two problems from one list of
-// items on a 1-D grid (joint): the items of seg[1] first, then those of seg[0], heaviest units first.
+// A launch runs the items of seg[1] first (none in a launch of one problem), then those of seg[0], heaviest units first.  The
+// grid is one-dimensional: the token blocks of a long sequence can be more than the other dimensions of a grid may have.
 struct AttnArgs {
     SegArgs seg[2];
-    int joint;
     DeviceStatus* status;
 };
 
@@ -89,7 +88,7 @@ extern "C" int daf_dbg_read_laps(void* host, size_t bytes) {
 #define DAF_LAP(acc) do { const long long now_ = clock64(); acc += now_ - lap_t; lap_t = now_; } while (0)
 #define DAF_STAMP(slot)                                                                         \
     do {                                                                                        \
-        const unsigned cta_ = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);   \
+        const unsigned cta_ = blockIdx.x;                                                     \
         if (cta_ < 65536u) g_trace[8 * cta_ + (slot)] = global_ns();                            \
     } while (0)
 #else
@@ -197,26 +196,15 @@ struct CtaWork {
 __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
     // ---- which item is this CTA's (uniform across the CTA)
     int seg_id = 0, item = (int)blockIdx.x;
-    if (args.joint) {
-        if (item < args.seg[1].n_items) seg_id = 1;
-        else item -= args.seg[1].n_items;
-    }
+    if (item < args.seg[1].n_items) seg_id = 1;
+    else item -= args.seg[1].n_items;
     a.n_q = DAF_SEG(n_q); a.n_kv = DAF_SEG(n_kv); a.G = DAF_SEG(G); a.Gp = DAF_SEG(Gp); a.Tt = DAF_SEG(Tt);
     a.n_tb = DAF_SEG(n_tb); a.causal_off = DAF_SEG(causal_off); a.q_pos = DAF_SEG(q_pos); a.scale_log2 = DAF_SEG(scale_log2);
 
-    int hb, unit, split;
-    if (!args.joint) {
-        // blocks are dispatched x-fastest: all head blocks of the heaviest (last) unit go first
-        hb = (int)blockIdx.x; unit = (int)gridDim.y - 1 - (int)blockIdx.y; split = (int)blockIdx.z;
-    } else {
-        const int n_hb = DAF_SEG(head_blocks), n_units = DAF_SEG(n_units);
-        hb = item % n_hb;
-        const int rest = item / n_hb;
-        unit = n_units - 1 - rest % n_units;
-        split = rest / n_units;
-    }
-    const int steps = DAF_SEG(steps_per_split);
-    a.seg_id = seg_id; a.hb = hb; a.unit = unit;
+    // all head blocks of the heaviest (last) unit go first
+    const int n_hb = DAF_SEG(head_blocks), n_units = DAF_SEG(n_units), steps = DAF_SEG(steps_per_split);
+    const int rest = item / n_hb, split = rest / n_units;
+    a.seg_id = seg_id; a.hb = item % n_hb; a.unit = n_units - 1 - rest % n_units;
     a.j_begin = split * steps;
     a.j_end = a.j_begin + steps;
     a.item_splits = DAF_SEG(n_splits);
@@ -817,7 +805,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         }
 #ifdef DAF_TRACE
         if (threadIdx.x == 0) {
-            const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+            const unsigned cta = blockIdx.x;
             if (cta < 65536u) {
                 long long* t = g_laps + 8 * cta;
                 const long long now = clock64();
@@ -841,7 +829,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
 #ifdef DAF_TRACE
     if (threadIdx.x == 0) {
         DAF_STAMP(5);
-        const unsigned cta = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+        const unsigned cta = blockIdx.x;
         if (cta < 65536u) {
             g_trace[8 * cta + 6] = (unsigned long long)n_t;
             unsigned smid; asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
@@ -1273,10 +1261,8 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     s.part_lse = pl.n_splits > 1 ? reinterpret_cast<float*>(reinterpret_cast<char*>(scratch) +
                                                             (size_t)pl.n_splits * n_q * Hq * kD * sizeof(float))
                                  : nullptr;
-    a.joint = 0;
     a.status = status;
-    dim3 grid((unsigned)pl.head_blocks, (unsigned)pl.n_tb, (unsigned)pl.n_splits);
-    cudaError_t e = launch_kernel(attn_fwd_kernel<false>, grid, dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
+    cudaError_t e = launch_kernel(attn_fwd_kernel<false>, dim3((unsigned)s.n_items), dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
                                   to, to, tq, a);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
@@ -1378,7 +1364,6 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
     si.n_units = jp.n_tb_i;
     si.n_splits = 1; si.steps_per_split = (k + kSubN - 1) / kSubN;
     si.n_items = jp.items_i;
-    a.joint = 1;
     a.status = status;
 
     const int items = jp.items_q + jp.items_i;

@@ -389,6 +389,22 @@ def test_full_causal_attention_matches_oracle(n, Hq, Hkv):
     _assert_close(out, ref, f"full causal n={n}")
 
 
+def test_full_causal_attention_over_more_token_blocks_than_a_grid_has_rows():
+    """128 query heads on one KV head, one token per tile: 65 600 token blocks.  Rows at both ends and around the 65 536th
+    against softmax attention in 64 bits."""
+    n, H = 65600, 128
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, k, v = (torch.randn((n, h, 128), generator=g, device="cuda", dtype=torch.bfloat16) for h in (H, 1, 1))
+    p = api.make_params(64, 0, 1.0, H, 1)
+    ws = api.alloc_workspace(p)
+    out = torch.full((n, H, 128), 5.0, dtype=torch.bfloat16, device="cuda")
+    _ok(api.daf_full_causal_attn(p, n, q, k, v, out, None, ws), ws, "daf_full_causal_attn")
+    for t in (0, 1, 63, 64, 32768, 65534, 65535, 65536, n - 1):
+        s = q[t].double() @ k[: t + 1, 0].double().T / math.sqrt(128)
+        ref = torch.softmax(s, dim=1) @ v[: t + 1, 0].double()
+        _assert_close(out[t], ref.cpu().numpy(), f"row {t}")
+
+
 @pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv", [(1024, 32, 0.15, 28, 4), (700, 5, 0.3, 8, 2), (2048, 128, 0.05, 40, 8),
                                                (300, 0, 1.0, 4, 4)])
 def test_full_context_variant_matches_oracle(L_d, L_q, r, Hq, Hkv):
