@@ -328,7 +328,7 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     // the question rows are read from q_fresh even when nothing is selected (r = 0)
     if (rp.L_q > 0 && (q_fresh == nullptr || kv_k == nullptr || kv_v == nullptr)) return DAF_ERR_INVALID_ARG;
     if (rp.k > 0 && (q_fresh == nullptr || (k_pack == nullptr) != (v_pack == nullptr))) return DAF_ERR_INVALID_ARG;
-    if (q_fresh != nullptr && !aligned16(q_fresh)) return DAF_ERR_ALIGNMENT;
+    if ((q_fresh != nullptr && !aligned16(q_fresh)) || (q_pack != nullptr && !aligned16(q_pack))) return DAF_ERR_ALIGNMENT;
     const int64_t row_bytes = (int64_t)rp.Hq * 256;
     if (int rc = check_out(hidden, row_bytes, rp.Hq)) return rc;
     // Step 2 reads its Q rows in place and packs them on the way (the largest of the packed tensors: the gather kernel is left

@@ -107,6 +107,13 @@ def test_host_side_argument_validation(lib):
     assert api.daf_layer(r0, None, 0, None, buf, buf, buf, None, buf, None, None, None, None, buf, None, ws) == api.DAF_ERR_INVALID_ARG
     # important rows without packed K/V buffers
     assert api.daf_layer(ok, buf, 1, None, buf, buf, buf, buf, buf, buf, buf, None, buf, buf, None, ws) == api.DAF_ERR_INVALID_ARG
+    # every buffer of a layer in turn off by 8 bytes (the packed Q rows too, which the attention kernel may be the one to write)
+    fresh, cache = torch.zeros(4096, dtype=torch.uint8), torch.zeros(4096, dtype=torch.uint8)
+    whole = [buf, None, fresh, fresh, fresh, cache, cache, buf, buf, buf, buf, buf]    # scores, idx_in, q/k/v, cache, idx_out, packed, hidden
+    for i in (0, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11):
+        a = list(whole)
+        a[i] = a[i][8:]
+        assert api.daf_layer(ok, a[0], 1, *a[1:], None, ws) == api.DAF_ERR_ALIGNMENT, i
     # selection straight from the signal layers' K/V: the number of layers and every pointer are checked first
     sig = lambda n: [buf] * n  # noqa: E731
     skv = lambda n, kf=None, wsp=ws: api.daf_select_from_kv(ok, kf if kf is not None else sig(n), sig(n), sig(n), sig(n), buf, buf, buf,  # noqa: E731
