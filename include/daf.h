@@ -245,6 +245,8 @@ int daf_full_causal_attn(const daf_params* p, int32_t n_tokens, const void* q, c
  * epilogues (device pointers; arguments as in daf_select, plus)
  *   hidden       compact: [k+L_q, n_q_heads*128]; scatter: [N, n_q_heads*128]
  *   row_pos_out  optional int32 [k+L_q]
+ *                With q_pack given it may share memory with rows of q_fresh below L_d (in scatter mode with all of it, at
+ *                the same address), and in compact mode begin with q_pack; what was there before is then lost.
  *   q_pack       may be NULL when L_q > 0.  (When L_q > 0 step 2 reads its Q rows in place either way; a buffer given
  *                receives the packed rows on the way.)
  *   k_pack, v_pack  may be NULL (both or neither) when k > 0 and L_q > 0: step 2 then reads its K/V rows in

@@ -866,6 +866,42 @@ def test_layer_leaves_the_packed_q_rows_it_read_in_place(L_d, L_q, r, Hq, Hkv, g
     assert torch.equal(qp[:k], g["q_fresh"][idx_out.long()]) and torch.all(qp[k] == 3.0)
 
 
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv,fuse_mode,shares", [
+    (3000, 40, 0.3, 14, 2, 0, "q_fresh"), (3000, 40, 0.3, 14, 2, 0, "q_fresh+512"), (3000, 40, 0.3, 14, 2, 0, "q_pack"),
+    (3000, 40, 0.3, 14, 2, 1, "q_fresh"), (2000, 9, 0.4, 4, 4, 0, "q_fresh"), (2000, 9, 0.4, 4, 4, 0, "q_pack"),
+    (2000, 9, 0.4, 16, 1, 0, "q_pack")])
+def test_layer_whose_output_rows_lie_where_its_q_rows_were(L_d, L_q, r, Hq, Hkv, fuse_mode, shares, given):
+    """`hidden` on the memory of q_fresh, of rows further on in it, or of q_pack: the same bits as with buffers of their own."""
+    w = W.Workload("t", 44, Hq, Hkv, 128, 1, L_d, L_d, L_q, r, "lognormal", 1)
+    L = W.make_layer(w, 0)
+    p = api.make_params(L_d, L_q, r, Hq, Hkv, fuse_mode=fuse_mode)
+    k, N = api.daf_num_important(L_d, r), L_d + L_q
+    rows = N if fuse_mode == 1 else k + L_q
+    idx = torch.from_numpy(oracle.select(L["scores"].numpy(), k)).cuda()
+    ws = api.alloc_workspace(p)
+    outs = []
+    for apart in (True, False):
+        g = {n: t.cuda() for n, t in L.items() if t is not None}
+        kv = [torch.cat([g[n], torch.zeros(L_q, Hkv, 128, dtype=torch.bfloat16, device="cuda")]) for n in ("k_cached", "v_cached")]
+        qp = torch.zeros((k + L_q if shares == "q_pack" else k), Hq, 128, dtype=torch.bfloat16, device="cuda")
+        if apart:
+            hidden = torch.zeros(rows, Hq, 128, dtype=torch.bfloat16, device="cuda")
+        elif shares == "q_pack":
+            hidden = qp
+        else:
+            hidden = g["q_fresh"][512 if shares == "q_fresh+512" else 0:][:rows]
+        kp, vp = (torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        idx_out = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+        _ok(api.daf_layer(p, None if given else g["scores"], 1, idx if given else None, g["q_fresh"], g["k_fresh"], g["v_fresh"],
+                          kv[0], kv[1], idx_out, qp[:k], kp, vp, hidden, None, ws), ws, "daf_layer")
+        pos = torch.cat([idx.long(), torch.arange(L_d, N, device="cuda")])
+        outs.append((hidden[pos] if fuse_mode == 1 else hidden).clone())
+    assert torch.equal(outs[0], outs[1])
+    ref = _oracle_layer(w, L, 0)["hidden"]
+    _assert_close(outs[1], ref, "rows written over the Q rows")
+
+
 @pytest.mark.parametrize("fuse_mode", [0, 1])
 def test_layer_without_packed_q_buffer(fuse_mode):
     """daf_layer with q_pack = NULL (step 2 reads its Q rows in place) gives the same bits as with the buffer,
