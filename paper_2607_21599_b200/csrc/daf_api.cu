@@ -339,12 +339,13 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     // Step 2 reads its Q rows in place and packs them on the way (the largest of the packed tensors: the gather kernel is left
     // with K/V), unless they lie in host memory: 6k layer 32.9 -> 31.4 us, 11k 113.9 -> 112.2, 28 layers of 6k 728 -> 716, 16k
     // 87.4 -> 87.7 (there the longer start of an item, positions and then rows from HBM, weighs as much as the copy saved).
-    // Not when the output rows share memory with what step 2 would still be reading or packing: then the gather kernel packs.
+    // Not with many tokens in a tile, where that is slower (step2_packs_q), nor when the output rows share memory with what
+    // step 2 would still be reading or packing: then the gather kernel packs.
     const size_t hidden_bytes = (size_t)row_bytes * (rp.fuse_mode == 1 ? rp.N : rp.k + rp.L_q);
     const bool shared = overlap(hidden, hidden_bytes, q_fresh, (size_t)row_bytes * rp.N) ||
                         overlap(hidden, hidden_bytes, q_pack, (size_t)row_bytes * rp.k) ||
                         (scores == nullptr && overlap(hidden, hidden_bytes, idx_in, (size_t)rp.k * 4));
-    const bool q_in_place = rows == nullptr && rp.k > 0 && rp.L_q > 0 && (q_pack == nullptr || !shared);
+    const bool q_in_place = rows == nullptr && rp.k > 0 && rp.L_q > 0 && (q_pack == nullptr || (!shared && step2_packs_q(rp.k, rp.L_q, rp.L_d, rp.Hq, rp.G)));
     if (int rc = do_select(rp, scores, n_sig, idx_in, rows ? rows->q : q_fresh, rows ? rows->k : k_fresh,
                            rows ? rows->v : v_fresh, kv_k, kv_v, idx_out, q_in_place ? nullptr : q_pack, k_pack,
                            v_pack, ws, st, rp.L_d > 0 ? fp8 : nullptr,

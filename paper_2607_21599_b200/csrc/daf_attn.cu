@@ -40,9 +40,11 @@ struct SegArgs {
     int n_tb;           // token blocks = ceil(n_q / Tt)
     int causal_off;     // token t sees keys <= t + causal_off ...
     const int32_t* q_pos; // ... or, when given, keys <= q_pos[t] (ascending positions of the query tokens)
-    // Query rows read in place instead of from a packed copy: query token t is row q_idx[t] of a tensor of q_src_rows rows
-    // (which the Q tensor map then covers, with a box of one token).  q_idx == nullptr: the map covers packed rows.
+    // Query rows read in place instead of from a packed copy: query token t is row q_idx[t] of a tensor of q_src_rows rows.
+    // q_idx == nullptr: the Q tensor map covers packed rows.  q_src == nullptr: it covers that tensor, with a box of one
+    // token, and a warp issues a copy per token; otherwise the softmax warps fetch the rows from q_src (see copies_per_token).
     const int32_t* q_idx;
+    const __nv_bfloat16* q_src;
     int q_src_rows;
     int q_early;        // q_idx and the rows are complete before the kernel launched just before this one started
     int q_save;         // the tiles so fetched are also written out as packed rows (second Q map)
@@ -400,7 +402,9 @@ struct AttnSmem {
 };
 constexpr size_t kAttnSmemBytes = 1024 + 3 * (size_t)kTileBytes + sizeof(AttnSmem);
 
-template <bool kGatherKV>
+// kGatherKV: the launch has a problem whose K/V rows three warps fetch in place through an index; kFetchQ: one whose Q rows the
+// softmax warps fetch.  Forms of their own, so that the plain form carries none of that code.
+template <bool kGatherKV, bool kFetchQ>
 __global__ void __launch_bounds__(kGatherKV ? kAttnThreadsGather : kAttnThreads, 2)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_constant__ CUtensorMap tmap_k0,
                   const __grid_constant__ CUtensorMap tmap_v0, const __grid_constant__ CUtensorMap tmap_q1,
@@ -429,8 +433,6 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     const int g_kv = h0 / a.G;
     const int t0 = a.unit * a.Tt;
     const int key_begin = a.j_begin * kSubN;
-    // kGatherKV: the launch has a problem whose K/V rows the producer warp fetches in place through an index (k_src
-    // non-null); a form of its own, so that the plain form carries none of that code
     const __nv_bfloat16* const k_src = kGatherKV ? DAF_SEG(k_src) : nullptr;
     const bool kv_gather = kGatherKV && k_src != nullptr;
     const int gather_warp = warp == 4 ? 0 : warp - 5;    // 0, 1, 2 for warps 4, 6, 7 (meaningful only for those)
@@ -506,6 +508,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     // dependent launch it runs while the kernel launched just before (gather / hybrid-cache update) drains.
     __shared__ int skip_cta;
     const int32_t* const q_idx = DAF_SEG(q_idx);     // non-null: Q rows are fetched token by token through this list
+    const __nv_bfloat16* const q_src = kFetchQ ? DAF_SEG(q_src) : nullptr;
     const bool q_save = q_idx != nullptr && DAF_SEG(q_save) != 0;
     const bool q_early = q_idx != nullptr && DAF_SEG(q_early) != 0;
     int q_first = -1;            // position of this lane's first token: asked for ahead of everything else
@@ -515,7 +518,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         tmem_relinquish();
     }
     if (warp == 4 && lane == 0) {
-        mbar_init(&sm->q_full, 1); mbar_init(&sm->q_saved, 1);
+        mbar_init(&sm->q_full, q_src != nullptr ? 4 : 1); mbar_init(&sm->q_saved, 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(&sm->k_full[s], kv_gather ? 32 * kGatherWarps : 1); mbar_init(&sm->v_full[s], kv_gather ? 32 * kGatherWarps : 1);
             mbar_init(&sm->s_full[s], 1); mbar_init(&sm->p_full[s], 4);
@@ -556,7 +559,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         hi = min(hi, (long long)a.j_end * kSubN);
         if (hi > key_begin) n_t = (int)((hi - key_begin + kSubN - 1) / kSubN);
     }
-    if (warp == 4 && q_idx != nullptr && !q_early) fetch_q();
+    if (warp == 4 && q_idx != nullptr && q_src == nullptr && !q_early) fetch_q();
     if (warp == 4 && lane == 0) {
         if (n_t > 0) {
             if (q_idx == nullptr) {
@@ -568,8 +571,33 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
                 for (int t = 0; t < 2 && t < n_t; ++t) { issue_kv(t, 0); issue_kv(t, 1); }
         }
     }
+    if (q_src != nullptr && n_t > 0 && warp < 4) {
+        // each warp fetches its 32 rows (16 lanes per 256-byte row) into the layout of the tiled copy (two 64-column halves of
+        // 128-byte rows, 16-byte chunks XOR-ed with the row number mod 8); rows without a token are zeros
+        const int rows = DAF_SEG(q_src_rows), Hq = DAF_SEG(Hq);
+        const int sub = lane >> 4, cidx = lane & 15, r0 = warp * 32 + sub;
+        int tok = t0 + r0 / a.Gp, head = r0 % a.Gp;
+        uint4 w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            w[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (r0 + 2 * i < a.Gp * a.Tt && tok < a.n_q) {
+                const int src = __ldg(q_idx + tok);
+                if ((unsigned)src < (unsigned)rows)   // a bad position is reported by the gather kernel
+                    w[i] = __ldg(reinterpret_cast<const uint4*>(q_src + ((size_t)src * Hq + h0 + head) * kD) + cidx);
+            }
+            tok += 2 / a.Gp; head += 2 % a.Gp;
+            if (head >= a.Gp) { head -= a.Gp; ++tok; }
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int rr = r0 + 2 * i;
+            *reinterpret_cast<uint4*>(q_smem + (cidx >> 3) * kHalfBytes + rr * 128 + (((cidx & 7) ^ (rr & 7)) << 4)) = w[i];
+        }
+        fence_proxy_async();
+    }
     // rows of the Q tile that the loads do not fill: zeros
-    if (warp == 3) {
+    if (warp == 3 && q_src == nullptr) {
         const int used = a.Gp * (q_idx == nullptr ? a.Tt : min(a.Tt, a.n_q - t0));
         for (int i = lane; i < (kBlockM - used) * 16; i += 32)
             *reinterpret_cast<uint4*>(q_smem + ((i >> 3) & 1) * kHalfBytes + (used + (i >> 4)) * 128 + ((i & 7) << 4)) = make_uint4(0u, 0u, 0u, 0u);
@@ -609,7 +637,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     if (skip) {
         // nothing is computed; the loads already under way get a bounded chance to land before the CTA retires
         if (warp == 4 && lane == 0 && n_t > 0) {
-            for (int i = 0; i < 4096 && !mbar_try_wait(&sm->q_full, 0); ++i) {}
+            for (int i = 0; i < 4096 && q_src == nullptr && !mbar_try_wait(&sm->q_full, 0); ++i) {}
             for (int s = 0; s < 2 && s < n_t && !kv_gather; ++s) {
                 for (int i = 0; i < 4096 && !mbar_try_wait(&sm->k_full[s], 0); ++i) {}
                 for (int i = 0; i < 4096 && !mbar_try_wait(&sm->v_full[s], 0); ++i) {}
@@ -757,6 +785,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         const uint32_t o_addr = tmem + lane_addr + (uint32_t)kBlockN;
         const float c = a.scale_log2;
 
+        if (q_src != nullptr && n_t > 0 && lane == 0) mbar_arrive(&sm->q_full);   // this warp's Q rows were stored before the set-up barrier
         float m = -INFINITY, l = 0.f;
         bool ok = true;
         DAF_LAP_DECL;
@@ -961,9 +990,11 @@ static int set_kernel_attributes() {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_done[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmemBytes);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(attn_fwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmemBytes);
+            e = cudaFuncSetAttribute(attn_fwd_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmemBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(attn_fwd_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAttnSmemBytes);
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         attr_done[dev].store(true, std::memory_order_release);
     }
@@ -1262,7 +1293,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
                                                             (size_t)pl.n_splits * n_q * Hq * kD * sizeof(float))
                                  : nullptr;
     a.status = status;
-    cudaError_t e = launch_kernel(attn_fwd_kernel<false>, dim3((unsigned)s.n_items), dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
+    cudaError_t e = launch_kernel(attn_fwd_kernel<false, false>, dim3((unsigned)s.n_items), dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
                                   to, to, tq, a);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
@@ -1291,6 +1322,15 @@ int launch_bounded_wait_selftest(DeviceStatus* status, int limit_ms, cudaStream_
     return check_launch();
 }
 
+// Q rows in place by one tiled copy per token and half row: for tiles of up to 32 tokens, one for each lane of the warp that
+// issues them.  The copies of longer tiles (fewer than four heads in them) queue up behind one another: there packed rows are
+// better, and where there is no buffer for them the softmax warps fetch the rows.  Layer with 32 heads on 32 over 1325 tokens,
+// 133 important: 14.9 us from packed rows, 21.0 by copies per token; 22 important of 438: 16.2 and 15.9; without a buffer 1017
+// of 3390: 30.8 by the softmax warps, 40.7 by copies per token.
+constexpr int kMaxTokenCopies = 32;
+static bool copies_per_token(const JointPlan& jp, int k) { return (jp.Tt_i < k ? jp.Tt_i : k) <= kMaxTokenCopies; }
+bool step2_packs_q(int k, int L_q, int L_d, int Hq, int G) { return copies_per_token(plan_joint(k, L_q, L_d, Hq, G), k); }
+
 size_t joint_partial_bytes(const JointPlan& jp) { return jp.part_bytes_q; }
 
 int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_place, bool q_early, const int32_t* idx, const void* k_imp, const void* v_imp,
@@ -1308,7 +1348,11 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
     // Q rows in place: read through idx, and left in q_imp as packed rows where the caller wants them
     const bool gather_q = q_in_place;
     if (gather_q ? (q_fresh == nullptr || idx == nullptr) : q_imp == nullptr) return DAF_ERR_INVALID_ARG;
-    if (int rc = gather_q ? make_tmap(&tq0, q_fresh, L_d, Hq, jp.Gp_i, 1) : make_tmap(&tq0, q_imp, k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
+    const bool by_warps = gather_q && !copies_per_token(jp, k);
+    if (by_warps && q_imp != nullptr) return DAF_ERR_INVALID_ARG;      // these do not pack
+    if (int rc = by_warps   ? make_tmap(&tq0, q_question, L_q, Hq, jp.Gp_q, jp.Tt_q)     // (not used)
+                 : gather_q ? make_tmap(&tq0, q_fresh, L_d, Hq, jp.Gp_i, 1)
+                            : make_tmap(&tq0, q_imp, k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
     CUtensorMap tqp = tq0;
     if (gather_q && q_imp != nullptr)
         if (int rc = make_tmap(&tqp, q_imp, k, Hq, jp.Gp_i, jp.Tt_i)) return rc;
@@ -1350,7 +1394,8 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
     if (gather_q) {
         si.q_idx = idx;
         si.q_src_rows = L_d;
-        si.q_early = q_early ? 1 : 0;
+        si.q_src = by_warps ? reinterpret_cast<const __nv_bfloat16*>(q_fresh) : nullptr;
+        si.q_early = q_early && !by_warps ? 1 : 0;
         si.q_save = q_imp != nullptr ? 1 : 0;
     }
     if (gather_kv) {
@@ -1368,11 +1413,9 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
 
     const int items = jp.items_q + jp.items_i;
     if (launches & 1) {
-        const cudaError_t e = gather_kv
-            ? launch_kernel(attn_fwd_kernel<true>, dim3((unsigned)items), dim3(kAttnThreadsGather), kAttnSmemBytes, stream,
-                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, tqp, a)
-            : launch_kernel(attn_fwd_kernel<false>, dim3((unsigned)items), dim3(kAttnThreads), kAttnSmemBytes, stream,
-                            tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, tqp, a);
+        auto* kernel = gather_kv ? attn_fwd_kernel<true, true> : by_warps ? attn_fwd_kernel<false, true> : attn_fwd_kernel<false, false>;
+        const cudaError_t e = launch_kernel(kernel, dim3((unsigned)items), dim3(gather_kv ? kAttnThreadsGather : kAttnThreads),
+                                            kAttnSmemBytes, stream, tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, tqp, a);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         if (int rc = check_launch()) return rc;

@@ -74,8 +74,10 @@ struct JointPlan {
 };
 JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G);
 size_t joint_partial_bytes(const JointPlan& jp);
+bool step2_packs_q(int k, int L_q, int L_d, int Hq, int G);     // step 2 can read its Q rows in place and pack them on the way
 int launch_bounded_wait_selftest(DeviceStatus* status, int limit_ms, cudaStream_t stream);
-// q_in_place: the important rows' Q is read in place, row idx[j] of q_fresh, and packed into q_imp (if not null) on the way;
+// q_in_place: the important rows' Q is read in place, row idx[j] of q_fresh, and packed into q_imp (if not null, and only
+// where step2_packs_q) on the way;
 // q_early: idx and q_fresh are complete before the kernel launched just before started;
 // k_imp == nullptr (then v_imp too): their K and V are read in place, rows idx[j] of k_fresh / v_fresh
 int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_place, bool q_early, const int32_t* idx, const void* k_imp, const void* v_imp,

@@ -902,6 +902,35 @@ def test_layer_whose_output_rows_lie_where_its_q_rows_were(L_d, L_q, r, Hq, Hkv,
     _assert_close(outs[1], ref, "rows written over the Q rows")
 
 
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv", [(700, 9, 0.3, 4, 4), (90, 3, 0.01, 2, 2), (330, 3, 0.1, 4, 4), (320, 3, 0.1, 4, 4),
+                                              (1000, 20, 0.13, 6, 3), (300, 5, 0.43, 4, 2), (1000, 20, 0.13, 12, 4), (260, 3, 0.17, 3, 1), (900, 4, 0.2, 129, 1)])
+def test_layer_without_packed_q_buffer_and_with_long_tiles(L_d, L_q, r, Hq, Hkv, given):
+    """One, two and three heads per tile (rows fetched by the softmax warps above 32 tokens), whole, partial and single-token
+    last tiles: the same bits as with a buffer, which holds the fresh rows at the selected positions."""
+    w = W.Workload("t", 45, Hq, Hkv, 128, 1, L_d, L_d, L_q, r, "lognormal", 1)
+    L = W.make_layer(w, 0)
+    p = api.make_params(L_d, L_q, r, Hq, Hkv)
+    k = api.daf_num_important(L_d, r)
+    idx = torch.from_numpy(oracle.select(L["scores"].numpy(), k)).cuda()
+    g = {n: t.cuda() for n, t in L.items() if t is not None}
+    ws = api.alloc_workspace(p)
+    outs = []
+    for qp in (torch.full((k + 1, Hq, 128), 3.0, dtype=torch.bfloat16, device="cuda"), None):
+        kv = [torch.cat([g[n], torch.zeros(L_q, Hkv, 128, dtype=torch.bfloat16, device="cuda")]) for n in ("k_cached", "v_cached")]
+        kp, vp = (torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        idx_out = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+        hidden = torch.zeros(k + L_q, Hq, 128, dtype=torch.bfloat16, device="cuda")
+        _ok(api.daf_layer(p, None if given else g["scores"], 1, idx if given else None, g["q_fresh"], g["k_fresh"], g["v_fresh"],
+                          kv[0], kv[1], idx_out, qp, kp, vp, hidden, None, ws), ws, "daf_layer")
+        assert torch.equal(idx_out, idx)
+        if qp is not None:
+            assert torch.equal(qp[:k], g["q_fresh"][idx.long()]) and torch.all(qp[k] == 3.0)
+        outs.append(hidden)
+    assert torch.equal(outs[0], outs[1])
+    _assert_close(outs[1], _oracle_layer(w, L, 0)["hidden"], "Q rows in place")
+
+
 @pytest.mark.parametrize("fuse_mode", [0, 1])
 def test_layer_without_packed_q_buffer(fuse_mode):
     """daf_layer with q_pack = NULL (step 2 reads its Q rows in place) gives the same bits as with the buffer,
