@@ -24,9 +24,11 @@ namespace daf {
 constexpr int kBlockM = 128;            // rows per query tile
 constexpr int kBlockN = 128;            // tensor-memory columns of the logits: two sub-steps of 64 keys
 constexpr int kD = 128;                 // head_dim
+constexpr int kSubN = 64;               // keys per sub-step
 constexpr int kTileBytes = kBlockN * kD * 2;      // 32 KB: one Q tile, or two sub-steps of K (or V)
 constexpr int kHalfBytes = kTileBytes / 2;        // one 64-column half (128-byte rows)
 constexpr int kMaxSplits = 32;
+constexpr int kMaxChainRanges = 6;      // into how many ranges a causal chain may be cut
 constexpr int kNumSMsDefault = 148;    // B200; the planners ask the device (num_sms below)
 constexpr float kRescaleThreshold = 8.0f;   // in log2 units: keep a stale row maximum up to 2^8
 
@@ -54,19 +56,22 @@ struct SegArgs {
     const __nv_bfloat16* v_src;
     const int32_t* kv_idx;
     int kv_src_rows, kv_heads;
-    // Work items.  A CTA owns one token block (a unit) of one head block, and one of n_splits KV ranges of
-    // steps_per_split sub-steps (64 keys each).
+    // Work items.  A CTA owns one token block (a unit) of one head block, and one range of its keys: either one of n_splits
+    // ranges of steps_per_split sub-steps (64 keys each), the same for every unit, or (chunk > 0, causal attention over the
+    // problem's own keys) units [g chunk, (g + 1) chunk) are cut into g + 1 equal ranges each, so that no item walks more
+    // than about Tt * chunk keys.
     int head_blocks, n_units;
     int n_splits, steps_per_split;
-    int n_items;           // head_blocks * n_units * n_splits
+    int chunk, n_slots;    // n_slots: number of (unit, range) pairs
+    int n_items;           // head_blocks * (n_units * n_splits  or  n_slots)
     float scale;        // softmax scale
     float scale_log2;   // scale * log2(e)
     __nv_bfloat16* out; long long out_row_stride;  // elements
     const int32_t* dst_rows;
     int out_tiled;      // final rows leave by one tiled bulk store per tile (rows in token order, no dst_rows)
     float* lse;         // [Hq, n_q] or null
-    float* part_o;      // partial results, fp32, normalised per range: [n_splits][n_q][Hq][128]
-    float* part_lse;    // [n_splits][n_q][Hq]
+    float* part_o;      // partial results, fp32, normalised per range: [n_splits][n_q][Hq][128], or [n_slots][Tt][Hq][128]
+    float* part_lse;    // the same without the last dimension
 };
 
 // A launch runs the items of seg[1] first (none in a launch of one problem), then those of seg[0], heaviest units first.  The
@@ -192,9 +197,10 @@ struct CtaWork {
     const int32_t* q_pos;
     float scale_log2;
     int seg_id, hb, unit, j_begin, j_end, item_splits;
-    long long part_row0;      // first row of the item's range in the partial-result arrays, in tokens
+    long long part_row0;      // the item's partial rows: token t's are number part_row0 + t of the partial-result arrays
 };
 
+template <bool kExtra>
 __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
     // ---- which item is this CTA's (uniform across the CTA)
     int seg_id = 0, item = (int)blockIdx.x;
@@ -204,6 +210,20 @@ __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
     a.n_tb = DAF_SEG(n_tb); a.causal_off = DAF_SEG(causal_off); a.q_pos = DAF_SEG(q_pos); a.scale_log2 = DAF_SEG(scale_log2);
 
     // all head blocks of the heaviest (last) unit go first
+    if (kExtra && DAF_SEG(chunk) > 0) {
+        // slot numbers ascend with the unit: group g's first slot is chunk g (g + 1) / 2
+        const int chunk = DAF_SEG(chunk), heads = DAF_SEG(head_blocks), slot = DAF_SEG(n_slots) - 1 - item / heads;
+        int g = 0;
+        while (chunk * (g + 1) * (g + 2) / 2 <= slot) ++g;       // (at most a few ranges per unit)
+        const int rem = slot - chunk * g * (g + 1) / 2, range = rem % (g + 1);
+        a.seg_id = seg_id; a.hb = item % heads; a.unit = g * chunk + rem / (g + 1);
+        const int n_steps = (min((a.unit + 1) * a.Tt, a.n_q) + kSubN - 1) / kSubN;
+        a.j_begin = range * n_steps / (g + 1);
+        a.j_end = (range + 1) * n_steps / (g + 1);
+        a.item_splits = g + 1;
+        a.part_row0 = (long long)(slot - a.unit) * a.Tt;
+        return;
+    }
     const int n_hb = DAF_SEG(head_blocks), n_units = DAF_SEG(n_units), steps = DAF_SEG(steps_per_split);
     const int rest = item / n_hb, split = rest / n_units;
     a.seg_id = seg_id; a.hb = item % n_hb; a.unit = n_units - 1 - rest % n_units;
@@ -382,7 +402,6 @@ extern "C" int daf_dbg_read_trace(void* host, size_t bytes) {
 // leave by tiled bulk stores from the dead Q tile.
 // Two tiles per CTA sharing every K/V tile (half the shared-memory fill traffic, one CTA per SM)
 // measured slower at every size from 1k to 136k tokens and was removed.
-constexpr int kSubN = 64;                               // keys per sub-step
 constexpr int kSubBytes = kSubN * kD * 2;               // 16 KB: K or V of one sub-step, two 64-column halves
 constexpr int kSubHalfBytes = kSubBytes / 2;
 constexpr int kAttnThreads = 192;                      // warps 0-3 softmax, warp 4 TMA, warp 5 MMA
@@ -402,9 +421,9 @@ struct AttnSmem {
 };
 constexpr size_t kAttnSmemBytes = 1024 + 3 * (size_t)kTileBytes + sizeof(AttnSmem);
 
-// kGatherKV: the launch has a problem whose K/V rows three warps fetch in place through an index; kFetchQ: one whose Q rows the
-// softmax warps fetch.  Forms of their own, so that the plain form carries none of that code.
-template <bool kGatherKV, bool kFetchQ>
+// kGatherKV: the launch has a problem whose K/V rows three warps fetch in place through an index; kExtra: one whose Q rows the
+// softmax warps fetch, or whose causal chains are cut.  Forms of their own, so that the plain form carries none of that code.
+template <bool kGatherKV, bool kExtra>
 __global__ void __launch_bounds__(kGatherKV ? kAttnThreadsGather : kAttnThreads, 2)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_constant__ CUtensorMap tmap_k0,
                   const __grid_constant__ CUtensorMap tmap_v0, const __grid_constant__ CUtensorMap tmap_q1,
@@ -423,7 +442,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     DAF_KT_BEGIN(0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     CtaWork a;
-    decode_work(args, a);
+    decode_work<kExtra>(args, a);
     const int seg_id = a.seg_id;
     const CUtensorMap* tmap_q = seg_id ? &tmap_q1 : &tmap_q0;
     const CUtensorMap* tmap_k = seg_id ? &tmap_k1 : &tmap_k0;
@@ -508,8 +527,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     // dependent launch it runs while the kernel launched just before (gather / hybrid-cache update) drains.
     __shared__ int skip_cta;
     const int32_t* const q_idx = DAF_SEG(q_idx);     // non-null: Q rows are fetched token by token through this list
-    const __nv_bfloat16* const q_src = kFetchQ ? DAF_SEG(q_src) : nullptr;
-    const bool q_save = q_idx != nullptr && DAF_SEG(q_save) != 0;
+    const __nv_bfloat16* const q_src = kExtra ? DAF_SEG(q_src) : nullptr;
+    const bool q_save = q_idx != nullptr && DAF_SEG(q_save) != 0 && (!kExtra || a.j_begin == 0);    // (once per tile)
     const bool q_early = q_idx != nullptr && DAF_SEG(q_early) != 0;
     int q_first = -1;            // position of this lane's first token: asked for ahead of everything else
     if (warp == 4 && q_early && lane < min(a.Tt, a.n_q - t0)) q_first = __ldcg(q_idx + t0 + lane);
@@ -876,6 +895,7 @@ struct CombineArgs {
     const float* part_o; const float* part_lse;
     int n_q, Hq;
     int n_splits;        // partials per row, n_q * Hq rows apart
+    int chunk, unit_tokens, tok_first;   // chunk > 0: cut causal chains, tokens tok_first on (the others' rows are final)
     __nv_bfloat16* out; long long out_row_stride; const int32_t* dst_rows; float* lse;
 };
 
@@ -883,20 +903,35 @@ struct CombineArgs {
 // log-sum-exps are requested at once (a second round is a second trip to L2: as eight and then four by four, 24 tokens of 28
 // heads over 14k keys, 22 ranges, took 22.4 us with their attention, at once 19.8; 28 layers of 6k, 7 ranges, 747 against 726).  Two CTAs per SM are asked for so that
 // the compiler has the registers to keep them all under way.
-template <int kMost>
+// kCut: the launch also merges the rows of a problem whose causal chains are cut (c), ahead of the others.
+template <int kMost, bool kCut>
 __global__ void __launch_bounds__(256, 2)
-attn_combine_kernel(const CombineArgs a) {
+attn_combine_kernel(const CombineArgs a, const CombineArgs c) {
     DAF_KT_BEGIN(2);
     pdl_wait();                // partial results come from the attention kernel launched just before
     DAF_KT_BEGIN(3);
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    const int Hq = a.Hq, n_q = a.n_q, n_splits = a.n_splits;
-    if (row >= n_q * Hq) return;
-    const size_t stride = (size_t)n_q * Hq;      // rows from one partial to the next
-    const float* const lse_src = a.part_lse + row;
-    const float4* const src = reinterpret_cast<const float4*>(a.part_o + (size_t)row * kD) + lane;
-    const int tok = row / Hq, head = row - tok * Hq;
+    const int cut_rows = kCut ? (c.n_q - c.tok_first) * c.Hq : 0;
+    const bool cut = kCut && row < cut_rows;
+    if (kCut && !cut) row -= cut_rows;
+#define DAF_CS(field) (kCut && cut ? c.field : a.field)
+    const int Hq = DAF_CS(Hq), n_q = DAF_CS(n_q);
+    int n_splits = a.n_splits;
+    if (!cut && row >= n_q * Hq) return;
+    int tok = row / Hq;
+    const int head = row - tok * Hq;
+    size_t first = (size_t)row, stride = (size_t)n_q * Hq;      // the row's first partial, and rows from one to the next
+    if (cut) {
+        tok += c.tok_first;
+        const int unit = tok / c.unit_tokens, g = unit / c.chunk;
+        n_splits = g + 1;
+        const int slot = c.chunk * g * (g + 1) / 2 + (unit - g * c.chunk) * (g + 1);
+        stride = (size_t)c.unit_tokens * Hq;
+        first = (size_t)slot * stride + (size_t)(tok - unit * c.unit_tokens) * Hq + head;
+    }
+    const float* const lse_src = DAF_CS(part_lse) + first;
+    const float4* const src = reinterpret_cast<const float4*>(DAF_CS(part_o) + first * kD) + lane;
     float4 v[kMost];
     float mx, wsum = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -905,7 +940,8 @@ attn_combine_kernel(const CombineArgs a) {
 #pragma unroll
     for (int u = 0; u < kMost; ++u)
         v[u] = u < n_splits ? __ldcs(src + (size_t)u * stride * (kD / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const long long drow = a.dst_rows ? (long long)a.dst_rows[tok] : (long long)tok;
+    const int32_t* const dst_rows = DAF_CS(dst_rows);
+    const long long drow = dst_rows ? (long long)dst_rows[tok] : (long long)tok;
     mx = my_lse;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
@@ -920,9 +956,11 @@ attn_combine_kernel(const CombineArgs a) {
     uint2 w2;
     w2.x = pack_bf16(acc.x * inv, acc.y * inv);
     w2.y = pack_bf16(acc.z * inv, acc.w * inv);
-    reinterpret_cast<uint2*>(a.out + drow * a.out_row_stride + (long long)head * kD)[lane] = w2;
-    if (a.lse != nullptr && lane == 0) a.lse[(size_t)head * n_q + tok] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
+    reinterpret_cast<uint2*>(DAF_CS(out) + drow * DAF_CS(out_row_stride) + (long long)head * kD)[lane] = w2;
+    float* const lse = DAF_CS(lse);
+    if (lse != nullptr && lane == 0) lse[(size_t)head * n_q + tok] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
     DAF_KT_END(2);
+#undef DAF_CS
 }
 
 // ----------------------------------------------------------------- host side
@@ -1104,18 +1142,27 @@ size_t attn_partial_bytes(int n_q, int Hq, int n_splits) {
     return o + l;
 }
 
-// Steps 2 and 3 of one layer as one list of work items.  One thing is free: into how many KV ranges the question rows
-// are cut.  Finer ranges balance the 296 CTA slots better but cost a fixed time per item, partial-result traffic and a
-// longer merge, and the optimum jumps around with the tile counts.  So the choice is made by replaying the hardware's
-// dispatch (items in grid order onto the slot that frees first) for every distinct number of ranges with a
-// three-constant cost model and keeping the cheapest; the result is cached per problem shape.
+// Number of (unit, range) slots of units [0, n_units) when groups of `chunk` units are cut into 1, 2, 3, ... ranges.
+static int slots_before(int n_units, int chunk) {
+    const int g = n_units / chunk;
+    return chunk * g * (g + 1) / 2 + (n_units - g * chunk) * (g + 1);
+}
+
+// Steps 2 and 3 of one layer as one list of work items.  Two things are free: into how many KV ranges the question rows
+// are cut, and into how many the long causal chains of the important tokens (`chunk`).  Finer ranges balance the 296 CTA
+// slots better but cost a fixed time per item, partial-result traffic and a longer merge, and the optimum jumps around with
+// the tile counts.  So the choice is made by replaying the hardware's dispatch (items in grid order onto the slot that frees
+// first) for every distinct number of ranges with a three-constant cost model and keeping the cheapest; the result is cached
+// per problem shape.
 namespace {
 constexpr float kCostItemUs = 7.0f;        // set-up, first logits and row epilogue of an item (5-6 us alone; fitted)
 constexpr float kCostSubStepUs = 1.05f;    // 64 keys through one tile with two CTAs per SM (measured 0.95-1.1 us)
 constexpr float kCostMergeUs = 2.0f;       // merge launch
 constexpr float kCostMergeUsPerMB = 0.15f; // plus re-reading the partial rows of the question ranges (fitted together with the item cost)
+constexpr float kCutGain = 0.78f;          // causal chains are cut where the prediction falls to this share (see plan_joint)
+constexpr float kCostMergeUsPerMBCut = 0.45f;  // partial rows of cut causal chains (measured: 7.0 us for 14.8 MB, 13.3 for 25, 42.6 for 96)
 
-int g_force_splits_q = 0;   // tuning builds can pin the choice
+int g_force_chunk = 0, g_force_splits_q = 0;   // tuning builds can pin the choice
 float g_last_predicted_us = 0.f;
 
 struct JointShape { int k, L_q, L_d, Hq, G; };
@@ -1127,8 +1174,13 @@ bool operator<(const JointShape& a, const JointShape& b) {
     return a.G < b.G;
 }
 
-// Fills the fields of `jp` that follow from n_splits_q.
-void set_choice(JointPlan& jp, int n_splits_q, int L_q, int L_d, int Hq) {
+// Fills the fields of `jp` that follow from chunk (n_tb_i or more: whole chains) and n_splits_q.
+void set_choice(JointPlan& jp, int chunk, int n_splits_q, int L_q, int L_d, int Hq) {
+    jp.chunk = chunk < jp.n_tb_i ? chunk : 0;
+    jp.n_slots = jp.chunk > 0 ? slots_before(jp.n_tb_i, jp.chunk) : jp.n_tb_i;
+    jp.items_i = jp.head_blocks_i * jp.n_slots;
+    const size_t rows = jp.chunk > 0 ? (size_t)jp.n_slots * jp.Tt_i * Hq : 0;
+    jp.part_bytes_i = rows * kD * sizeof(float) + (rows * sizeof(float) + 255) / 256 * 256;
     const int steps_q = (L_d + L_q + kSubN - 1) / kSubN;
     if (n_splits_q < 1) n_splits_q = 1;
     jp.steps_per_split_q = (steps_q + n_splits_q - 1) / n_splits_q;
@@ -1139,13 +1191,14 @@ void set_choice(JointPlan& jp, int n_splits_q, int L_q, int L_d, int Hq) {
 }
 
 // Predicted time of the attention launch + merge for a filled plan, in microseconds.
-float predict_us(const JointPlan& jp, int k, int L_q, int L_d) {
+float predict_us(const JointPlan& jp, int k, int L_q, int L_d, int Hq, float* busy_us = nullptr) {
     const int slots = num_sms() * 2;
     std::priority_queue<float, std::vector<float>, std::greater<float>> free_at;
     for (int i = 0; i < slots; ++i) free_at.push(0.f);
-    float makespan = 0.f;
+    float makespan = 0.f, busy = 0.f;
     auto run = [&](int count, int substeps) {
         const float cost = kCostItemUs + kCostSubStepUs * (float)substeps;
+        busy += cost * (float)count / (float)slots;
         for (int i = 0; i < count; ++i) {
             const float t = free_at.top() + cost;
             free_at.pop();
@@ -1163,9 +1216,18 @@ float predict_us(const JointPlan& jp, int k, int L_q, int L_d) {
             if (end > begin) run(jp.head_blocks_q, (end - begin + kSubN - 1) / kSubN);
         }
     // important-token items: units from the last one down, head blocks together
-    for (int u = jp.n_tb_i - 1; u >= 0; --u)
-        run(jp.head_blocks_i, (((u + 1) * jp.Tt_i < k ? (u + 1) * jp.Tt_i : k) + kSubN - 1) / kSubN);
-    return makespan + (jp.n_splits_q > 1 ? kCostMergeUs + kCostMergeUsPerMB * (float)jp.part_bytes_q / 1e6f : 0.f);
+    size_t cut_rows = 0;
+    for (int u = jp.n_tb_i - 1; u >= 0; --u) {
+        const int steps = (((u + 1) * jp.Tt_i < k ? (u + 1) * jp.Tt_i : k) + kSubN - 1) / kSubN;
+        const int ranges = jp.chunk > 0 ? u / jp.chunk + 1 : 1;
+        for (int j = ranges - 1; j >= 0; --j) run(jp.head_blocks_i, (j + 1) * steps / ranges - j * steps / ranges);
+        if (ranges > 1) cut_rows += (size_t)ranges * jp.Tt_i * Hq;
+    }
+    if (busy_us != nullptr) *busy_us = busy;
+    float us = makespan;
+    if (jp.n_splits_q > 1 || jp.chunk > 0)
+        us += kCostMergeUs + kCostMergeUsPerMB * (float)jp.part_bytes_q / 1e6f + kCostMergeUsPerMBCut * (float)(cut_rows * 516) / 1e6f;
+    return us;
 }
 }  // namespace
 
@@ -1173,7 +1235,7 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     static std::mutex mu;
     static std::map<JointShape, JointPlan> cache;
     const JointShape shape{k, L_q, L_d, Hq, G};
-    const bool forced = g_force_splits_q > 0;
+    const bool forced = g_force_chunk > 0 || g_force_splits_q > 0;
     // a layer loop asks for the same shape over and over: each thread keeps its last answer (no lock)
     static thread_local bool have_last = false;
     static thread_local JointShape last_shape;
@@ -1189,27 +1251,43 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     jp.Tt_i = kBlockM / jp.Gp_i;
     jp.n_tb_i = (k + jp.Tt_i - 1) / jp.Tt_i;
     jp.head_blocks_i = Hq / jp.Gp_i;
-    jp.items_i = jp.head_blocks_i * jp.n_tb_i;
     jp.Gp_q = G > 128 ? 1 : G;
     jp.Tt_q = kBlockM / jp.Gp_q;
     jp.n_tb_q = (L_q + jp.Tt_q - 1) / jp.Tt_q;
     jp.head_blocks_q = Hq / jp.Gp_q;
     const int steps_q = (L_d + L_q + kSubN - 1) / kSubN;
     if (forced) {
-        set_choice(jp, g_force_splits_q, L_q, L_d, Hq);
-        g_last_predicted_us = predict_us(jp, k, L_q, L_d);
+        set_choice(jp, g_force_chunk > 0 ? g_force_chunk : jp.n_tb_i, g_force_splits_q, L_q, L_d, Hq);
+        g_last_predicted_us = predict_us(jp, k, L_q, L_d, Hq);
         return jp;
     }
+    // Candidates: the causal chains whole, or cut so that the longest has 2 to 6 ranges; every distinct number of question
+    // ranges.  Cuts are taken only on a large predicted gain, since the model knows no difference between a CTA alone on its
+    // SM and one beside another: measured over 320 shapes, calls predicted to fall to 0.75 and below all got faster (3709
+    // important tokens of 4 heads on 4: 45.6 -> 28.5 us, 1008: 18.1 -> 12.7), half of those around 0.8 and most above got
+    // slower (28/4, 475 tokens, 0.94: 13.8 -> 18.1).
     JointPlan best = jp;
-    float best_us = -1.f;
-    int last_steps = -1;
-    for (int n = 1; n <= kMaxSplits && n <= steps_q; ++n) {
-        JointPlan cand = jp;
-        set_choice(cand, n, L_q, L_d, Hq);
-        if (cand.steps_per_split_q == last_steps) continue;
-        last_steps = cand.steps_per_split_q;
-        const float us = predict_us(cand, k, L_q, L_d);
-        if (best_us < 0.f || us < best_us) { best_us = us; best = cand; }
+    float best_us = -1.f, whole_us = 0.f, whole_busy = 0.f;
+    int last_chunk = 0;
+    for (int m = 1; m <= kMaxChainRanges; ++m) {
+        const int chunk = (jp.n_tb_i + m - 1) / m;
+        if (chunk == last_chunk) continue;              // the same cut as the candidate before
+        if (m > 1 && (chunk * jp.Tt_i < kSubN || whole_busy > kCutGain * whole_us)) break;   // empty ranges, or nothing to balance
+        last_chunk = chunk;
+        int last_steps = -1;
+        for (int n = 1; n <= kMaxSplits && n <= steps_q; ++n) {
+            JointPlan cand = jp;
+            set_choice(cand, chunk, n, L_q, L_d, Hq);
+            if (cand.steps_per_split_q == last_steps) continue;
+            last_steps = cand.steps_per_split_q;
+            if (cand.part_bytes_i > ((size_t)256 << 20)) continue;   // partials of a large problem: not worth their memory
+            float busy;
+            const float us = predict_us(cand, k, L_q, L_d, Hq, &busy);
+            if (best_us < 0.f || us < (m == 1 || best.chunk > 0 ? best_us : kCutGain * whole_us)) {
+                best_us = us; best = cand;
+                if (m == 1) { whole_us = us; whole_busy = busy; }
+            }
+        }
     }
     g_last_predicted_us = best_us;
     std::lock_guard<std::mutex> lock(mu);
@@ -1219,11 +1297,11 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
 }
 
 #if defined(DAF_TRACE) || defined(DAF_TUNE)     // tuning builds: pin the planner's choice, read its prediction
-extern "C" void daf_dbg_joint_force(int n_splits_q) { g_force_splits_q = n_splits_q; }
+extern "C" void daf_dbg_joint_force(int chunk, int n_splits_q) { g_force_chunk = chunk; g_force_splits_q = n_splits_q; }
 extern "C" float daf_dbg_joint_predicted_us(void) { return g_last_predicted_us; }
 extern "C" void daf_dbg_joint_plan(int k, int L_q, int L_d, int Hq, int G, int* out) {
     const JointPlan jp = plan_joint(k, L_q, L_d, Hq, G);
-    out[0] = jp.Gp_i; out[1] = jp.n_tb_i; out[2] = jp.n_splits_q; out[3] = jp.items_i + jp.items_q;
+    out[0] = jp.Gp_i; out[1] = jp.n_tb_i; out[2] = jp.n_splits_q; out[3] = jp.items_i + jp.items_q; out[4] = jp.chunk;
 }
 #endif
 
@@ -1241,17 +1319,31 @@ static void fill_problem(SegArgs* s, int n_q, int n_kv, int Hq, int G, int Gp, i
     s->lse = lse;
 }
 
-static int launch_combine(const SegArgs& s, cudaStream_t stream) {
-    if (s.n_splits <= 1) return DAF_OK;
-    const CombineArgs c{s.part_o, s.part_lse, s.n_q, s.Hq, s.n_splits, s.out, s.out_row_stride, s.dst_rows, s.lse};
-    const dim3 grid((unsigned)((s.n_q * s.Hq + 7) / 8));
-    auto* kernel = s.n_splits <= 4    ? attn_combine_kernel<4>
-                   : s.n_splits <= 8  ? attn_combine_kernel<8>
-                   : s.n_splits <= 12 ? attn_combine_kernel<12>
-                   : s.n_splits <= 16 ? attn_combine_kernel<16>
-                   : s.n_splits <= 24 ? attn_combine_kernel<24>
-                                      : attn_combine_kernel<kMaxSplits>;
-    const cudaError_t e = launch_kernel(kernel, grid, dim3(256), 0, stream, c);
+static CombineArgs combine_args(const SegArgs& s) {
+    CombineArgs c{};
+    c.part_o = s.part_o; c.part_lse = s.part_lse;
+    c.n_q = s.n_q; c.Hq = s.Hq; c.n_splits = s.n_splits;
+    c.chunk = s.chunk; c.unit_tokens = s.Tt; c.tok_first = s.chunk * s.Tt;
+    c.out = s.out; c.out_row_stride = s.out_row_stride; c.dst_rows = s.dst_rows; c.lse = s.lse;
+    return c;
+}
+
+// Merges the rows of s (ranges of all its rows' keys) and of cut (cut causal chains), either of which may have nothing to merge.
+static int launch_combine(const SegArgs* s, const SegArgs* cut, cudaStream_t stream) {
+    CombineArgs a{}, c{};
+    if (s != nullptr && s->n_splits > 1) a = combine_args(*s);
+    if (cut != nullptr && cut->chunk > 0) c = combine_args(*cut);
+    const int rows = a.n_q * a.Hq + (c.n_q - c.tok_first) * c.Hq;
+    if (rows <= 0) return DAF_OK;
+    const int most = c.n_q > 0 && kMaxChainRanges > a.n_splits ? kMaxChainRanges : a.n_splits;
+    auto* kernel = c.n_q > 0 ? (most <= 8 ? attn_combine_kernel<8, true> : most <= 16 ? attn_combine_kernel<16, true> : attn_combine_kernel<kMaxSplits, true>)
+                   : most <= 4  ? attn_combine_kernel<4, false>
+                   : most <= 8  ? attn_combine_kernel<8, false>
+                   : most <= 12 ? attn_combine_kernel<12, false>
+                   : most <= 16 ? attn_combine_kernel<16, false>
+                   : most <= 24 ? attn_combine_kernel<24, false>
+                                : attn_combine_kernel<kMaxSplits, false>;
+    const cudaError_t e = launch_kernel(kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, stream, a, c);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     return check_launch();
@@ -1298,7 +1390,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
     if (int rc = check_launch()) return rc;
-    return launch_combine(s, stream);
+    return launch_combine(&s, nullptr, stream);
 }
 
 // Self-test of the bounded wait every kernel here relies on: two warps wait on a barrier that nothing ever
@@ -1331,7 +1423,7 @@ constexpr int kMaxTokenCopies = 32;
 static bool copies_per_token(const JointPlan& jp, int k) { return (jp.Tt_i < k ? jp.Tt_i : k) <= kMaxTokenCopies; }
 bool step2_packs_q(int k, int L_q, int L_d, int Hq, int G) { return copies_per_token(plan_joint(k, L_q, L_d, Hq, G), k); }
 
-size_t joint_partial_bytes(const JointPlan& jp) { return jp.part_bytes_q; }
+size_t joint_partial_bytes(const JointPlan& jp) { return jp.part_bytes_q + jp.part_bytes_i; }
 
 int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_place, bool q_early, const int32_t* idx, const void* k_imp, const void* v_imp,
                            const void* k_fresh, const void* v_fresh,
@@ -1388,7 +1480,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
     sq.n_items = jp.items_q;
     sq.part_o = reinterpret_cast<float*>(sc);
     sq.part_lse = reinterpret_cast<float*>(sc + (size_t)jp.n_splits_q * L_q * Hq * kD * sizeof(float));
-    // important tokens: causal attention over the condensed sequence, keys never cut
+    // important tokens: causal attention over the condensed sequence
     SegArgs& si = a.seg[0];
     fill_problem(&si, k, k, Hq, G, jp.Gp_i, 0, nullptr, scale, out_imp, out_row_stride_bytes, dst_rows_imp, nullptr);
     if (gather_q) {
@@ -1408,12 +1500,15 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
     si.out_tiled = imp_tiled ? 1 : 0;
     si.n_units = jp.n_tb_i;
     si.n_splits = 1; si.steps_per_split = (k + kSubN - 1) / kSubN;
+    si.chunk = jp.chunk; si.n_slots = jp.n_slots;
     si.n_items = jp.items_i;
+    si.part_o = reinterpret_cast<float*>(sc + jp.part_bytes_q);
+    si.part_lse = si.part_o + (size_t)jp.n_slots * jp.Tt_i * Hq * kD;
     a.status = status;
 
     const int items = jp.items_q + jp.items_i;
     if (launches & 1) {
-        auto* kernel = gather_kv ? attn_fwd_kernel<true, true> : by_warps ? attn_fwd_kernel<false, true> : attn_fwd_kernel<false, false>;
+        auto* kernel = gather_kv ? attn_fwd_kernel<true, true> : by_warps || jp.chunk > 0 ? attn_fwd_kernel<false, true> : attn_fwd_kernel<false, false>;
         const cudaError_t e = launch_kernel(kernel, dim3((unsigned)items), dim3(gather_kv ? kAttnThreadsGather : kAttnThreads),
                                             kAttnSmemBytes, stream, tq0, tk0, tv0, tq1, tk1, tv1, to0, to1, tqp, a);
         count_launch();
@@ -1421,7 +1516,7 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
         if (int rc = check_launch()) return rc;
     }
     if (!(launches & 2)) return DAF_OK;
-    return launch_combine(sq, stream);
+    return launch_combine(&sq, &si, stream);
 }
 
 }  // namespace daf

@@ -68,9 +68,9 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
                      cudaStream_t stream, const int32_t* q_pos = nullptr, const AttnPlan* plan = nullptr);   // plan: null = planned here
 // Steps 2 and 3 of a layer from one list of work items (one attention launch and one merge launch).
 struct JointPlan {
-    int Gp_i, Tt_i, n_tb_i, head_blocks_i, items_i;                       // important-token stage
+    int Gp_i, Tt_i, n_tb_i, head_blocks_i, chunk, n_slots, items_i;       // important-token stage (chunk > 0: causal chains cut)
     int Gp_q, Tt_q, n_tb_q, head_blocks_q, n_splits_q, steps_per_split_q, items_q;   // question stage
-    size_t part_bytes_q;        // partial results of the question ranges
+    size_t part_bytes_q, part_bytes_i;        // partial results of each stage
 };
 JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G);
 size_t joint_partial_bytes(const JointPlan& jp);

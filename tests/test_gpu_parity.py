@@ -866,6 +866,34 @@ def test_layer_leaves_the_packed_q_rows_it_read_in_place(L_d, L_q, r, Hq, Hkv, g
     assert torch.equal(qp[:k], g["q_fresh"][idx_out.long()]) and torch.all(qp[k] == 3.0)
 
 
+@pytest.mark.parametrize("buffers", ["all", "no q", "no q, k, v"])
+@pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv,fuse_mode", [(3513, 9, 0.6, 4, 4, 0), (1200, 2, 1.0, 4, 4, 1), (1683, 3, 0.6, 7, 1, 0),
+                                                       (1003, 5, 1.0, 8, 8, 0), (4000, 2, 0.3, 12, 4, 1), (882, 1, 1.0, 8, 2, 0)])
+def test_layer_whose_causal_chains_are_cut(L_d, L_q, r, Hq, Hkv, fuse_mode, buffers):
+    """Few heads and long chains, whose keys are walked in ranges by several CTAs: tiles of one to seven heads, partial last tiles, Q
+    and K/V rows packed and in place, against the oracle.  (The plan shows in the workspace: the partial rows of one question
+    token are small beside those of the important tokens.)"""
+    p, p0 = api.make_params(L_d, L_q, r, Hq, Hkv, fuse_mode=fuse_mode), api.make_params(L_d, L_q, 0.0, Hq, Hkv)
+    k = api.daf_num_important(L_d, r)
+    assert api.daf_workspace_bytes(p) - api.daf_workspace_bytes(p0) > k * Hq * 516, "not cut"
+    w = W.Workload("t", 46, Hq, Hkv, 128, 1, L_d, L_d, L_q, r, "lognormal", 1)
+    L = W.make_layer(w, 0)
+    g = {n: t.cuda() for n, t in L.items() if t is not None}
+    kv = [torch.cat([g[n], torch.zeros(L_q, Hkv, 128, dtype=torch.bfloat16, device="cuda")]) for n in ("k_cached", "v_cached")]
+    qp = torch.full((k + 1, Hq, 128), 3.0, dtype=torch.bfloat16, device="cuda") if buffers == "all" else None
+    kp, vp = (torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda") if "k" not in buffers else None for _ in range(2))
+    idx_out = torch.full((k,), -1, dtype=torch.int32, device="cuda")
+    hidden = torch.full((w.N if fuse_mode == 1 else k + L_q, Hq, 128), -9.0, dtype=torch.bfloat16, device="cuda")
+    ws = api.alloc_workspace(p)
+    _ok(api.daf_layer(p, g["scores"], 1, None, g["q_fresh"], g["k_fresh"], g["v_fresh"], kv[0], kv[1], idx_out, qp, kp, vp, hidden,
+                      None, ws), ws, "daf_layer")
+    ref = _oracle_layer(w, L, fuse_mode)
+    assert np.array_equal(idx_out.cpu().numpy(), ref["idx"])
+    if qp is not None:
+        assert torch.equal(qp[:k], g["q_fresh"][idx_out.long()]) and torch.all(qp[k] == 3.0)
+    _assert_close(hidden, ref["hidden"], "cut chains")
+
+
 @pytest.mark.parametrize("given", [False, True])
 @pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv,fuse_mode,shares", [
     (3000, 40, 0.3, 14, 2, 0, "q_fresh"), (3000, 40, 0.3, 14, 2, 0, "q_fresh+512"), (3000, 40, 0.3, 14, 2, 0, "q_pack"),
