@@ -209,8 +209,9 @@ int daf_imp_qd_attn_launches(const daf_params* p, const void* q_pack, const void
  * cudaMalloc/cudaFree and calls no allocating routine.
  *
  *   - Arguments as in daf_qd_attn, without workspace.
- *   - Problems whose scratch need exceeds daf_qd_attn_static_max_bytes() are
- *     rejected with DAF_ERR_WORKSPACE before anything is launched.
+ *   - Problems whose scratch need, with one range of keys per CTA slot (two per
+ *     SM), exceeds daf_qd_attn_static_max_bytes() are rejected with
+ *     DAF_ERR_WORKSPACE before anything is launched.
  *   - The first call on each device looks up the array's device address (with
  *     that device current); make that first call outside any stream capture.
  *   - All calls on one device share the array, and it keeps the previous call's

@@ -72,6 +72,7 @@ struct SegArgs {
     float* lse;         // [Hq, n_q] or null
     float* part_o;      // partial results, fp32, normalised per range: [n_splits][n_q][Hq][128], or [n_slots][Tt][Hq][128]
     float* part_lse;    // the same without the last dimension
+    int lse_stride;     // kExtra: rows of lse are this far apart (the problem is some of the tokens of a larger one)
 };
 
 // A launch runs the items of seg[1] first (none in a launch of one problem), then those of seg[0], heaviest units first.  The
@@ -236,6 +237,7 @@ __device__ __forceinline__ void decode_work(const AttnArgs& args, CtaWork& a) {
 // Final step of a tile: the warp's 32 rows of O (fp32 in tensor memory at o_addr, this thread's row
 // unnormalised with running maximum m and sum l) leave as bf16 output rows, or -- for an item that
 // covers only part of the keys -- as fp32 partial rows with their log-sum-exp.
+template <bool kExtra>
 __device__ __forceinline__ void write_rows(const AttnArgs& args, const CtaWork& a, int t0, bool has_keys, bool row_valid,
                                            bool row_valid_tile, int tok, int head, int h0, unsigned char* q_tile,
                                            const CUtensorMap* tmap_o, uint64_t* rows_parked, volatile int* abort_flag,
@@ -267,7 +269,7 @@ __device__ __forceinline__ void write_rows(const AttnArgs& args, const CtaWork& 
         // Rows in token order: the tile is parked in the layout of a tiled copy (two 64-column halves of
         // 128-byte rows, 16-byte chunks XOR-ed with the row number mod 8 -- the layout the Q tile came in)
         // and leaves by two bulk tensor stores, which clip the rows past the end of the output.
-        if (row_valid && e.lse != nullptr) e.lse[(size_t)head * e.n_q + tok] = lse_val;
+        if (row_valid && e.lse != nullptr) e.lse[(size_t)head * (kExtra ? DAF_SEG(lse_stride) : e.n_q) + tok] = lse_val;
         const int r = quad * 32 + lane;
         if (has_keys) {
 #pragma unroll
@@ -303,7 +305,7 @@ __device__ __forceinline__ void write_rows(const AttnArgs& args, const CtaWork& 
             }
         }
     } else if (a.item_splits == 1) {
-        if (row_valid && e.lse != nullptr) e.lse[(size_t)head * e.n_q + tok] = lse_val;
+        if (row_valid && e.lse != nullptr) e.lse[(size_t)head * (kExtra ? DAF_SEG(lse_stride) : e.n_q) + tok] = lse_val;
         if (has_keys) {
 #pragma unroll
             for (int cchunk = 0; cchunk < 4; ++cchunk) {
@@ -422,7 +424,7 @@ struct AttnSmem {
 constexpr size_t kAttnSmemBytes = 1024 + 3 * (size_t)kTileBytes + sizeof(AttnSmem);
 
 // kGatherKV: the launch has a problem whose K/V rows three warps fetch in place through an index; kExtra: one whose Q rows the
-// softmax warps fetch, or whose causal chains are cut.  Forms of their own, so that the plain form carries none of that code.
+// softmax warps fetch, whose causal chains are cut or whose log-sum-exps lie in a wider tensor.  Forms of their own, so that the plain form carries none of that code.
 template <bool kGatherKV, bool kExtra>
 __global__ void __launch_bounds__(kGatherKV ? kAttnThreadsGather : kAttnThreads, 2)
 attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_constant__ CUtensorMap tmap_k0,
@@ -848,7 +850,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         }
         if (ok) {
             tc_fence_after();
-            write_rows(args, a, t0, n_t > 0, row_valid, row_valid_tile, tok, head, h0, q_smem, seg_id ? &tmap_o1 : &tmap_o0,
+            write_rows<kExtra>(args, a, t0, n_t > 0, row_valid, row_valid_tile, tok, head, h0, q_smem, seg_id ? &tmap_o1 : &tmap_o0,
                        &sm->rows_parked, abort_flag, o_addr, quad, lane, m, l);
         }
 #ifdef DAF_TRACE
@@ -896,15 +898,16 @@ struct CombineArgs {
     int n_q, Hq;
     int n_splits;        // partials per row, n_q * Hq rows apart
     int chunk, unit_tokens, tok_first;   // chunk > 0: cut causal chains, tokens tok_first on (the others' rows are final)
-    __nv_bfloat16* out; long long out_row_stride; const int32_t* dst_rows; float* lse;
+    __nv_bfloat16* out; long long out_row_stride; const int32_t* dst_rows; float* lse; int lse_stride;
 };
 
 // kMost: the largest number of partials a launch of this form merges.  Bound by latency: all of a row's partials and their
 // log-sum-exps are requested at once (a second round is a second trip to L2: as eight and then four by four, 24 tokens of 28
 // heads over 14k keys, 22 ranges, took 22.4 us with their attention, at once 19.8; 28 layers of 6k, 7 ranges, 747 against 726).  Two CTAs per SM are asked for so that
 // the compiler has the registers to keep them all under way.
-// kCut: the launch also merges the rows of a problem whose causal chains are cut (c), ahead of the others.
-template <int kMost, bool kCut>
+// kExtra: the launch may also merge the rows of a problem whose causal chains are cut (c), ahead of the others, and the rows of
+// lse may be further apart than n_q.  A form of its own, as for the attention kernel.
+template <int kMost, bool kExtra>
 __global__ void __launch_bounds__(256, 2)
 attn_combine_kernel(const CombineArgs a, const CombineArgs c) {
     DAF_KT_BEGIN(2);
@@ -912,10 +915,10 @@ attn_combine_kernel(const CombineArgs a, const CombineArgs c) {
     DAF_KT_BEGIN(3);
     int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    const int cut_rows = kCut ? (c.n_q - c.tok_first) * c.Hq : 0;
-    const bool cut = kCut && row < cut_rows;
-    if (kCut && !cut) row -= cut_rows;
-#define DAF_CS(field) (kCut && cut ? c.field : a.field)
+    const int cut_rows = kExtra ? (c.n_q - c.tok_first) * c.Hq : 0;
+    const bool cut = kExtra && row < cut_rows;
+    if (kExtra && !cut) row -= cut_rows;
+#define DAF_CS(field) (kExtra && cut ? c.field : a.field)
     const int Hq = DAF_CS(Hq), n_q = DAF_CS(n_q);
     int n_splits = a.n_splits;
     if (!cut && row >= n_q * Hq) return;
@@ -958,7 +961,7 @@ attn_combine_kernel(const CombineArgs a, const CombineArgs c) {
     w2.y = pack_bf16(acc.z * inv, acc.w * inv);
     reinterpret_cast<uint2*>(DAF_CS(out) + drow * DAF_CS(out_row_stride) + (long long)head * kD)[lane] = w2;
     float* const lse = DAF_CS(lse);
-    if (lse != nullptr && lane == 0) lse[(size_t)head * n_q + tok] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
+    if (lse != nullptr && lane == 0) lse[(size_t)head * (kExtra ? DAF_CS(lse_stride) : n_q) + tok] = wsum > 0.f ? mx + logf(wsum) : -INFINITY;
     DAF_KT_END(2);
 #undef DAF_CS
 }
@@ -1316,7 +1319,7 @@ static void fill_problem(SegArgs* s, int n_q, int n_kv, int Hq, int G, int Gp, i
     s->out = reinterpret_cast<__nv_bfloat16*>(out);
     s->out_row_stride = out_row_stride_bytes / 2;
     s->dst_rows = dst_rows;
-    s->lse = lse;
+    s->lse = lse; s->lse_stride = n_q;
 }
 
 static CombineArgs combine_args(const SegArgs& s) {
@@ -1324,7 +1327,7 @@ static CombineArgs combine_args(const SegArgs& s) {
     c.part_o = s.part_o; c.part_lse = s.part_lse;
     c.n_q = s.n_q; c.Hq = s.Hq; c.n_splits = s.n_splits;
     c.chunk = s.chunk; c.unit_tokens = s.Tt; c.tok_first = s.chunk * s.Tt;
-    c.out = s.out; c.out_row_stride = s.out_row_stride; c.dst_rows = s.dst_rows; c.lse = s.lse;
+    c.out = s.out; c.out_row_stride = s.out_row_stride; c.dst_rows = s.dst_rows; c.lse = s.lse; c.lse_stride = s.lse_stride;
     return c;
 }
 
@@ -1336,7 +1339,7 @@ static int launch_combine(const SegArgs* s, const SegArgs* cut, cudaStream_t str
     const int rows = a.n_q * a.Hq + (c.n_q - c.tok_first) * c.Hq;
     if (rows <= 0) return DAF_OK;
     const int most = c.n_q > 0 && kMaxChainRanges > a.n_splits ? kMaxChainRanges : a.n_splits;
-    auto* kernel = c.n_q > 0 ? (most <= 8 ? attn_combine_kernel<8, true> : most <= 16 ? attn_combine_kernel<16, true> : attn_combine_kernel<kMaxSplits, true>)
+    auto* kernel = c.n_q > 0 || a.lse_stride != a.n_q ? (most <= 8 ? attn_combine_kernel<8, true> : most <= 16 ? attn_combine_kernel<16, true> : attn_combine_kernel<kMaxSplits, true>)
                    : most <= 4  ? attn_combine_kernel<4, false>
                    : most <= 8  ? attn_combine_kernel<8, false>
                    : most <= 12 ? attn_combine_kernel<12, false>
@@ -1352,7 +1355,7 @@ static int launch_combine(const SegArgs* s, const SegArgs* cut, cudaStream_t str
 int launch_attention(const void* q, const void* k, const void* v, int n_q, int n_kv, int Hq, int Hkv, int causal_off,
                      float scale, bool pack_group, bool allow_split, void* out, long long out_row_stride_bytes,
                      const int32_t* dst_rows, float* lse, DeviceStatus* status, void* scratch, size_t scratch_bytes,
-                     cudaStream_t stream, const int32_t* q_pos, const AttnPlan* plan) {
+                     cudaStream_t stream, const int32_t* q_pos, const AttnPlan* plan, int lse_stride) {
     if (n_q <= 0) return DAF_OK;
     const int G = Hq / Hkv;
     // a causal problem over its own keys chooses how many heads share a tile; the question rows always pack the group
@@ -1376,6 +1379,7 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
     memset(&a, 0, sizeof(a));
     SegArgs& s = a.seg[0];
     fill_problem(&s, n_q, n_kv, Hq, G, pl.Gp, causal_off, q_pos, scale, out, out_row_stride_bytes, dst_rows, lse);
+    if (lse_stride > 0) s.lse_stride = lse_stride;
     s.out_tiled = out_tiled ? 1 : 0;
     s.n_units = pl.n_tb;
     s.n_splits = pl.n_splits; s.steps_per_split = pl.steps_per_split;
@@ -1385,7 +1389,8 @@ int launch_attention(const void* q, const void* k, const void* v, int n_q, int n
                                                             (size_t)pl.n_splits * n_q * Hq * kD * sizeof(float))
                                  : nullptr;
     a.status = status;
-    cudaError_t e = launch_kernel(attn_fwd_kernel<false, false>, dim3((unsigned)s.n_items), dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
+    cudaError_t e = launch_kernel(s.lse_stride != n_q ? attn_fwd_kernel<false, true> : attn_fwd_kernel<false, false>, dim3((unsigned)s.n_items),
+                                  dim3(kAttnThreads), kAttnSmemBytes, stream, tq, tk, tv, tq, tk, tv,
                                   to, to, tq, a);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
@@ -1576,8 +1581,7 @@ extern "C" int daf_qd_attn_static(const daf_params* p, const void* q_question, c
     if (!aligned16(q_question) || !aligned16(kv_k) || !aligned16(kv_v) || !aligned16(out) ||
         out_row_stride_bytes % 16 != 0) return DAF_ERR_ALIGNMENT;
     if (out_row_stride_bytes < (int64_t)rp.Hq * 256) return DAF_ERR_INVALID_ARG;
-    // The problems served are those whose scratch fits with as many ranges of 128 keys as there are CTA slots for; within
-    // those the planned number of ranges is used, or as many as fit.
+    // The problems served are those whose scratch fits with as many ranges of 128 keys as there are CTA slots for.
     AttnPlan pl = plan_attention(rp.L_q, rp.N, rp.Hq, rp.G, rp.L_d, true, true);
     const int tiles = (rp.N + 127) / 128, ctas = pl.n_tb * pl.head_blocks;
     int want = 2 * num_sms() / ctas;
@@ -1585,19 +1589,30 @@ extern "C" int daf_qd_attn_static(const daf_params* p, const void* q_question, c
     if (want > tiles) want = tiles;
     const int per = want > 1 ? (tiles + want - 1) / want : tiles;
     if (kStatusBytes + attn_partial_bytes(rp.L_q, rp.Hq, (tiles + per - 1) / per) > kStaticScratchBytes) return DAF_ERR_WORKSPACE;
-    while (pl.n_splits > 1 && kStatusBytes + attn_partial_bytes(rp.L_q, rp.Hq, pl.n_splits) > kStaticScratchBytes) {
-        ++pl.steps_per_split;
-        pl.n_splits = ((rp.N + kSubN - 1) / kSubN + pl.steps_per_split - 1) / pl.steps_per_split;
-    }
     void* base = nullptr;
     if (int rc = static_scratch_address(&base)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     // the array keeps whatever the previous call left: the status word has to start at zero
     cudaError_t e = cudaMemsetAsync(base, 0, kStatusBytes, st);
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
-    return launch_attention(q_question, kv_k, kv_v, rp.L_q, rp.N, rp.Hq, rp.Hkv, rp.L_d, rp.scale, true, true, out,
-                            out_row_stride_bytes, dst_rows, lse, reinterpret_cast<DeviceStatus*>(base),
-                            reinterpret_cast<char*>(base) + kStatusBytes, kStaticScratchBytes - kStatusBytes, st, nullptr, &pl);
+    // The keys are cut as daf_qd_attn cuts them, so that the results are the same.  Where the partial rows of all tokens do not
+    // fit, the tokens are taken in groups one behind the other: a row does not depend on which rows share its tile.
+    const size_t scratch = kStaticScratchBytes - kStatusBytes;
+    int group = rp.L_q;
+    if (attn_partial_bytes(rp.L_q, rp.Hq, pl.n_splits) > scratch)
+        group = (int)((scratch - 256) / ((size_t)pl.n_splits * rp.Hq * (kD + 1) * sizeof(float)));
+    for (int t0 = 0; t0 < rp.L_q; t0 += group) {
+        const int n = rp.L_q - t0 < group ? rp.L_q - t0 : group;
+        AttnPlan part = pl;
+        part.n_tb = (n + pl.Tt - 1) / pl.Tt;
+        if (int rc = launch_attention(reinterpret_cast<const char*>(q_question) + (size_t)t0 * rp.Hq * 256, kv_k, kv_v, n, rp.N, rp.Hq, rp.Hkv,
+                                      rp.L_d + t0, rp.scale, true, true,
+                                      reinterpret_cast<char*>(out) + (dst_rows != nullptr ? 0 : t0 * out_row_stride_bytes), out_row_stride_bytes,
+                                      dst_rows != nullptr ? dst_rows + t0 : nullptr, lse != nullptr ? lse + t0 : nullptr,
+                                      reinterpret_cast<DeviceStatus*>(base), reinterpret_cast<char*>(base) + kStatusBytes, scratch, st, nullptr,
+                                      &part, rp.L_q)) return rc;
+    }
+    return DAF_OK;
 }
 
 // Status of the calls made through daf_qd_attn_static on the current device since the last poll: the

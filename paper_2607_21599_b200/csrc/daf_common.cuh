@@ -65,7 +65,7 @@ size_t attn_partial_bytes(int n_q, int Hq, int n_splits);
 int launch_attention(const void* q, const void* k, const void* v, int n_q, int n_kv, int Hq, int Hkv, int causal_off,
                      float scale, bool pack_group, bool allow_split, void* out, long long out_row_stride_bytes,
                      const int32_t* dst_rows, float* lse, DeviceStatus* status, void* scratch, size_t scratch_bytes,
-                     cudaStream_t stream, const int32_t* q_pos = nullptr, const AttnPlan* plan = nullptr);   // plan: null = planned here
+                     cudaStream_t stream, const int32_t* q_pos = nullptr, const AttnPlan* plan = nullptr, int lse_stride = 0);   // null, 0: planned here, n_q
 // Steps 2 and 3 of a layer from one list of work items (one attention launch and one merge launch).
 struct JointPlan {
     int Gp_i, Tt_i, n_tb_i, head_blocks_i, chunk, n_slots, items_i;       // important-token stage (chunk > 0: causal chains cut)

@@ -74,6 +74,23 @@ def test_static_scratch_entry_point_matches_workspace_entry_point_twice():
     assert torch.equal(third[2], first[2])
 
 
+@pytest.mark.parametrize("L_d,L_q,Hq,Hkv", [(890, 1309, 4, 1), (32793, 237, 32, 4), (503, 2858, 14, 2), (3132, 5089, 8, 8)])
+def test_static_scratch_entry_point_gives_the_same_bits_where_the_partial_rows_outgrow_it(L_d, L_q, Hq, Hkv):
+    """Rows and log-sum-exps of daf_qd_attn, also where its plan needs more scratch for partial rows than the array has."""
+    p = api.make_params(L_d, L_q, 0.0, Hq, Hkv)
+    partial = api.daf_workspace_bytes(p) - api.daf_workspace_bytes(api.make_params(L_d, 0, 0.0, Hq, Hkv))
+    assert partial > api.daf_qd_attn_static_max_bytes()
+    ref, ref_lse, got, got_lse, _ = _run_both(L_d, L_q, Hq, Hkv, seed=303)
+    assert torch.equal(got[:L_q], ref) and torch.all(got[L_q] == 5.0)
+    assert torch.equal(got_lse, ref_lse)
+    # the same rows scattered
+    N = L_d + L_q
+    q, k, v = (W.normal_bf16(s, 303 + i).cuda() for i, s in enumerate([(L_q, Hq, 128), (N, Hkv, 128), (N, Hkv, 128)]))
+    rows = torch.randperm(L_q, generator=torch.Generator().manual_seed(1)).to(torch.int32).cuda()
+    api.check(api.daf_qd_attn_static(p, q, k, v, got, Hq * 256, rows, None), "daf_qd_attn_static")
+    assert torch.equal(got[rows.long()], ref)
+
+
 def test_static_scratch_entry_point_rejects_oversized_problems():
     build.build()
     # 128 question rows x 64 heads split four ways over the context needs a little more than the array holds
