@@ -138,6 +138,18 @@ def test_host_side_argument_validation(lib):
     assert api.daf_layer_host_end(ok, None) == api.DAF_ERR_WORKSPACE
 
 
+def _partial_bytes(L_d, L_q, Hq, Hkv):
+    """Scratch for the partial rows of a question's key ranges."""
+    return api.daf_workspace_bytes(api.make_params(L_d, L_q, 0.0, Hq, Hkv)) - api.daf_workspace_bytes(api.make_params(L_d, 0, 0.0, Hq, Hkv))
+
+
+@pytest.mark.parametrize("L_d,L_q,Hq,Hkv,cut", [(248, 5186, 16, 1, False), (1507, 5875, 8, 8, False), (289, 5810, 16, 8, False),
+                                                (1838, 2565, 16, 1, False), (28188, 4866, 16, 8, True), (32768, 64, 28, 4, True)])
+def test_keys_of_a_long_question_are_cut_only_where_that_pays(lib, L_d, L_q, Hq, Hkv, cut):
+    """Token blocks that fill the GPU by themselves, over a staircase that is most of the keys: whole."""
+    assert (_partial_bytes(L_d, L_q, Hq, Hkv) > 0) == cut
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(api, "_lib", None)
     monkeypatch.setattr(api, "LIB_PATH", str(tmp_path / "nope.so"))
