@@ -1096,7 +1096,9 @@ static int question_steps_per_split(int total, int ctas, int n_q, float mb) {
     const int sms = num_sms(), slots = 2 * sms;
     float best_us = 0.f;
     int best = total;
-    const int most = ctas > slots && 2 * n_q > total * kSubN ? 1 : kMaxSplits;
+    int most = ctas > slots && 2 * n_q > total * kSubN ? 1 : kMaxSplits;
+    // partial rows of a very long question are not worth more memory than this (a range per CTA slot takes 20 MB at most)
+    if (most > 1 && mb * (float)most > 256.f) most = mb > 128.f ? 1 : (int)(256.f / mb);
     for (int n = 1; n <= most && n <= total; ++n) {
         const int even = (total + n - 1) / n;
         for (int j = 0; j < 8; ++j) {

@@ -150,6 +150,11 @@ def test_keys_of_a_long_question_are_cut_only_where_that_pays(lib, L_d, L_q, Hq,
     assert (_partial_bytes(L_d, L_q, Hq, Hkv) > 0) == cut
 
 
+@pytest.mark.parametrize("L_d,L_q,Hq,Hkv", [(53127, 4798, 32, 1), (135013, 1212, 128, 1), (151821, 3106, 64, 1), (200000, 900, 256, 2)])
+def test_partial_rows_of_a_long_question_take_a_bounded_workspace(lib, L_d, L_q, Hq, Hkv):
+    assert _partial_bytes(L_d, L_q, Hq, Hkv) <= 256 << 20
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(api, "_lib", None)
     monkeypatch.setattr(api, "LIB_PATH", str(tmp_path / "nope.so"))
