@@ -480,7 +480,15 @@ struct SideLane {
         if (stream) cudaStreamDestroy(stream);
     }
 };
+// While a stream of this thread is being captured (or, in the global mode, of any thread), calls that create or query another
+// stream fail and spoil that capture, unless the thread says that it knows what it does: these touch no captured stream.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 SideLane* side_lane() {
+    RelaxedCapture relaxed;
     constexpr int kDevices = 16;
     static thread_local SideLane lanes[kDevices][2];
     static thread_local unsigned turn = 0;

@@ -4,6 +4,7 @@ attention outputs must be within max-abs 2e-2 and mean-abs 2e-3 of the oracle
 (bf16 operands and output, fp32 accumulation), plus a relative Frobenius bound
 that stays meaningful where outputs are small."""
 import math
+import threading
 
 import numpy as np
 import pytest
@@ -545,6 +546,51 @@ def test_host_layer_with_a_pinned_cache_changes_only_the_rows_that_change(fuse_m
             assert np.array_equal(_f(got), ref[name] if copy_back else _f(before)), name
         rows = torch.from_numpy(ref["row_pos"]).long() if fuse_mode == 1 else slice(None)
         _assert_close(hidden[rows], ref["hidden"][rows] if fuse_mode == 0 else ref["hidden"][ref["row_pos"]], "hidden rows")
+
+
+def test_host_layer_begun_while_another_stream_is_captured():
+    """A layer from pinned memory begun on one stream while the thread captures another (global mode): the capture stays whole,
+    on the thread's first such layer and on later ones."""
+    w = W.Workload("t", 47, 8, 2, 128, 1, 1200, 1200, 20, 0.25, "lognormal", 1)
+    L = W.make_layer(w, 0)
+    p = api.make_params(w.L_d, w.L_q, w.r, w.n_q_heads, w.n_kv_heads)
+    k = api.daf_num_important(w.L_d, w.r)
+    arena = torch.zeros(api.daf_layer_host_arena_bytes(p), dtype=torch.uint8, device="cuda")
+    h = {n: t.pin_memory() for n, t in L.items() if t is not None}
+    ref = _oracle_layer(w, L, 0)
+    failed = []
+
+    def work():          # (a thread of its own: it has no second stream yet)
+        try:
+            x = torch.zeros(16, device="cuda")
+            captured, other = torch.cuda.Stream(), torch.cuda.Stream()
+            for turn in range(3):
+                kv = [torch.cat([L[n], torch.zeros(w.L_q, w.n_kv_heads, 128, dtype=torch.bfloat16)]).pin_memory()
+                      for n in ("k_cached", "v_cached")]
+                hidden = torch.full((k + w.L_q, w.n_q_heads, 128), -9.0, dtype=torch.bfloat16).pin_memory()
+                idx_out = torch.full((k,), -1, dtype=torch.int32).pin_memory()
+                torch.cuda.synchronize()
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=captured):
+                    x.add_(1.0)
+                    rc = api.daf_layer_host_begin(p, h["scores"], 1, None, h["q_fresh"], h["k_fresh"], h["v_fresh"], kv[0], kv[1], 1,
+                                                  hidden, idx_out, arena, other)
+                    x.add_(1.0)
+                api.check(rc, "daf_layer_host_begin")
+                api.check(api.daf_layer_host_end(p, arena, other), "daf_layer_host_end")
+                graph.replay()
+                torch.cuda.synchronize()
+                assert torch.all(x == 2.0 * (turn + 1)) and np.array_equal(idx_out.numpy(), ref["idx"])
+                assert np.array_equal(_f(kv[0]), ref["kv_k"]) and np.array_equal(_f(kv[1]), ref["kv_v"])
+                _assert_close(hidden, ref["hidden"], "hidden rows")
+        except BaseException as e:      # noqa: BLE001 (handed to the test)
+            failed.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    if failed:
+        raise failed[0]
 
 
 def test_host_layers_pipelined_on_two_arenas_match_the_plain_host_call():
