@@ -507,12 +507,19 @@ SideLane* side_lane() {
     return &l;
 }
 
-// True (and *dev set) when `h` is pinned host memory that kernels on the current device can address.
-bool mapped_host_pointer(const void* h, const void** dev) {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, h) != cudaSuccess) { (void)cudaGetLastError(); return false; }
-    if (attr.type != cudaMemoryTypeHost || attr.devicePointer == nullptr) return false;
-    *dev = attr.devicePointer;
+// True (and *dev set) when the `bytes` at `h` are pinned host memory that kernels on the current device can address.  (Both ends
+// are asked for: a buffer of which only a part is registered must not be read or written by a kernel.)
+bool mapped_host_range(const void* h, size_t bytes, const void** dev) {
+    const char* ends[2] = {reinterpret_cast<const char*>(h), reinterpret_cast<const char*>(h) + (bytes - 1)};
+    const char* at[2];
+    for (int i = 0; i < 2; ++i) {
+        cudaPointerAttributes attr{};
+        if (cudaPointerGetAttributes(&attr, ends[i]) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+        if (attr.type != cudaMemoryTypeHost || attr.devicePointer == nullptr) return false;
+        at[i] = reinterpret_cast<const char*>(attr.devicePointer);
+    }
+    if (at[1] != at[0] + (bytes - 1)) return false;
+    *dev = at[0];
     return true;
 }
 
@@ -614,13 +621,13 @@ int daf_layer_host_begin(const daf_params* p, const float* h_scores, int32_t n_s
     // rows straight from the host (k + L_q rows instead of N cross the link) and only the question's Q rows, which
     // the attention kernel reads through a tensor map, are copied; otherwise the tensors are copied whole.
     RowSource rows = {};
-    const bool in_place_rows = rp.k > 0 && mapped_host_pointer(h_q_fresh, &rows.q) && mapped_host_pointer(h_k_fresh, &rows.k) &&
-                               mapped_host_pointer(h_v_fresh, &rows.v);
+    const bool in_place_rows = rp.k > 0 && mapped_host_range(h_q_fresh, qrow * rp.N, &rows.q) &&
+                               mapped_host_range(h_k_fresh, kvrow * rp.N, &rows.k) && mapped_host_range(h_v_fresh, kvrow * rp.N, &rows.v);
     // Of the cache a layer changes only the rows of the important tokens and of the question.  When the caller's cache is
     // pinned too, the same kernel writes those rows straight back to it; otherwise the cache is copied back whole.
     const void *host_k = nullptr, *host_v = nullptr;
-    const bool rows_back = in_place_rows && mapped_host_pointer(h_kv_k, &host_k) && mapped_host_pointer(h_kv_v, &host_v) &&
-                           aligned16(host_k) && aligned16(host_v);
+    const bool rows_back = in_place_rows && mapped_host_range(h_kv_k, kvrow * rp.N, &host_k) &&
+                           mapped_host_range(h_kv_v, kvrow * rp.N, &host_v) && aligned16(host_k) && aligned16(host_v);
     if (rows_back && copy_back_kv) { rows.host_k = const_cast<void*>(host_k); rows.host_v = const_cast<void*>(host_v); }
     if (rows_back && rp.L_q > 0 && rp.fuse_mode == 0) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;

@@ -548,6 +548,40 @@ def test_host_layer_with_a_pinned_cache_changes_only_the_rows_that_change(fuse_m
         _assert_close(hidden[rows], ref["hidden"][rows] if fuse_mode == 0 else ref["hidden"][ref["row_pos"]], "hidden rows")
 
 
+@pytest.mark.parametrize("part", ["q_fresh", "k_fresh", "v_fresh", "kv_k", "kv_v"])
+def test_host_layer_with_a_buffer_of_which_only_a_part_is_registered(part):
+    """Such a buffer is left to the copies, which may refuse it; the other four are pinned."""
+    w = W.Workload("t", 48, 8, 2, 128, 1, 1200, 1200, 20, 0.25, "lognormal", 1)
+    L = W.make_layer(w, 0)
+    p = api.make_params(w.L_d, w.L_q, w.r, w.n_q_heads, w.n_kv_heads)
+    k = api.daf_num_important(w.L_d, w.r)
+    arena = torch.zeros(api.daf_layer_host_arena_bytes(p), dtype=torch.uint8, device="cuda")
+    h = {n: L[n] for n in ("q_fresh", "k_fresh", "v_fresh")}
+    h["kv_k"], h["kv_v"] = (torch.cat([L[n], torch.zeros(w.L_q, w.n_kv_heads, 128, dtype=torch.bfloat16)])
+                            for n in ("k_cached", "v_cached"))
+    raw = torch.zeros(h[part].nbytes + 8192, dtype=torch.uint8)
+    start = -raw.data_ptr() % 4096
+    held = raw[start: start + h[part].nbytes].view(torch.bfloat16).view(h[part].shape)
+    held.copy_(h[part])
+    h = {n: held if n == part else t.pin_memory() for n, t in h.items()}
+    hidden = torch.full((k + w.L_q, w.n_q_heads, 128), -9.0, dtype=torch.bfloat16).pin_memory()
+    idx_out = torch.full((k,), -1, dtype=torch.int32).pin_memory()
+    cudart = torch.cuda.cudart()
+    assert int(cudart.cudaHostRegister(held.data_ptr(), held.nbytes // 2 // 4096 * 4096, 0)) == 0
+    try:
+        rc = api.daf_layer_host(p, L["scores"].pin_memory(), 1, None, h["q_fresh"], h["k_fresh"], h["v_fresh"], h["kv_k"], h["kv_v"],
+                                1, hidden, idx_out, arena)
+        torch.cuda.synchronize()
+    finally:
+        assert int(cudart.cudaHostUnregister(held.data_ptr())) == 0
+    assert rc in (api.DAF_OK, api.DAF_ERR_CUDA)
+    if rc == api.DAF_OK:
+        ref = _oracle_layer(w, L, 0)
+        assert np.array_equal(idx_out.numpy(), ref["idx"])
+        assert np.array_equal(_f(h["kv_k"]), ref["kv_k"]) and np.array_equal(_f(h["kv_v"]), ref["kv_v"])
+        _assert_close(hidden, ref["hidden"], "hidden rows")
+
+
 def test_host_layer_begun_while_another_stream_is_captured():
     """A layer from pinned memory begun on one stream while the thread captures another (global mode): the capture stays whole,
     on the thread's first such layer and on later ones."""
