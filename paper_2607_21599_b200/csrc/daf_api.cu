@@ -490,12 +490,12 @@ struct RelaxedCapture {
 SideLane* side_lane() {
     RelaxedCapture relaxed;
     constexpr int kDevices = 16;
-    static thread_local SideLane lanes[kDevices][2];
-    static thread_local unsigned turn = 0;
+    static thread_local struct { SideLane lane[2]; unsigned turn = 0; } devices[kDevices];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) { (void)cudaGetLastError(); return nullptr; }
-    SideLane& l = lanes[dev][turn & 1u];
-    const SideLane& other = lanes[dev][++turn & 1u];
+    auto& d = devices[dev];
+    SideLane& l = d.lane[d.turn & 1u];
+    const SideLane& other = d.lane[++d.turn & 1u];
     if ((l.stream == nullptr && cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking) != cudaSuccess) ||
         (l.fork == nullptr && cudaEventCreateWithFlags(&l.fork, cudaEventDisableTiming) != cudaSuccess) ||
         (l.join == nullptr && cudaEventCreateWithFlags(&l.join, cudaEventDisableTiming) != cudaSuccess)) {

@@ -1135,11 +1135,11 @@ AttnPlan plan_attention(int n_q, int n_kv, int Hq, int G, int causal_off, bool p
     pl.steps_per_split = total > 0 ? total : 1;
     if (allow_split && total > 1) {
         // a loop over layers or questions asks for the same shape over and over: each thread keeps its last answer
-        struct Last { int total, ctas, n_q, Hq, steps; };
-        static thread_local Last last = {0, 0, 0, 0, 0};
-        const int ctas = pl.n_tb * pl.head_blocks;
-        if (last.total != total || last.ctas != ctas || last.n_q != n_q || last.Hq != Hq)
-            last = Last{total, ctas, n_q, Hq, question_steps_per_split(total, ctas, n_q, (float)n_q * (float)Hq * 516e-6f)};
+        struct Last { int total, ctas, n_q, Hq, sms, steps; };
+        static thread_local Last last = {0, 0, 0, 0, 0, 0};
+        const int ctas = pl.n_tb * pl.head_blocks, sms = num_sms();
+        if (last.total != total || last.ctas != ctas || last.n_q != n_q || last.Hq != Hq || last.sms != sms)
+            last = Last{total, ctas, n_q, Hq, sms, question_steps_per_split(total, ctas, n_q, (float)n_q * (float)Hq * 516e-6f)};
         pl.steps_per_split = last.steps;
         pl.n_splits = (total + pl.steps_per_split - 1) / pl.steps_per_split;
     }
@@ -1176,13 +1176,14 @@ constexpr float kCostMergeUsPerMBCut = 0.45f;  // partial rows of cut causal cha
 int g_force_chunk = 0, g_force_splits_q = 0;   // tuning builds can pin the choice
 float g_last_predicted_us = 0.f;
 
-struct JointShape { int k, L_q, L_d, Hq, G; };
+struct JointShape { int k, L_q, L_d, Hq, G, sms; };
 bool operator<(const JointShape& a, const JointShape& b) {
     if (a.k != b.k) return a.k < b.k;
     if (a.L_q != b.L_q) return a.L_q < b.L_q;
     if (a.L_d != b.L_d) return a.L_d < b.L_d;
     if (a.Hq != b.Hq) return a.Hq < b.Hq;
-    return a.G < b.G;
+    if (a.G != b.G) return a.G < b.G;
+    return a.sms < b.sms;
 }
 
 // Fills the fields of `jp` that follow from chunk (n_tb_i or more: whole chains) and n_splits_q.
@@ -1245,7 +1246,7 @@ float predict_us(const JointPlan& jp, int k, int L_q, int L_d, int Hq, float* bu
 JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     static std::mutex mu;
     static std::map<JointShape, JointPlan> cache;
-    const JointShape shape{k, L_q, L_d, Hq, G};
+    const JointShape shape{k, L_q, L_d, Hq, G, num_sms()};      // (a plan is made for a number of SMs)
     const bool forced = g_force_chunk > 0 || g_force_splits_q > 0;
     // a layer loop asks for the same shape over and over: each thread keeps its last answer (no lock)
     static thread_local bool have_last = false;
