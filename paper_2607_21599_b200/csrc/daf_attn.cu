@@ -1202,44 +1202,56 @@ void set_choice(JointPlan& jp, int chunk, int n_splits_q, int L_q, int L_d, int 
     jp.part_bytes_q = attn_partial_bytes(L_q, Hq, jp.n_splits_q);
 }
 
-// Predicted time of the attention launch + merge for a filled plan, in microseconds.
-float predict_us(const JointPlan& jp, int k, int L_q, int L_d, int Hq, float* busy_us = nullptr) {
+// Predicted time of the attention launch + merge for a filled plan, in microseconds; of a plan that cannot come below `limit`
+// only a lower bound.
+float predict_us(const JointPlan& jp, int k, int L_q, int L_d, int Hq, float limit, float* busy_us) {
+    auto cost = [](int substeps) { return kCostItemUs + kCostSubStepUs * (float)substeps; };
+    // question items first (grid order: splits, then units from the last one down)
+    auto question_items = [&](auto&& run) {
+        for (int s = 0; s < jp.n_splits_q; ++s)
+            for (int u = jp.n_tb_q - 1; u >= 0; --u) {
+                const int last_tok = (u + 1) * jp.Tt_q < L_q ? (u + 1) * jp.Tt_q : L_q;
+                const int begin = s * jp.steps_per_split_q * kSubN;
+                int end = begin + jp.steps_per_split_q * kSubN;
+                if (end > L_d + last_tok) end = L_d + last_tok;
+                if (end > begin) run(jp.head_blocks_q, (end - begin + kSubN - 1) / kSubN);
+            }
+    };
+    // important-token items: units from the last one down, head blocks together
+    size_t cut_rows = 0;
+    auto important_items = [&](auto&& run) {
+        for (int u = jp.n_tb_i - 1; u >= 0; --u) {
+            const int steps = (((u + 1) * jp.Tt_i < k ? (u + 1) * jp.Tt_i : k) + kSubN - 1) / kSubN;
+            const int ranges = jp.chunk > 0 ? u / jp.chunk + 1 : 1;
+            for (int j = ranges - 1; j >= 0; --j) run(jp.head_blocks_i, (j + 1) * steps / ranges - j * steps / ranges);
+            if (ranges > 1) cut_rows += (size_t)ranges * jp.Tt_i * Hq;
+        }
+    };
     const int slots = num_sms() * 2;
+    float busy = 0.f;
+    auto add = [&](int count, int substeps) { busy += cost(substeps) * (float)count; };
+    question_items(add);
+    important_items(add);
+    busy /= (float)slots;
+    *busy_us = busy;
+    const float merge_us = jp.n_splits_q > 1 || jp.chunk > 0 ? kCostMergeUs + kCostMergeUsPerMB * (float)jp.part_bytes_q / 1e6f +
+                                                                   kCostMergeUsPerMBCut * (float)(cut_rows * 516) / 1e6f
+                                                             : 0.f;
+    if (busy + merge_us >= limit) return busy + merge_us;
     std::priority_queue<float, std::vector<float>, std::greater<float>> free_at;
     for (int i = 0; i < slots; ++i) free_at.push(0.f);
-    float makespan = 0.f, busy = 0.f;
-    auto run = [&](int count, int substeps) {
-        const float cost = kCostItemUs + kCostSubStepUs * (float)substeps;
-        busy += cost * (float)count / (float)slots;
+    float makespan = 0.f;
+    auto dispatch = [&](int count, int substeps) {
         for (int i = 0; i < count; ++i) {
-            const float t = free_at.top() + cost;
+            const float t = free_at.top() + cost(substeps);
             free_at.pop();
             free_at.push(t);
             if (t > makespan) makespan = t;
         }
     };
-    // question items: split-major, token blocks from the last one down, head blocks together
-    for (int s = 0; s < jp.n_splits_q; ++s)
-        for (int u = jp.n_tb_q - 1; u >= 0; --u) {
-            const int last_tok = (u + 1) * jp.Tt_q < L_q ? (u + 1) * jp.Tt_q : L_q;
-            const int begin = s * jp.steps_per_split_q * kSubN;
-            int end = begin + jp.steps_per_split_q * kSubN;
-            if (end > L_d + last_tok) end = L_d + last_tok;
-            if (end > begin) run(jp.head_blocks_q, (end - begin + kSubN - 1) / kSubN);
-        }
-    // important-token items: units from the last one down, head blocks together
-    size_t cut_rows = 0;
-    for (int u = jp.n_tb_i - 1; u >= 0; --u) {
-        const int steps = (((u + 1) * jp.Tt_i < k ? (u + 1) * jp.Tt_i : k) + kSubN - 1) / kSubN;
-        const int ranges = jp.chunk > 0 ? u / jp.chunk + 1 : 1;
-        for (int j = ranges - 1; j >= 0; --j) run(jp.head_blocks_i, (j + 1) * steps / ranges - j * steps / ranges);
-        if (ranges > 1) cut_rows += (size_t)ranges * jp.Tt_i * Hq;
-    }
-    if (busy_us != nullptr) *busy_us = busy;
-    float us = makespan;
-    if (jp.n_splits_q > 1 || jp.chunk > 0)
-        us += kCostMergeUs + kCostMergeUsPerMB * (float)jp.part_bytes_q / 1e6f + kCostMergeUsPerMBCut * (float)(cut_rows * 516) / 1e6f;
-    return us;
+    question_items(dispatch);
+    important_items(dispatch);
+    return makespan + merge_us;
 }
 }  // namespace
 
@@ -1270,7 +1282,8 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     const int steps_q = (L_d + L_q + kSubN - 1) / kSubN;
     if (forced) {
         set_choice(jp, g_force_chunk > 0 ? g_force_chunk : jp.n_tb_i, g_force_splits_q, L_q, L_d, Hq);
-        g_last_predicted_us = predict_us(jp, k, L_q, L_d, Hq);
+        float busy;
+        g_last_predicted_us = predict_us(jp, k, L_q, L_d, Hq, INFINITY, &busy);
         return jp;
     }
     // Candidates: the causal chains whole, or cut so that the longest has 2 to 6 ranges; every distinct number of question
@@ -1279,7 +1292,7 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
     // important tokens of 4 heads on 4: 45.6 -> 28.5 us, 1008: 18.1 -> 12.7), half of those around 0.8 and most above got
     // slower (28/4, 475 tokens, 0.94: 13.8 -> 18.1).
     JointPlan best = jp;
-    float best_us = -1.f, whole_us = 0.f, whole_busy = 0.f;
+    float best_us = INFINITY, whole_us = 0.f, whole_busy = 0.f;
     int last_chunk = 0;
     for (int m = 1; m <= kMaxChainRanges; ++m) {
         const int chunk = (jp.n_tb_i + m - 1) / m;
@@ -1293,9 +1306,10 @@ JointPlan plan_joint(int k, int L_q, int L_d, int Hq, int G) {
             if (cand.steps_per_split_q == last_steps) continue;
             last_steps = cand.steps_per_split_q;
             if (cand.part_bytes_i > ((size_t)256 << 20)) continue;   // partials of a large problem: not worth their memory
+            const float limit = m == 1 || best.chunk > 0 ? best_us : kCutGain * whole_us;
             float busy;
-            const float us = predict_us(cand, k, L_q, L_d, Hq, &busy);
-            if (best_us < 0.f || us < (m == 1 || best.chunk > 0 ? best_us : kCutGain * whole_us)) {
+            const float us = predict_us(cand, k, L_q, L_d, Hq, limit, &busy);
+            if (us < limit) {
                 best_us = us; best = cand;
                 if (m == 1) { whole_us = us; whole_busy = busy; }
             }
