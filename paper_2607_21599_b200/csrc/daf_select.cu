@@ -838,10 +838,12 @@ __device__ __forceinline__ uint4 expand8(uint2 bytes, float scale) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Bound by HBM.  A CTA takes 2048 runs of 8 elements that lie together, a thread eight of them: each warp reads 256 and
-// writes 512 consecutive bytes at a time (16 elements per thread, two stores 32 bytes apart, moved 5.5 TB/s at 16k tokens
-// of 8 heads: 18.4 us; this way 6.9 TB/s, 14.5 us; layer 105 -> 102.5).
-constexpr int kExpandPerThread = 8;
+// A streaming pass, read and write.  A CTA takes 256 kPer runs of 8 elements that lie together, a thread kPer of them: each warp
+// reads 256 and writes 512 consecutive bytes at a time (16 elements per thread, two stores 32 bytes apart: 18.4 us at 16k tokens
+// of 8 heads, 100 MB in all; this way 14.5, of which L2 takes part of the writes; layer 105 -> 102.5).  Eight runs a thread
+// keep enough loads under way on a full GPU; a cache of which eight would leave SMs without a CTA takes one (322 tokens of 4
+// heads 3.3 us with eight).
+template <int kPer>
 __global__ void __launch_bounds__(256)
 expand_fp8_cache_kernel(const uint2* __restrict__ k8, const uint2* __restrict__ v8, const float* __restrict__ k_scale,
                         const float* __restrict__ v_scale, uint4* __restrict__ kv_k, uint4* __restrict__ kv_v,
@@ -852,15 +854,15 @@ expand_fp8_cache_kernel(const uint2* __restrict__ k8, const uint2* __restrict__ 
     const uint2* src = is_v ? v8 : k8;
     const float* sc = is_v ? v_scale : k_scale;
     uint4* dst = is_v ? kv_v : kv_k;
-    const long long r0 = (long long)blockIdx.x * (256 * kExpandPerThread) + threadIdx.x;
-    uint2 in[kExpandPerThread];
+    const long long r0 = (long long)blockIdx.x * (256 * kPer) + threadIdx.x;
+    uint2 in[kPer];
 #pragma unroll
-    for (int u = 0; u < kExpandPerThread; ++u)
+    for (int u = 0; u < kPer; ++u)
         if (r0 + u * 256 < n_runs) in[u] = __ldcs(src + r0 + u * 256);
 #pragma unroll
-    for (int u = 0; u < kExpandPerThread; ++u) {
+    for (int u = 0; u < kPer; ++u) {
         const long long r = r0 + u * 256;
-        if (r < n_runs) dst[r] = expand8(in[u], sc != nullptr ? __ldg(sc + (int)((r >> 4) % Hkv)) : 1.0f);   // a head is 16 runs
+        if (r < n_runs) dst[r] = expand8(in[u], sc != nullptr ? __ldg(sc + (unsigned)(r >> 4) % (unsigned)Hkv) : 1.0f);   // a head is 16 runs
     }
     if (beside_selection) pdl_wait();      // see launch_select
 }
@@ -868,9 +870,10 @@ expand_fp8_cache_kernel(const uint2* __restrict__ k8, const uint2* __restrict__ 
 int launch_expand_fp8(const ResolvedParams& rp, const Fp8Cache& c, void* kv_k, void* kv_v, cudaStream_t stream, bool beside_selection) {
     const long long n_runs = (long long)rp.L_d * rp.Hkv * 16;     // per tensor
     if (n_runs == 0) return DAF_OK;
-    const long long per_cta = 256 * kExpandPerThread;
-    const cudaError_t e = launch_kernel(expand_fp8_cache_kernel, dim3((unsigned)((n_runs + per_cta - 1) / per_cta), 2), dim3(256), 0, stream,
-                                        reinterpret_cast<const uint2*>(c.k8), reinterpret_cast<const uint2*>(c.v8), c.k_scale, c.v_scale,
+    auto ctas = [&](int per) { return (unsigned)((n_runs + 256 * per - 1) / (256 * per)); };
+    const bool small = !beside_selection && 2 * ctas(8) < 148;     // (beside the selection more CTAs would only wait for it)
+    const cudaError_t e = launch_kernel(small ? expand_fp8_cache_kernel<1> : expand_fp8_cache_kernel<8>, dim3(ctas(small ? 1 : 8), 2), dim3(256), 0,
+                                        stream, reinterpret_cast<const uint2*>(c.k8), reinterpret_cast<const uint2*>(c.v8), c.k_scale, c.v_scale,
                                         reinterpret_cast<uint4*>(kv_k), reinterpret_cast<uint4*>(kv_v), n_runs, rp.Hkv,
                                         beside_selection ? 1 : 0);
     count_launch();

@@ -25,7 +25,8 @@ def _fp8_cache(shape, seed, dev):
     return b.to(dev)
 
 
-@pytest.mark.parametrize("L_d,Hkv,scaled", [(1024, 4, False), (777, 8, True), (5, 1, True), (6144, 4, True)])
+@pytest.mark.parametrize("L_d,Hkv,scaled", [(1024, 4, False), (777, 8, True), (5, 1, True), (6144, 4, True), (1168, 8, True), (1169, 8, True),
+                                              (1169, 3, True)])
 def test_expansion_is_bit_exact(L_d, Hkv, scaled):
     build.build()
     dev = "cuda"
