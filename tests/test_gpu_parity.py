@@ -548,6 +548,47 @@ def test_host_layer_with_a_pinned_cache_changes_only_the_rows_that_change(fuse_m
         _assert_close(hidden[rows], ref["hidden"][rows] if fuse_mode == 0 else ref["hidden"][ref["row_pos"]], "hidden rows")
 
 
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("overwrite", [0, 1])
+@pytest.mark.parametrize("L_d,L_q,r,Hq,Hkv,cut_in", [(1100, 33, 0.2, 14, 2, "K"), (1101, 5, 0.1, 8, 8, "V"), (1100, 33, 0.25, 8, 2, "between")])
+def test_host_layer_copies_part_of_the_cache_beside_the_gather(L_d, L_q, r, Hq, Hkv, cut_in, overwrite, pipelined):
+    """All host tensors pinned: the first part of the cache is copied in on the second stream, cut within K, within V or between
+    them (2 L_d KV rows less the important Q rows' bytes), and one layer at a time or two at once; against the oracle."""
+    w = W.Workload("t", 49, Hq, Hkv, 128, 3, L_d, L_d, L_q, r, "lognormal", 1)
+    p = api.make_params(L_d, L_q, r, Hq, Hkv, overwrite_doc_kv=overwrite)
+    k, cache = api.daf_num_important(L_d, r), L_d * Hkv * 256
+    early = 2 * cache - k * Hq * 256
+    assert {"K": 0 < early < cache, "V": cache < early < 2 * cache, "between": early == cache}[cut_in]
+    arenas = [torch.zeros(api.daf_layer_host_arena_bytes(p), dtype=torch.uint8, device="cuda") for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    layers = []
+    for i in range(w.layers):
+        L = W.make_layer(w, i)
+        h = {n: t.pin_memory() for n, t in L.items() if t is not None}
+        h["kv_k"], h["kv_v"] = (torch.cat([L[n], torch.zeros(L_q, Hkv, 128, dtype=torch.bfloat16)]).pin_memory()
+                                for n in ("k_cached", "v_cached"))
+        h["hidden"] = torch.full((k + L_q, Hq, 128), -9.0, dtype=torch.bfloat16).pin_memory()
+        h["idx_out"] = torch.full((k,), -1, dtype=torch.int32).pin_memory()
+        layers.append((L, h))
+    for i, (_, h) in enumerate(layers):
+        # layers alternate between positions ranked from scores and positions given
+        given = torch.from_numpy(oracle.select(layers[i][0]["scores"].numpy(), k)).pin_memory() if i % 2 else None
+        h["given"] = given
+        api.check(api.daf_layer_host_begin(p, None if i % 2 else h["scores"], 1, given, h["q_fresh"], h["k_fresh"], h["v_fresh"],
+                                           h["kv_k"], h["kv_v"], 1, h["hidden"], h["idx_out"], arenas[i & 1], streams[i & 1]), "begin")
+        if not pipelined:
+            api.check(api.daf_layer_host_end(p, arenas[i & 1], streams[i & 1]), "end")
+        elif i > 0:
+            api.check(api.daf_layer_host_end(p, arenas[(i - 1) & 1], streams[(i - 1) & 1]), "end")
+    if pipelined:
+        api.check(api.daf_layer_host_end(p, arenas[(w.layers - 1) & 1], streams[(w.layers - 1) & 1]), "end")
+    for L, h in layers:
+        ref = _oracle_layer(w, L, 0, overwrite)
+        assert np.array_equal(h["idx_out"].numpy(), ref["idx"])
+        assert np.array_equal(_f(h["kv_k"]), ref["kv_k"]) and np.array_equal(_f(h["kv_v"]), ref["kv_v"])
+        _assert_close(h["hidden"], ref["hidden"], "hidden rows")
+
+
 @pytest.mark.parametrize("part", ["q_fresh", "k_fresh", "v_fresh", "kv_k", "kv_v"])
 def test_host_layer_with_a_buffer_of_which_only_a_part_is_registered(part):
     """Such a buffer is left to the copies, which may refuse it; the other four are pinned."""
