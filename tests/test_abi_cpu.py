@@ -150,6 +150,14 @@ def test_keys_of_a_long_question_are_cut_only_where_that_pays(lib, L_d, L_q, Hq,
     assert (_partial_bytes(L_d, L_q, Hq, Hkv) > 0) == cut
 
 
+@pytest.mark.parametrize("L_d,L_q,Hq,Hkv,ranges", [(130, 5, 4, 4, 1), (450, 16, 7, 1, 8), (700, 20, 14, 2, 12), (900, 9, 7, 1, 15),
+                                                   (1500, 16, 8, 2, 24), (9000, 3, 4, 1, 29), (600, 300, 16, 8, 3), (1000, 64, 64, 8, 4)])
+def test_planned_ranges_of_the_question_shapes_that_cover_the_merge(lib, L_d, L_q, Hq, Hkv, ranges):
+    """On 148 SMs: 1, up to 4, 8, 12, 16, 24 and 32 ranges are merged by forms of their own."""
+    row = L_q * Hq * 516                     # an fp32 row of 128 and its log-sum-exp; the latter padded to 256 bytes in all
+    assert 0 <= _partial_bytes(L_d, L_q, Hq, Hkv) - (ranges * row if ranges > 1 else 0) < 256
+
+
 @pytest.mark.parametrize("L_d,L_q,Hq,Hkv", [(53127, 4798, 32, 1), (135013, 1212, 128, 1), (151821, 3106, 64, 1), (200000, 900, 256, 2)])
 def test_partial_rows_of_a_long_question_take_a_bounded_workspace(lib, L_d, L_q, Hq, Hkv):
     assert _partial_bytes(L_d, L_q, Hq, Hkv) <= 256 << 20

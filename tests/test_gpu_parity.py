@@ -363,9 +363,10 @@ def test_question_attention_matches_oracle(L_d, L_q, Hq, Hkv, qscale):
 
 
 @pytest.mark.parametrize("L_d,L_q,Hq,Hkv", [(130, 5, 4, 4), (450, 16, 7, 1), (700, 20, 14, 2), (900, 9, 7, 1),
-                                            (1500, 16, 8, 2), (9000, 3, 4, 1)])
+                                            (1500, 16, 8, 2), (9000, 3, 4, 1), (600, 300, 16, 8), (1000, 64, 64, 8)])
 def test_question_attention_over_few_and_many_ranges(L_d, L_q, Hq, Hkv):
-    """Every form of the merge (8, 12, 15, 24 and 29 ranges, and none) and ranges that are not whole 128 keys."""
+    """Every form of the merge (8, 12, 15, 24, 29, 3 and 4 ranges, and none; the plans are checked on the host) and ranges that
+    are not whole 128 keys."""
     N = L_d + L_q
     q, k, v = _normal((L_q, Hq, 128), 44), _normal((N, Hkv, 128), 45), _normal((N, Hkv, 128), 46)
     p = api.make_params(L_d, L_q, 0.1, Hq, Hkv)
