@@ -290,7 +290,7 @@ int daf_layer_fp8(const daf_params* p, const float* scores, int32_t n_sig, const
  * the device is part of the call.  `arena` is caller-owned device memory of at
  * least daf_layer_host_arena_bytes(p) bytes.
  *   h_kv_k, h_kv_v  [N, n_kv_heads, 128] host IN/OUT like kv_k/kv_v above
- *                   (copied back only if copy_back_kv != 0)
+ *                   (brought up to date only if copy_back_kv != 0)
  *   h_hidden        host output, layout by fuse_mode (compact mode recommended)
  *   h_idx_out       host int32 [k] (optional)
  * The call synchronises `stream` before returning.
@@ -298,10 +298,18 @@ int daf_layer_fp8(const daf_params* p, const float* scores, int32_t n_sig, const
  * h_k_fresh and h_v_fresh are all pinned memory that the device can address, those rows are read straight from the
  * host by the gather / cache-update kernel (k + L_q rows cross the link instead of N) and only the question's Q rows
  * are copied; otherwise the three tensors are copied whole.  Same results either way.
+ * When h_kv_k and h_kv_v are such memory as well, the cache is not copied back whole: that kernel writes the rows that
+ * change (important rows if overwrite_doc_kv, question rows) straight into them, while `stream` is at it.  In compact
+ * mode with L_q > 0, and unless `stream` is being captured, the layer then also works on a second stream, which starts
+ * behind `stream` and which `stream` waits for: the question's Q rows and the first part of the cache are copied in
+ * beside the gather, and the important tokens' attention and its copy out run beside the rest.  Each host thread keeps
+ * two such streams and four events per device, made on its first layer of this form and given back when it ends.  The
+ * two stages are then cut into work items one by one instead of together, so that hidden rows may differ from those of
+ * the other forms in the order of fp32 sums.
  *
  * daf_layer_host_begin / daf_layer_host_end are the two halves of that call: `begin` (same arguments) enqueues the
- * copies in, the layer and the copies out on `stream` and returns without waiting; `end` waits for `stream` and
- * returns the layer's status.  A caller with two arenas and two streams begins layer i + 1 before it ends layer
+ * copies in, the layer and the copies out (on `stream`, or joined to it) and returns without waiting; `end` waits for
+ * `stream` and returns the layer's status.  A caller with two arenas and two streams begins layer i + 1 before it ends layer
  * i, so that the copies in of one layer run beside the kernels and the copies out of the other (the link to the
  * host carries both directions at once).  Between `begin` and `end` the host buffers and the arena belong to the
  * call; the host buffers must be pinned for the copies to overlap anything.  `end` without a `begin` on that

@@ -142,9 +142,9 @@ def lib() -> ctypes.CDLL:
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
-    if t.is_contiguous():
-        return t.data_ptr()
-    raise ValueError("tensors passed to the DAF library must be contiguous")
+    if not t.is_contiguous():
+        raise ValueError("tensors passed to the DAF library must be contiguous")
+    return t.data_ptr()
 
 
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)

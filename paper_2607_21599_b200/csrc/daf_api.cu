@@ -337,8 +337,8 @@ int layer_impl(const daf_params* p, const Fp8Cache* fp8, const float* scores, in
     const int64_t row_bytes = (int64_t)rp.Hq * 256;
     if (int rc = check_out(hidden, row_bytes, rp.Hq)) return rc;
     // Step 2 reads its Q rows in place and packs them on the way (the largest of the packed tensors: the gather kernel is left
-    // with K/V), unless they lie in host memory: 6k layer 32.9 -> 31.4 us, 11k 113.9 -> 112.2, 28 layers of 6k 728 -> 716, 16k
-    // 87.4 -> 87.7 (there the longer start of an item, positions and then rows from HBM, weighs as much as the copy saved).
+    // with K/V), unless they lie in host memory: 6k layer 31.4 us, 32.9 with the gather kernel packing; 11k 112.2 and 113.9; 16k
+    // 87.7 and 87.4 (there the longer start of an item, positions and then rows from HBM, weighs as much as the copy saved).
     // Not with many tokens in a tile, where that is slower (step2_packs_q), nor when the output rows share memory with what
     // step 2 would still be reading or packing: then the gather kernel packs.
     const size_t hidden_bytes = (size_t)row_bytes * (rp.fuse_mode == 1 ? rp.N : rp.k + rp.L_q);

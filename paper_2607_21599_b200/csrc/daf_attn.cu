@@ -402,8 +402,8 @@ extern "C" int daf_dbg_read_trace(void* host, size_t bytes) {
 // issued as each P_t arrives, in order; only a row that has to be rescaled waits for the product before
 // it to complete (pv_done).  The second CTA of the SM fills what gaps remain.  Final rows in token order
 // leave by tiled bulk stores from the dead Q tile.
-// Two tiles per CTA sharing every K/V tile (half the shared-memory fill traffic, one CTA per SM)
-// measured slower at every size from 1k to 136k tokens and was removed.
+// (Two tiles per CTA sharing every K/V tile, half the shared-memory fill traffic but one CTA per SM, measured slower at every
+// size from 1k to 136k tokens.)
 constexpr int kSubBytes = kSubN * kD * 2;               // 16 KB: K or V of one sub-step, two 64-column halves
 constexpr int kSubHalfBytes = kSubBytes / 2;
 constexpr int kAttnThreads = 192;                      // warps 0-3 softmax, warp 4 TMA, warp 5 MMA
@@ -525,8 +525,8 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
     // Set-up.  The producer thread prepares the barriers and at once starts the loads that need no free
     // slot (Q and the first two sub-steps), so that their latency overlaps the rest of the set-up: the
     // status check (a global read) and the tensor-memory allocation.
-    // Everything up to the wait below touches no memory an earlier kernel writes, so with programmatic
-    // dependent launch it runs while the kernel launched just before (gather / hybrid-cache update) drains.
+    // Everything up to the wait below runs while the kernel launched just before (gather / hybrid-cache update) drains; of memory
+    // it touches only what that kernel does not write, positions and Q rows to be read early (see launch_kernel).
     __shared__ int skip_cta;
     const int32_t* const q_idx = DAF_SEG(q_idx);     // non-null: Q rows are fetched token by token through this list
     const __nv_bfloat16* const q_src = kExtra ? DAF_SEG(q_src) : nullptr;
@@ -797,8 +797,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
         const bool row_valid = (r < a.Gp * a.Tt) && (tok < a.n_q) && row_valid_tile;
         // Last visible key.  A row without a token (a tile's remainder, Q rows of zeros) takes the limit its place would
         // have: its logits are plain zeros and it never leaves, whereas a limit of its own would put its warp through the
-        // masking code in every sub-step (28 query heads on 4, where a tile has two such rows: question rows at 32k
-        // 49.4 -> 47.2 us, 6k layer 35.7 -> 34.5, 28 layers of it 811 -> 792).
+        // masking code in every sub-step (28 query heads on 4, two such rows a tile, question rows at 32k: 49.4 us so, 47.2).
         const long long lim_ll = (a.q_pos && tok < a.n_q) ? (long long)__ldg(a.q_pos + tok) : (long long)tok + a.causal_off;
         const int limit = (int)min(lim_ll, (long long)a.n_kv - 1);
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
@@ -902,9 +901,9 @@ struct CombineArgs {
 };
 
 // kMost: the largest number of partials a launch of this form merges.  Bound by latency: all of a row's partials and their
-// log-sum-exps are requested at once (a second round is a second trip to L2: as eight and then four by four, 24 tokens of 28
-// heads over 14k keys, 22 ranges, took 22.4 us with their attention, at once 19.8; 28 layers of 6k, 7 ranges, 747 against 726).  Two CTAs per SM are asked for so that
-// the compiler has the registers to keep them all under way.
+// log-sum-exps are requested at once, since a second round is a second trip to L2 (24 tokens of 28 heads over 14k keys, 22 ranges,
+// with their attention: eight and then four by four 22.4 us, at once 19.8).  Two CTAs per SM are asked for so that the compiler
+// has the registers for it: 118 of 128 hold 24 partials; of 25 to 32 the last ones are requested as the first arrive.
 // kExtra: the launch may also merge the rows of a problem whose causal chains are cut (c), ahead of the others, and the rows of
 // lse may be further apart than n_q.  A form of its own, as for the attention kernel.
 template <int kMost, bool kExtra>
@@ -1062,8 +1061,8 @@ static int num_sms() {
 // Query heads per tile of a causal problem over its own keys.  With the whole group in a tile (rows = G heads x 128/G
 // tokens) the causal staircase of a tile is only 128/G tokens deep instead of 128, so fewer masked sub-steps are computed;
 // against that stand the rows that a group leaves over in a tile (128 - G * (128/G), e.g. 2 of 128 for G = 7).  Both are
-// counted, in sub-steps of all tiles: at 922 tokens and G = 7 it is 413 against 497 (28 layers of 6k 787 -> 747 us), at
-// 2201 and G = 5 1608 against 1705 (layer 116 -> 113 us), at 41780 and G = 7 1.2 % more, so there tiles keep one head.
+// counted, in sub-steps of all tiles: at 922 tokens and G = 7 it is 413 against 497 with one head a tile (28 layers of 6k: 747
+// and 787 us), at 41780 and G = 7 1.2 % more, so there tiles keep one head.
 static long long causal_substeps(int n, int G, int Gp) {
     const int Tt = kBlockM / Gp, last = (n + Tt - 1) / Tt;      // tiles 1 .. last see ceil(min(j Tt, n) / kSubN) sub-steps each
     auto below = [&](int m) {                                   // sum of ceil(j Tt / kSubN) for j = 1 .. m; kSubN tiles advance Tt sub-steps

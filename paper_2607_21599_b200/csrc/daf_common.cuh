@@ -92,11 +92,15 @@ int launch_attention_joint(const void* q_imp, const void* q_fresh, bool q_in_pla
 #ifdef __CUDACC__
 
 // Launch helper.  Every kernel of the path is launched with the programmatic-serialization attribute: it may start while
-// the previous kernel of the stream is still draining and calls pdl_wait() before it touches any memory.  (A kernel that
-// is launched plainly starts only after the one before it has drained and costs 1-2 us more; with all of them dependent the
-// 6k layer went from 37.3 to 35.7 us, the question rows alone from 50.9 to 49.0, selection from K/V at 32k from 111.9 to
-// 109.9.)  A kernel that lets its dependent start early does so behind its own wait, so that the dependent, whatever it
-// waits for itself, starts with everything before that kernel complete.
+// the previous kernel of the stream is still draining and calls pdl_wait() before it touches memory that one may use (a kernel
+// launched plainly starts only after the one before it has drained and costs 1-2 us more).  A kernel that lets its dependent
+// start early does so behind its own wait: the dependent starts with everything before that kernel complete.
+// Two kernels touch memory ahead of their wait, and rest on just that, for everything but the kernel launched just before:
+//   - expand_fp8_cache_kernel beside the selection (it releases its dependent ahead of its wait too): the selection uses none
+//     of its memory, and it waits for the selection before it retires, so the gather, which waits for it, finds both complete;
+//   - attn_fwd_kernel with q_early reads idx and q_fresh, which the gather does not write: the selection was complete before
+//     the gather passed its wait.
+// A kernel put between expansion and gather or between gather and attention has to wait before it releases its dependent.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                  Args... args) {

@@ -201,14 +201,15 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     if (lane == 31) { sh->scan_gt[warp] = in_gt; sh->scan_eq[warp] = in_eq; }
     __syncthreads();
     if (warp == 0) {
-        uint32_t a = lane < kSelWarps ? sh->scan_gt[lane] : 0u, b = lane < kSelWarps ? sh->scan_eq[lane] : 0u;
+        static_assert(kSelWarps == 32, "one warp's total per lane");
+        const uint32_t a = sh->scan_gt[lane], b = sh->scan_eq[lane];
         uint32_t ia = a, ib = b;
         for (int o = 1; o < 32; o <<= 1) {
             uint32_t x = __shfl_up_sync(0xFFFFFFFFu, ia, o), y = __shfl_up_sync(0xFFFFFFFFu, ib, o);
             if (lane >= o) { ia += x; ib += y; }
         }
-        if (lane < kSelWarps) { sh->scan_gt[lane] = ia - a; sh->scan_eq[lane] = ib - b; }
-        if (lane == kSelWarps - 1) { sh->cta_counts[0] = ia; sh->cta_counts[1] = ib; }
+        sh->scan_gt[lane] = ia - a; sh->scan_eq[lane] = ib - b;
+        if (lane == 31) { sh->cta_counts[0] = ia; sh->cta_counts[1] = ib; }
     }
     cluster.sync();   // every CTA's counts are visible
     uint32_t gt_before = sh->scan_gt[warp] + in_gt - n_gt;
@@ -668,8 +669,6 @@ deviation_sum_kernel(const SignalLayers layers, int L_d, int chunks_per_row, flo
 // ----------------------------------------------------------------- host side
 // Measured (selection alone, back to back in a graph, lognormal scores): one CTA 5.6 / 6.4 us at 6K / 8K tokens, the cluster
 // of eight 6.7 / 7.1 there and 7.3 / 8.1 / 10.1 / 22.1 at 11K / 16K / 32K / 136K: one CTA up to 8K tokens, the cluster beyond.
-// (The cluster with 512 threads a CTA, one load in flight each and a pass of its own for the first histogram: 7.5 / 8.7 /
-// 12.1 / 32.0.  Digits of 12 bits, whose histograms are 16 times as much to exchange: 12.0 / 14.4 / 11.9 / 22.0.)
 static int g_sel1_max_keys = 8192;
 #ifdef DAF_TRACE
 extern "C" void daf_dbg_sel1_max_keys(int n) { g_sel1_max_keys = n < kSel1MaxKeys ? n : kSel1MaxKeys; }
@@ -839,10 +838,9 @@ __device__ __forceinline__ uint4 expand8(uint2 bytes, float scale) {
 }
 
 // A streaming pass, read and write.  A CTA takes 256 kPer runs of 8 elements that lie together, a thread kPer of them: each warp
-// reads 256 and writes 512 consecutive bytes at a time (16 elements per thread, two stores 32 bytes apart: 18.4 us at 16k tokens
-// of 8 heads, 100 MB in all; this way 14.5, of which L2 takes part of the writes; layer 105 -> 102.5).  Eight runs a thread
-// keep enough loads under way on a full GPU; a cache of which eight would leave SMs without a CTA takes one (322 tokens of 4
-// heads 3.3 us with eight).
+// reads 256 and writes 512 consecutive bytes at a time (16k tokens of 8 heads, 100 MB in all, part of whose writes stay in L2:
+// 14.5 us; 18.4 with 16 elements a thread and its two stores 32 bytes apart).  Eight runs a thread keep enough loads under way
+// on a full GPU; a cache of which eight would leave SMs without a CTA takes one (322 tokens of 4 heads: 2.4 us, 3.3 with eight).
 template <int kPer>
 __global__ void __launch_bounds__(256)
 expand_fp8_cache_kernel(const uint2* __restrict__ k8, const uint2* __restrict__ v8, const float* __restrict__ k_scale,
