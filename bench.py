@@ -39,10 +39,10 @@ from paper_2607_21599_b200 import workloads as W  # noqa: E402
 METRIC = "daf_prefill_attention_us_per_layer"
 UNIT = "us/layer"
 
-Q_IN_PLACE_MIN_K = 16384    # from this many important tokens on, the layer is called without a packed-Q buffer
+Q_IN_PLACE_MIN_K = 16384    # from this many important tokens on, the layer is called without a packed-Q buffer (see layer_call)
 # DRAM bytes per launch of the dominant kernel (the joint attention launch), dram__bytes_read.sum +
 # dram__bytes_write.sum of the committed ncu capture of that workload; no entry where none was captured.
-NCU_TRAFFIC_BYTES = {"c1": 21746944, "c2": 93970176, "c3": 148794368}
+NCU_TRAFFIC_BYTES = {"c1": 21758720, "c2": 99594240, "c3": 181295104}
 DEFAULT_PRIMARY, DEFAULT_OTHERS = "c3", ("c1", "c2")
 
 
@@ -281,10 +281,10 @@ def measure_config(env: Env, w: W.Workload, primary: bool):
     row_bytes = Hq * 256
 
     # All launches below go to torch's current stream (the capture stream while a graph is recorded).
-    # With both stages present the layer needs no packed copy of the Q rows: step 2 can read them in place.
-    # That saves most of the gather traffic but costs each work item a scattered fetch of its Q rows; measured
-    # on B200 the layer time changes by -2 % (k = 41780), +-1 % (k = 6554) and +10 % (k = 922), so only very
-    # long condensed sequences are run that way.
+    # With both stages present the layer needs no packed copy of the Q rows.  With the buffers given here it reads them in
+    # place all the same wherever that is faster, and leaves the packed rows as a result; calling it without one saves
+    # storing them: 25.2 -> 24.8 us per layer at k = 922, 70.5 -> 69.5 at 1639, 385 -> 380 at 6554, nothing at 41780, where
+    # the threshold is about memory (a packed copy of 300 MB).
     both = w.k > 0 and w.L_q > 0
     q_in_place = both and w.k >= Q_IN_PLACE_MIN_K
     # Likewise the K/V rows of step 2 (--kv-in-place; slower, for comparison): the attention kernel fetches them

@@ -248,8 +248,9 @@ int daf_full_causal_attn(const daf_params* p, int32_t n_tokens, const void* q, c
  *   row_pos_out  optional int32 [k+L_q]
  *                With q_pack given it may share memory with rows of q_fresh below L_d (in scatter mode with all of it, at
  *                the same address), and in compact mode begin with q_pack; what was there before is then lost.
- *   q_pack       may be NULL when L_q > 0: step 2 then reads its Q rows in place.  A buffer given receives the packed
- *                rows (from 4 query heads per KV head on mostly written by step 2, which reads in place all the same).
+ *   q_pack       may be NULL when L_q > 0: step 2 then reads its Q rows in place, the cheaper form by 0 to 2 % of a layer
+ *                unless there are fewer than 4 query heads per KV head and few tokens (32 on 32, 133 of 1325: 4 % the
+ *                other way).  A buffer given receives the packed rows.
  *   k_pack, v_pack  may be NULL (both or neither) when k > 0 and L_q > 0: step 2 then reads its K/V rows in
  *                place too -- rows idx of k_fresh / v_fresh, fetched by the attention kernel itself -- and
  *                the kernel in front of it only updates the hybrid cache.  Same results, bit for bit, and no
