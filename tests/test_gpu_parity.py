@@ -109,6 +109,33 @@ def test_select_indices_bit_exact(L_d, r, n_sig, kind):
     assert np.array_equal(idx_out[:k].cpu().numpy(), ref)
 
 
+# L_d: either side of where the cluster takes over, slices of 8 CTAs that are ragged and a last one that is empty, keys in
+# global scratch.  in_bin: how many keys share the top 12 bits with the threshold, either side of the number up to which they
+# are counted straight into the cluster's sums; low: all of them differ in the last 8 bits at most, so that every pass is needed.
+@pytest.mark.parametrize("L_d,in_bin,low", [
+    (3072, 500, False), (3073, 500, False), (3073, 3073, True), (3079, 1, False), (4097, 2048, True), (9000, 2048, False),
+    (9000, 2049, False), (9000, 2049, True), (40007, 12, True), (330000, 2048, True), (330000, 5000, False),
+])
+def test_selection_whose_threshold_bin_holds_a_given_number_of_keys(L_d, in_bin, low):
+    g = torch.Generator().manual_seed(L_d + in_bin)
+    above = min(700, L_d - in_bin)
+    S = -torch.rand(L_d, generator=g)                       # of either sign: the lowest keys
+    place = torch.randperm(L_d, generator=g)
+    S[place[:above]] = 2.0 + torch.rand(above, generator=g)
+    step = torch.randint(0, 200, (in_bin,), generator=g) if low else torch.randint(0, 1 << 20, (in_bin,), generator=g)
+    S[place[above:above + in_bin]] = (1.0 + step.double() * 2.0 ** -23).float()      # within [1, 1.125): one value of the top bits
+    k = above + (in_bin + 1) // 2
+    r = k / L_d
+    if api.daf_num_important(L_d, r) != k:
+        r = (k - 0.5) / L_d if api.daf_num_important(L_d, r) > k else (k + 0.5) / L_d
+    k = api.daf_num_important(L_d, r)
+    p = api.make_params(L_d, 4, r, 4, 2)
+    ws = api.alloc_workspace(p)
+    idx = torch.full((k + 1,), -1, dtype=torch.int32, device="cuda")
+    _ok(api.daf_select_topk(p, S.cuda(), 1, idx, ws), ws, "daf_select_topk")
+    assert np.array_equal(idx[:k].cpu().numpy(), oracle.select(S[None].numpy(), k)) and int(idx[k]) == -1
+
+
 # --------------------------------------------------------------------------- deviation signal
 @pytest.mark.parametrize("L_d,L_q,Hkv", [(1024, 32, 4), (777, 0, 8), (6144, 64, 4), (5, 3, 1), (40000, 16, 8)])
 def test_deviation_scores_match_oracle(L_d, L_q, Hkv):
