@@ -629,24 +629,52 @@ __device__ __forceinline__ float sq_dev8(const int4 a, const int4 b) {
     return acc;
 }
 
-__global__ void __launch_bounds__(256)
+// 16 bytes that are read once.
+__device__ __forceinline__ int4 ld_once(const int4* p) {
+    int4 r;
+    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+// A token's value of one layer, this lane's part of it: chunks lane, lane + 32, ... of its rows in that order, two of them
+// (eight loads) requested at a time.
+__device__ __forceinline__ float sq_dev_rows(const int4* kf, const int4* vf, const int4* kc, const int4* vc, int chunks, int lane) {
+    float acc = 0.f;
+    int c = lane;
+    for (; c + 32 < chunks; c += 64) {
+        const int4 kf0 = ld_once(kf + c), kc0 = ld_once(kc + c), vf0 = ld_once(vf + c), vc0 = ld_once(vc + c);
+        const int4 kf1 = ld_once(kf + c + 32), kc1 = ld_once(kc + c + 32), vf1 = ld_once(vf + c + 32), vc1 = ld_once(vc + c + 32);
+        acc += sq_dev8(kf0, kc0);
+        acc += sq_dev8(vf0, vc0);
+        acc += sq_dev8(kf1, kc1);
+        acc += sq_dev8(vf1, vc1);
+    }
+    if (c < chunks) {
+        const int4 kf0 = ld_once(kf + c), kc0 = ld_once(kc + c), vf0 = ld_once(vf + c), vc0 = ld_once(vc + c);
+        acc += sq_dev8(kf0, kc0);
+        acc += sq_dev8(vf0, vc0);
+    }
+    return acc;
+}
+
+// One warp per token, as many CTAs as that takes, each lane's loads of a layer (eight at four heads) requested together.  Bound by
+// HBM: three layers of 32k tokens of 4 heads, 403 MB, with the ranking and the gather behind it 92.8 us, of which about 56 are this
+// pass (7.2 TB/s; it only reads).  As a grid of 8 CTAs per SM whose warps walked several tokens, of which 6 were resident and the
+// rest ran as a second wave, 104.9 and 67; CTAs of 8 and 16 warps 92.2 and 97.9, but with few tokens they reach fewer SMs (1146
+// tokens of 8 heads 23.0 us before, 18.7 with 8 warps, 16.8 with 4; 6840 tokens 48.8, 46.5, 45.4).
+constexpr int kSignalWarps = 4;
+__global__ void __launch_bounds__(32 * kSignalWarps)
 deviation_scores_kernel(const int4* __restrict__ k_fresh, const int4* __restrict__ v_fresh,
                         const int4* __restrict__ k_cached, const int4* __restrict__ v_cached,
                         int L_d, int chunks_per_row, float* __restrict__ scores) {
     pdl_wait();
     const int lane = threadIdx.x & 31;
-    const int warps_per_grid = (int)(gridDim.x * (blockDim.x >> 5));
-    for (int tok = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); tok < L_d; tok += warps_per_grid) {
-        const size_t base = (size_t)tok * chunks_per_row;
-        float acc = 0.f;
-        for (int c = lane; c < chunks_per_row; c += 32) {
-            acc += sq_dev8(__ldg(k_fresh + base + c), __ldg(k_cached + base + c));
-            acc += sq_dev8(__ldg(v_fresh + base + c), __ldg(v_cached + base + c));
-        }
+    const int tok = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (tok >= L_d) return;
+    const size_t base = (size_t)tok * chunks_per_row;
+    float acc = sq_dev_rows(k_fresh + base, v_fresh + base, k_cached + base, v_cached + base, chunks_per_row, lane);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-        if (lane == 0) scores[tok] = acc;
-    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    if (lane == 0) scores[tok] = acc;
 }
 
 // The same signal for several layers at once, aggregated on the fly (Methods, item 1: the signals of several
@@ -664,29 +692,23 @@ struct SignalLayers {
     int n;
 };
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(32 * kSignalWarps)
 deviation_sum_kernel(const SignalLayers layers, int L_d, int chunks_per_row, float* __restrict__ sums) {
     pdl_wait();
     pdl_launch_dependents();   // the selection kernel may start launching; it waits for this grid before reading sums
     const int lane = threadIdx.x & 31;
-    const int warps_per_grid = (int)(gridDim.x * (blockDim.x >> 5));
-    for (int tok = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); tok < L_d; tok += warps_per_grid) {
-        const size_t base = (size_t)tok * chunks_per_row;
-        float total = 0.f;
-        for (int l = 0; l < layers.n; ++l) {
-            const int4* kf = layers.k_fresh[l]; const int4* vf = layers.v_fresh[l];
-            const int4* kc = layers.k_cached[l]; const int4* vc = layers.v_cached[l];
-            float acc = 0.f;
-            for (int c = lane; c < chunks_per_row; c += 32) {
-                acc += sq_dev8(__ldg(kf + base + c), __ldg(kc + base + c));
-                acc += sq_dev8(__ldg(vf + base + c), __ldg(vc + base + c));
-            }
+    const int tok = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+    if (tok >= L_d) return;
+    const size_t base = (size_t)tok * chunks_per_row;
+    float total = 0.f;
+    for (int l = 0; l < layers.n; ++l) {
+        float acc = sq_dev_rows(layers.k_fresh[l] + base, layers.v_fresh[l] + base, layers.k_cached[l] + base,
+                                layers.v_cached[l] + base, chunks_per_row, lane);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-            total = l == 0 ? acc : add_rn_keep_subnormals(total, acc);
-        }
-        if (lane == 0) sums[tok] = total;
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+        total = l == 0 ? acc : add_rn_keep_subnormals(total, acc);
     }
+    if (lane == 0) sums[tok] = total;
 }
 
 // ----------------------------------------------------------------- host side
@@ -777,10 +799,7 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
 int launch_deviation_scores(const ResolvedParams& rp, const void* k_fresh, const void* v_fresh, const void* k_cached,
                             const void* v_cached, float* scores, cudaStream_t stream) {
     if (rp.L_d == 0) return DAF_OK;
-    const int warps = 8;
-    int blocks = (rp.L_d + warps - 1) / warps;
-    const int max_blocks = 148 * 8;          // a few waves of 256-thread CTAs; each warp then walks several tokens
-    if (blocks > max_blocks) blocks = max_blocks;
+    const int warps = kSignalWarps, blocks = (rp.L_d + warps - 1) / warps;
     const cudaError_t e = launch_kernel(deviation_scores_kernel, dim3(blocks), dim3(warps * 32), 0, stream,
         reinterpret_cast<const int4*>(k_fresh), reinterpret_cast<const int4*>(v_fresh),
         reinterpret_cast<const int4*>(k_cached), reinterpret_cast<const int4*>(v_cached), rp.L_d, rp.Hkv * 16, scores);
@@ -802,10 +821,7 @@ int launch_deviation_sum(const ResolvedParams& rp, int n_sig, const void* const*
         layers.k_cached[l] = reinterpret_cast<const int4*>(k_cached[j]);
         layers.v_cached[l] = reinterpret_cast<const int4*>(v_cached[j]);
     }
-    const int warps = 8;
-    int blocks = (rp.L_d + warps - 1) / warps;
-    const int max_blocks = 148 * 8;
-    if (blocks > max_blocks) blocks = max_blocks;
+    const int warps = kSignalWarps, blocks = (rp.L_d + warps - 1) / warps;
     const cudaError_t e = launch_kernel(deviation_sum_kernel, dim3(blocks), dim3(warps * 32), 0, stream, layers, rp.L_d,
                                         rp.Hkv * 16, sums);
     count_launch();

@@ -137,6 +137,21 @@ def test_selection_whose_threshold_bin_holds_a_given_number_of_keys(L_d, in_bin,
 
 
 # --------------------------------------------------------------------------- deviation signal
+# rows of 32, 48, 80 and 96 chunks: a lane's second chunk is there for none, half or all of a warp; token counts that leave a
+# last CTA of 1 to 3 warps.  fp32 sums of Hkv * 256 non-negative terms: relative error at most that many roundings in a lane's
+# chain of 8 * ceil(Hkv / 2) * 2 products and 5 of the tree, 2^-24 each: below 2e-5 for Hkv <= 6.
+@pytest.mark.parametrize("L_d,Hkv", [(1, 2), (5, 3), (1031, 5), (1030, 6), (4099, 3)])
+def test_deviation_scores_of_rows_that_do_not_fill_a_warps_loads(L_d, Hkv):
+    kf, vf, kc, vc = (_normal((L_d, Hkv, 128), 91 + i) for i in range(4))
+    p = api.make_params(L_d, 0, 0.5, Hkv, Hkv)
+    s = torch.full((L_d + 1,), -1.0, dtype=torch.float32, device="cuda")
+    api.check(api.daf_deviation_scores(p, kf.cuda(), vf.cuda(), kc.cuda(), vc.cuda(), s), "daf_deviation_scores")
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(s[:L_d].cpu().numpy().astype(np.float64), oracle.deviation_scores(_f(kf), _f(vf), _f(kc), _f(vc), L_d),
+                               rtol=2e-5, atol=0)
+    assert float(s[L_d]) == -1.0, "wrote past the end"
+
+
 @pytest.mark.parametrize("L_d,L_q,Hkv", [(1024, 32, 4), (777, 0, 8), (6144, 64, 4), (5, 3, 1), (40000, 16, 8)])
 def test_deviation_scores_match_oracle(L_d, L_q, Hkv):
     N = L_d + L_q
