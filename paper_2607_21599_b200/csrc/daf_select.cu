@@ -461,7 +461,7 @@ select_topk_cta_kernel(const float* __restrict__ scores, int n_sig, int L_d, int
 // One CTA per row.  Rows 0..k-1 are the important tokens: their fresh Q/K/V rows
 // go to the packed buffers and (K/V) into the cache rows at their positions.
 // Rows k..k+L_q-1 are the question tokens: fresh K/V rows are appended to the cache.
-constexpr int kRowThreads = 192;
+constexpr int kRowThreads = 128;
 
 struct GatherArgs {
     const int4* q_fresh; const int4* k_fresh; const int4* v_fresh;
@@ -471,18 +471,20 @@ struct GatherArgs {
     int32_t* idx_copy;        // when non-null, also receives idx (the idx_in path)
     int k, L_d, L_q, cq, ckv; // cq/ckv: 16-byte chunks per Q row / per K (or V) row
     int overwrite;
-    // kFar only: the caller's cache in host memory (null: not written), and whether the important rows of the device's
+    // kBatched only: the caller's cache in host memory (null: not written), and whether the important rows of the device's
     // cache are left to update_cache_kernel because the document rows are still on their way to it
     int4* host_k; int4* host_v;
     int cache_later;
     DeviceStatus* status;
 };
 
-// kFar: the fresh rows come from far away (pinned host memory, read over the host link): every thread requests all
-// its chunks of the row before it stores any, so that one round trip covers them.  For rows in device memory the
-// plain loop is the faster one inside a layer (the batched form made the layer 0.4 us slower at 16k).
-constexpr int kRowMaxChunks = 4;      // 4 x 192 x 16 B = 12 KB: a row of 32 + 2 x 8 heads
-template <bool kFar>
+// kBatched: every thread requests all its chunks of the row before it stores any, so that one round trip covers them: for rows
+// that come from far away (pinned host memory, read over the host link), and where Q rows are packed as well, 9 KB a row at 28
+// heads on 4 (selection from K/V at 32k 92.3 -> 90.9 us).  For K/V rows in device memory the plain loop is the faster one inside a
+// layer (6k layer 31.1 us, 31.8 batched).  128 threads a CTA: 6k layer 31.11 -> 30.96 us, 11k 105.8 -> 104.9 against 192, whose
+// CTAs no longer all fit on the GPU at once from 1480 rows on.
+constexpr int kRowMaxChunks = 6;      // 6 x 128 x 16 B = 12 KB: a row of 32 + 2 x 8 heads
+template <bool kBatched>
 __global__ void __launch_bounds__(kRowThreads)
 gather_update_kernel(const GatherArgs a) {
     DAF_KT_BEGIN(1);
@@ -503,7 +505,7 @@ gather_update_kernel(const GatherArgs a) {
         // no packed Q wanted: K, V only; no packed K/V wanted and nothing to overwrite in the cache: nothing at all
         const int c_end = (a.k_pack != nullptr || a.overwrite) ? per_row : a.cq;
         const int c0 = (a.q_pack != nullptr ? 0 : a.cq) + threadIdx.x;
-        if (kFar) {
+        if (kBatched) {
             for (int base = c0; base < c_end; base += kRowThreads * kRowMaxChunks) {
                 int4 v[kRowMaxChunks];
 #pragma unroll
@@ -554,7 +556,7 @@ gather_update_kernel(const GatherArgs a) {
             const size_t at = off + (c < a.ckv ? c : c - a.ckv);
             const int4 v = __ldg((c < a.ckv ? a.k_fresh : a.v_fresh) + at);
             (c < a.ckv ? a.kv_k : a.kv_v)[at] = v;
-            if (kFar && a.host_k != nullptr) (c < a.ckv ? a.host_k : a.host_v)[at] = v;
+            if (kBatched && a.host_k != nullptr) (c < a.ckv ? a.host_k : a.host_v)[at] = v;
         }
     }
     DAF_KT_END(1);
@@ -787,7 +789,7 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         // kernel to complete before it touches anything (so the result is that of a plain launch), but its CTAs are
         // already in place then -- after this library's selection kernel, and equally after the previous layer's
         // merge when layers are issued back to back.
-        cudaError_t e = far != nullptr ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a)
+        cudaError_t e = far != nullptr || q_pack != nullptr ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a)
                                  : launch_kernel(gather_update_kernel<false>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }

@@ -137,6 +137,28 @@ def test_selection_whose_threshold_bin_holds_a_given_number_of_keys(L_d, in_bin,
 
 
 # --------------------------------------------------------------------------- deviation signal
+# Rows of 128, 576, 768, 896 and 1536 chunks (a thread requests six of 128 at once: less than one round, a ragged one, one full
+# round, a second that is ragged, two full ones), with packed Q rows; copies, so bit for bit.
+@pytest.mark.parametrize("Hq,Hkv", [(4, 2), (28, 4), (32, 8), (40, 8), (64, 16)])
+def test_gather_packs_rows_of_any_length(Hq, Hkv):
+    L_d, L_q, r = 301, 7, 0.3
+    N, k = L_d + L_q, api.daf_num_important(L_d, r)
+    p = api.make_params(L_d, L_q, r, Hq, Hkv)
+    ws = api.alloc_workspace(p)
+    idx = torch.randperm(L_d, generator=torch.Generator().manual_seed(Hq))[:k].sort().values.to(torch.int32).cuda()
+    qf, kf, vf = (_normal((N, h, 128), 61 + i).cuda() for i, h in enumerate((Hq, Hkv, Hkv)))
+    kc, vc = (_normal((N, Hkv, 128), 65 + i).cuda() for i in range(2))
+    want_k, want_v = kc.clone(), vc.clone()
+    for want, fresh in ((want_k, kf), (want_v, vf)):
+        want[idx.long()] = fresh[idx.long()]
+        want[L_d:] = fresh[L_d:]
+    qp = torch.zeros(k, Hq, 128, dtype=torch.bfloat16, device="cuda")
+    kp, vp = (torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    _ok(api.daf_select(p, None, 0, idx, qf, kf, vf, kc, vc, None, qp, kp, vp, ws), ws, "daf_select")
+    for got, want in ((qp, qf[idx.long()]), (kp, kf[idx.long()]), (vp, vf[idx.long()]), (kc, want_k), (vc, want_v)):
+        assert torch.equal(got, want)
+
+
 # rows of 32, 48, 80 and 96 chunks: a lane's second chunk is there for none, half or all of a warp; token counts that leave a
 # last CTA of 1 to 3 warps.  fp32 sums of Hkv * 256 non-negative terms: relative error at most that many roundings in a lane's
 # chain of 8 * ceil(Hkv / 2) * 2 products and 5 of the tree, 2^-24 each: below 2e-5 for Hkv <= 6.
