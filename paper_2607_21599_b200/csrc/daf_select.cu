@@ -659,8 +659,8 @@ __device__ __forceinline__ float sq_dev_rows(const int4* kf, const int4* vf, con
 }
 
 // One warp per token, as many CTAs as that takes, each lane's loads of a layer (eight at four heads) requested together.  Bound by
-// HBM: three layers of 32k tokens of 4 heads, 403 MB, with the ranking and the gather behind it 92.8 us, of which about 56 are this
-// pass (7.2 TB/s; it only reads).  As a grid of 8 CTAs per SM whose warps walked several tokens, of which 6 were resident and the
+// HBM: three layers of 32k tokens of 4 heads, 403 MB, with the ranking and the gather behind it 92.8 us, of which 57 are this
+// pass (7.0 TB/s; it only reads).  As a grid of 8 CTAs per SM whose warps walked several tokens, of which 6 were resident and the
 // rest ran as a second wave, 104.9 and 67; CTAs of 8 and 16 warps 92.2 and 97.9, but with few tokens they reach fewer SMs (1146
 // tokens of 8 heads 23.0 us before, 18.7 with 8 warps, 16.8 with 4; 6840 tokens 48.8, 46.5, 45.4).
 constexpr int kSignalWarps = 4;
