@@ -631,10 +631,13 @@ __device__ __forceinline__ float sq_dev8(const int4 a, const int4 b) {
     return acc;
 }
 
-// 16 bytes that are read once.
+// 16 bytes that are read once.  An ordinary load that stays behind the wait for the kernel before, which may be the one that
+// writes them: not a function of the address alone (volatile, memory), nor of memory that is constant while this kernel is
+// there (.nc).
 __device__ __forceinline__ int4 ld_once(const int4* p) {
     int4 r;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.L2::256B.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p) : "memory");
     return r;
 }
 // A token's value of one layer, this lane's part of it: chunks lane, lane + 32, ... of its rows in that order, two of them

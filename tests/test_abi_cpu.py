@@ -168,3 +168,16 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(api, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="missing"):
         api.daf_num_important(10, 0.5)
+
+
+def test_inline_reads_of_global_memory_stay_behind_the_wait_for_the_kernel_before(repo_root):
+    """Every kernel may start while the one before it still writes.  An asm that is a function of its address to the
+    compiler may move ahead of griddepcontrol.wait, and .nc asks for memory that nobody writes while the kernel is there."""
+    csrc = os.path.join(repo_root, "paper_2607_21599_b200", "csrc")
+    reads = []
+    for name in sorted(os.listdir(csrc)):
+        text = open(os.path.join(csrc, name)).read()
+        reads += [(name, m.group(0)) for m in re.finditer(r"\basm\b[^;]*?\((?:\"[^\"]*\"|[^\";])*\);", text) if "ld.global" in m.group(0)]
+    assert reads, "no inline read found: the pattern no longer fits the sources"
+    for name, stmt in reads:
+        assert re.match(r"asm\s+volatile\b", stmt) and '"memory"' in stmt and ".nc" not in stmt, (name, stmt)
