@@ -505,6 +505,7 @@ gather_update_kernel(const GatherArgs a) {
         // no packed Q wanted: K, V only; no packed K/V wanted and nothing to overwrite in the cache: nothing at all
         const int c_end = (a.k_pack != nullptr || a.overwrite) ? per_row : a.cq;
         const int c0 = (a.q_pack != nullptr ? 0 : a.cq) + threadIdx.x;
+        const int k_end = min(a.cq + a.ckv, c_end);      // (a batch may reach past c_end)
         if (kBatched) {
             for (int base = c0; base < c_end; base += kRowThreads * kRowMaxChunks) {
                 int4 v[kRowMaxChunks];
@@ -512,7 +513,7 @@ gather_update_kernel(const GatherArgs a) {
                 for (int u = 0; u < kRowMaxChunks; ++u) {
                     const int c = base + u * kRowThreads;
                     if (c < a.cq) v[u] = __ldg(a.q_fresh + qsrc + c);
-                    else if (c < a.cq + a.ckv) v[u] = __ldg(a.k_fresh + ksrc + (c - a.cq));
+                    else if (c < k_end) v[u] = __ldg(a.k_fresh + ksrc + (c - a.cq));
                     else if (c < c_end) v[u] = __ldg(a.v_fresh + ksrc + (c - a.cq - a.ckv));
                 }
 #pragma unroll
@@ -520,7 +521,7 @@ gather_update_kernel(const GatherArgs a) {
                     const int c = base + u * kRowThreads;
                     if (c < a.cq) {
                         a.q_pack[qdst + c] = v[u];
-                    } else if (c < a.cq + a.ckv) {
+                    } else if (c < k_end) {
                         const int cc = c - a.cq;
                         if (a.k_pack != nullptr) a.k_pack[kdst + cc] = v[u];
                         if (a.overwrite && !a.cache_later) a.kv_k[ksrc + cc] = v[u];

@@ -159,6 +159,37 @@ def test_gather_packs_rows_of_any_length(Hq, Hkv):
         assert torch.equal(got, want)
 
 
+# Q rows alone (no packed K/V, the cache's document rows left as they are): right, and in the time of their own bytes.  K rows of
+# the same width, read in vain, would be half as many bytes again; 1.2 leaves room for noise.
+@pytest.mark.parametrize("Hq", [24, 40])
+def test_gather_of_q_alone_reads_no_k_or_v(Hq):
+    L_d, r = 65536, 0.5
+    k = api.daf_num_important(L_d, r)
+    idx = (2 * torch.arange(k, dtype=torch.int32)).cuda()
+    qf = torch.arange(L_d * Hq * 128, dtype=torch.int32, device="cuda").to(torch.int16).view(torch.bfloat16).view(L_d, Hq, 128)
+    qp = torch.zeros(k, Hq, 128, dtype=torch.bfloat16, device="cuda")
+    us = {}
+    for Hkv in (1, Hq):
+        p = api.make_params(L_d, 0, r, Hq, Hkv, overwrite_doc_kv=0)
+        ws = api.alloc_workspace(p)
+        kf, vf, kc, vc = (torch.zeros(L_d, Hkv, 128, dtype=torch.bfloat16, device="cuda") for _ in range(4))
+        qp.zero_()
+        gather = lambda: api.check(api.daf_select(p, None, 0, idx, qf, kf, vf, kc, vc, None, qp, None, None, ws), "daf_select")  # noqa: E731
+        gather()
+        _ok(0, ws, "daf_select")
+        assert torch.equal(qp.view(torch.int16), qf[idx.long()].view(torch.int16)) and not bool(kc.any()) and not bool(vc.any())
+        us[Hkv] = []
+        for _ in range(7):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(20):
+                gather()
+            e1.record()
+            torch.cuda.synchronize()
+            us[Hkv].append(e0.elapsed_time(e1) * 50)
+    assert min(us[Hq]) <= 1.2 * min(us[1]), us
+
+
 # rows of 32, 48, 80 and 96 chunks: a lane's second chunk is there for none, half or all of a warp; token counts that leave a
 # last CTA of 1 to 3 warps.  fp32 sums of Hkv * 256 non-negative terms: relative error at most that many roundings in a lane's
 # chain of 8 * ceil(Hkv / 2) * 2 products and 5 of the tree, 2^-24 each: below 2e-5 for Hkv <= 6.
