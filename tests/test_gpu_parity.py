@@ -190,6 +190,26 @@ def test_gather_of_q_alone_reads_no_k_or_v(Hq):
     assert min(us[Hq]) <= 1.2 * min(us[1]), us
 
 
+# Rows of 16, 384, 512, 528 and 1040 chunks (a thread requests four of 128 at once: part of one round, three quarters, one, one
+# and a ragged second, two and a third); copies, so bit for bit.
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("Hq", [1, 24, 32, 33, 65])
+def test_fuse_copies_rows_of_any_length(Hq, mode):
+    L_d, L_q, k = 301, 7, 90
+    N = L_d + L_q
+    p = api.make_params(L_d, L_q, 0.3, Hq, 1, fuse_mode=mode)
+    idx = torch.randperm(L_d, generator=torch.Generator().manual_seed(Hq))[:k].sort().values.to(torch.int32).cuda()
+    o_imp, o_q = _normal((k, Hq, 128), 71).cuda(), _normal((L_q, Hq, 128), 72).cuda()
+    pos = torch.cat([idx.long(), torch.arange(L_d, N, device="cuda")])
+    hidden = torch.full((N if mode else k + L_q, Hq, 128), 3.0, dtype=torch.bfloat16, device="cuda")
+    row_pos = torch.full((k + L_q,), -1, dtype=torch.int32, device="cuda")
+    want = hidden.clone()
+    want[pos if mode else torch.arange(k + L_q, device="cuda")] = torch.cat([o_imp, o_q])
+    api.check(api.daf_fuse(p, k, idx, o_imp, o_q, hidden, row_pos), "daf_fuse")
+    torch.cuda.synchronize()
+    assert torch.equal(hidden, want) and torch.equal(row_pos.long(), pos)
+
+
 # rows of 32, 48, 80 and 96 chunks: a lane's second chunk is there for none, half or all of a warp; token counts that leave a
 # last CTA of 1 to 3 warps.  fp32 sums of Hkv * 256 non-negative terms: relative error at most that many roundings in a lane's
 # chain of 8 * ceil(Hkv / 2) * 2 products and 5 of the tree, 2^-24 each: below 2e-5 for Hkv <= 6.
