@@ -22,22 +22,26 @@ DAF_KT_READER(daf_dbg_kt_select)
 // A cluster of 8 CTAs ranks all L_d aggregated scores.  Each CTA keeps a
 // contiguous slice of the keys in its shared memory.  Radix passes over 12, 12
 // and 8 bits find the key of the k-th largest score: every CTA counts the digits
-// of its slice and adds its counts to a copy of the cluster's sums in the shared
-// memory of every CTA, so that after one cluster barrier each finds the sums at
-// home and picks the same digit.  An ordered compaction then emits the selected
-// positions in ascending order.  Ties at the threshold are broken by position
-// (lower first), so the result is unique.
+// of its slice and adds its counts to the cluster's sums in shared memory, so
+// that after one cluster barrier each can pick the same digit.  An ordered
+// compaction then emits the selected positions in ascending order.  Ties at the
+// threshold are broken by position (lower first), so the result is unique.
 //
 // Bound by latency: a barrier and a scan per pass.  Twelve bits a pass because
 // sign, exponent and three bits of the fraction spread real scores over a hundred
 // bins, few of which are not empty, and 24 bits usually leave nothing to tell
-// apart; once a bin holds few keys, they are counted straight into every CTA's
-// sums, without a histogram of the CTA's own in between.  (8-bit digits whose
-// histograms every CTA read from its peers behind the barrier, clustered scores,
-// back to back: 7.8 / 8.0 / 9.6 / 12.9 / 23.6 us at 11k / 16k / 32k / 64k / 136k
-// tokens; this form 5.8 / 5.6 / 7.6 / 10.7 / 22.6, with histograms in every pass
-// 6.4 / 6.1 / 8.4 / 11.8 / 23.2.  Digits of 11, 11 and 10 bits needed the third
-// pass more often: 7.7 / 10.0 at 16k / 32k.)
+// apart.  Where the counts go (times back to back, in us):
+//   - straight into the sums while few keys are left, without a histogram of the
+//     CTA's own; equal keys of a warp as one count;
+//   - into a copy of the sums in every CTA, which then finds them at home, or, as
+//     a CTA sends about one word a clock, to one owner per range of bins where
+//     many words may have to leave one CTA: from kSelToAll keys left on, and by
+//     histogram where a CTA has more than a key per thread.
+// Clustered scores at 6k / 16k / 32k / 64k tokens 4.7 / 5.7 / 7.2 / 11.8, with a copy
+// everywhere in every pass 4.7 / 5.6 / 7.0 / 11.5; 2000 equal keys around the
+// threshold 6.2 / 7.5 / 9.5 / 13.6, each key counted by itself in every CTA 14.2 /
+// 14.0 / 12.1 / 16.9; ascending scores 5.2 / 6.2 / 8.1 / 13.7 and 6.8 / 9.4 / 13.3 /
+// 16.2; uniform ones at 64k 10.9 and 14.3.
 
 constexpr int kSelCluster = 8;
 constexpr int kSelThreads = 1024;
@@ -68,10 +72,11 @@ constexpr int kSelBits = 12;                    // digits of 12, 12 and 8 bits
 constexpr int kSelBins = 1 << kSelBits;
 constexpr int kSelLastBins = 1 << (32 - 2 * kSelBits);
 constexpr int kSelDirect = 2048;                // up to so many keys in a bin are counted straight into the cluster's sums
+constexpr int kSelToAll = 256;                  // and up to so many into every CTA's copy
 
 struct SelShared {
     uint32_t hist[kSelBins];                // this CTA's keys
-    uint32_t total[2 * kSelBins + kSelLastBins];   // the cluster's, one array per pass: every CTA adds its keys to all of them
+    uint32_t total[2 * kSelBins + kSelLastBins];   // the cluster's, one array per pass: all of them here, or those of the bins this CTA owns
     uint32_t before[2];                     // keys above / equal to the threshold in the CTAs ahead (added by those)
     uint32_t scan_a[kSelWarps];
     uint32_t scan_b[kSelWarps];
@@ -147,11 +152,23 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     // Radix selection from the top digit down.  It stops as soon as every key left in the chosen bin is taken (with distinct
     // scores usually after two passes): the comparisons below then look only at the bits resolved so far.
     uint32_t prefix = 0u, mask = 0u, k_rem = (uint32_t)k, left = 0xFFFFFFFFu;    // left: keys in the chosen bin
+#pragma unroll
     for (int pass = 0; pass < 3; ++pass) {
         const int shift = pass == 0 ? 32 - kSelBits : pass == 1 ? 32 - 2 * kSelBits : 0;
         const int n_bins = pass == 2 ? kSelLastBins : kSelBins;
         uint32_t* const total = sh->total + pass * kSelBins;
         const bool direct = left <= (uint32_t)kSelDirect;
+        const bool to_all = pass == 0 || left <= (uint32_t)kSelToAll || (!direct && per_cta <= kSelThreads);    // the same in all CTAs
+        const int owner_shift = pass == 2 ? 32 - 2 * kSelBits - 3 : kSelBits - 3;    // CTA r owns the r-th eighth of the bins
+        static_assert(kSelCluster == 1 << 3, "");
+        auto add = [&](uint32_t bin, uint32_t c) {
+            if (to_all) {
+#pragma unroll
+                for (int r = 0; r < kSelCluster; ++r) atomicAdd(cluster.map_shared_rank(&total[bin], r), c);
+            } else {
+                atomicAdd(cluster.map_shared_rank(&total[bin], (int)(bin >> owner_shift)), c);
+            }
+        };
         if (pass > 0) {
             for (int base = 0; base < n_loc; base += kSelThreads) {
                 const int i = base + tid;
@@ -160,27 +177,34 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
                 const uint32_t bin = (key >> shift) & (uint32_t)(n_bins - 1);
                 if (!direct) {
                     count(in, bin);
-                } else if (in) {
-#pragma unroll
-                    for (int r = 0; r < kSelCluster; ++r) atomicAdd(cluster.map_shared_rank(&total[bin], r), 1u);
+                    continue;
                 }
+                const uint32_t active = __ballot_sync(0xFFFFFFFFu, in);
+                if (active == 0u) continue;
+                const int lead = __ffs(active) - 1;
+                const uint32_t lead_bin = __shfl_sync(0xFFFFFFFFu, bin, lead);
+                const bool one_bin = __ballot_sync(0xFFFFFFFFu, in && bin == lead_bin) == active;
+                if (one_bin ? lane == lead : in) add(bin, one_bin ? (uint32_t)__popc(active) : 1u);
             }
         }
         if (!direct) {
-            __syncthreads();   // this CTA's histogram is complete: its bins go to every CTA's sums (few are not empty)
+            __syncthreads();   // this CTA's histogram is complete: its bins go to the cluster's sums (few are not empty)
             for (int bin = tid; bin < n_bins; bin += kSelThreads) {
                 const uint32_t c = sh->hist[bin];
                 if (c != 0u) {
                     sh->hist[bin] = 0u;
-#pragma unroll
-                    for (int r = 0; r < kSelCluster; ++r) atomicAdd(cluster.map_shared_rank(&total[bin], r), c);
+                    add((uint32_t)bin, c);
                 }
             }
         }
         cluster.sync();    // the sums of this pass are complete
         // thread t owns the four bins from n_bins - 4 - 4t on: the running count from the top
         const int low = n_bins - 4 - 4 * tid;
-        const uint4 four = low >= 0 ? *reinterpret_cast<const uint4*>(&total[low]) : make_uint4(0u, 0u, 0u, 0u);
+        uint4 four = make_uint4(0u, 0u, 0u, 0u);
+        if (low >= 0) {
+            if (to_all) four = *reinterpret_cast<const uint4*>(&total[low]);
+            else four = *reinterpret_cast<const uint4*>(cluster.map_shared_rank(&total[low], low >> owner_shift));
+        }
         const uint32_t own = four.x + four.y + four.z + four.w;
         uint32_t incl = own;
 #pragma unroll

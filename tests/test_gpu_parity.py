@@ -136,6 +136,65 @@ def test_selection_whose_threshold_bin_holds_a_given_number_of_keys(L_d, in_bin,
     assert np.array_equal(idx[:k].cpu().numpy(), oracle.select(S[None].numpy(), k)) and int(idx[k]) == -1
 
 
+# Keys that share the top 12 bits with the threshold and have few values among them, over the whole context or side by side in one
+# CTA's slice: counted once per warp where a warp's keys are equal, into the sums of every CTA (up to 256 of them) or of one (more).
+@pytest.mark.parametrize("L_d,in_bin,values,together", [
+    (4097, 256, 1, False), (4097, 257, 1, False), (4097, 256, 256, True), (4097, 257, 257, True), (4100, 4000, 3, False),
+    (8192, 2048, 1, False), (8193, 2049, 1, False), (8193, 2049, 900, False), (9000, 2000, 7, True), (40007, 2048, 2048, True),
+    (330000, 2048, 2, False), (330000, 200000, 70000, False),
+])
+def test_selection_among_tied_keys(L_d, in_bin, values, together):
+    g = torch.Generator().manual_seed(L_d + in_bin + values)
+    above = min(700, L_d - in_bin)
+    S = -torch.rand(L_d, generator=g)
+    place = torch.arange(L_d).roll(1000) if together else torch.randperm(L_d, generator=g)
+    S[place[:above]] = 2.0 + torch.rand(above, generator=g)
+    step = torch.randint(0, values, (in_bin,), generator=g)
+    S[place[above:above + in_bin]] = (1.0 + step.double() * ((1 << 20) // values) * 2.0 ** -23).float()      # within [1, 1.125)
+    for part in (0.01, 0.5, 1.0):
+        k = above + max(1, int(in_bin * part))
+        r = min(1.0, (k - 0.5) / L_d)
+        assert api.daf_num_important(L_d, r) == k
+        p = api.make_params(L_d, 4, r, 4, 2)
+        ws = api.alloc_workspace(p)
+        idx = torch.full((k + 1,), -1, dtype=torch.int32, device="cuda")
+        _ok(api.daf_select_topk(p, S.cuda(), 1, idx, ws), ws, "daf_select_topk")
+        assert np.array_equal(idx[:k].cpu().numpy(), oracle.select(S[None].numpy(), k)) and int(idx[k]) == -1
+
+
+def _replayed_us(call, n=20):
+    """Time of a call, the best of some replays of n of them in a graph."""
+    call()
+    torch.cuda.synchronize()
+    graph, best = torch.cuda.CUDAGraph(), float("inf")
+    with torch.cuda.graph(graph):
+        for _ in range(n):
+            call()
+    for _ in range(10):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        graph.replay()
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1) * 1e3 / n)
+    return best
+
+
+def test_selection_among_ties_takes_about_as_long_as_without():
+    """2000 equal scores around the threshold: one more pass and nothing that goes by the number of equal keys.  (7.4 us against 5.0
+    without ties; each key counted by itself in every CTA 12.5.)"""
+    L_d, r = 6144, 0.15
+    p = api.make_params(L_d, 4, r, 4, 2)
+    ws = api.alloc_workspace(p)
+    idx = torch.empty(api.daf_num_important(L_d, r), dtype=torch.int32, device="cuda")
+    S = torch.rand(L_d, generator=torch.Generator().manual_seed(5))
+    tied = S.clone()
+    order = torch.argsort(S, descending=True)
+    tied[order[200:2200]] = S[order[900]]
+    us = [_replayed_us(lambda s=s: api.check(api.daf_select_topk(p, s, 1, idx, ws), "daf_select_topk")) for s in (S.cuda(), tied.cuda())]
+    assert us[1] <= 1.8 * us[0], us
+
+
 # --------------------------------------------------------------------------- deviation signal
 # Rows of 128, 576, 768, 896 and 1536 chunks (a thread requests six of 128 at once: less than one round, a ragged one, one full
 # round, a second that is ragged, two full ones), with packed Q rows; copies, so bit for bit.
