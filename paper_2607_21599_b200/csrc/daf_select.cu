@@ -280,7 +280,7 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     DAF_KT_END(0);
 }
 
-// ------------------------------------------------ selection, one CTA (up to 3K tokens)
+// ------------------------------------------------ selection, one CTA (up to 4K tokens)
 // Few keys run in one CTA with no cluster traffic.  The keys are first reduced to their offset from the smallest key.  One
 // pass over all keys histograms the top 11 of the bits that offset needs (typically 24-27 of 32, fewer
 // when the scores are close together) with shared-memory atomics and finds the bin that holds the k-th
@@ -290,7 +290,7 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
 // candidates, but the result stays correct.  An ordered compaction then emits the positions.
 constexpr int kSel1Threads = 1024;
 constexpr int kSel1Warps = kSel1Threads / 32;
-constexpr int kSel1MaxKeys = 3072;    // see launch_select
+constexpr int kSel1MaxKeys = 4096;    // see launch_select
 constexpr int kSel1TopBits = 11;      // first pass, over all keys
 constexpr int kSel1TopBins = 1 << kSel1TopBits;
 constexpr int kSel1Bits = 9;          // later passes, over the candidates
@@ -782,8 +782,10 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
             if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
             attr_done[dev].store(true, std::memory_order_release);
         }
-        // One CTA and the cluster of eight, alone, back to back in a graph, clustered scores: 3.7 and 4.4 us at 1K tokens, 4.5 and
-        // 4.5 at 3K, 5.7 and 5.1 at 6K, 6.4 and 6.1 at 8K.
+        // One CTA and the cluster of eight.  The whole layer, clustered scores: 4000 tokens of 28 / 40 / 4 heads on 4 / 8 / 4 22.8 / 25.4 /
+        // 19.8 us and 23.4 / 26.0 / 20.4, 3500 tokens of 28 26.0 and 26.5, 5200 of 28 25.8 and 25.8, 8192 36.9 and 36.6; scores within
+        // 2^-17 of each other 22.9 and 24.7 at 4000, 25.6 and 27.4 at 5200; of either sign 25.1 and 23.6, 28.5 and 26.2.  Alone and back
+        // to back the cluster is level at 3000 already (4.7 and 4.5): in a layer its eight CTAs start later than one.
         if (rp.L_d <= kSel1MaxKeys) {
             const size_t smem1 = sizeof(Sel1Shared) + ((size_t)padded(rp.L_d) + rp.L_d) * sizeof(uint32_t);   // keys and candidate list
             const cudaError_t e = launch_kernel(select_topk_cta_kernel, dim3(1), dim3(kSel1Threads), smem1, stream,

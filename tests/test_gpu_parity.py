@@ -109,11 +109,11 @@ def test_select_indices_bit_exact(L_d, r, n_sig, kind):
     assert np.array_equal(idx_out[:k].cpu().numpy(), ref)
 
 
-# L_d: either side of where the cluster takes over, slices of 8 CTAs that are ragged and a last one that is empty, keys in
+# L_d: one CTA and either side of where the cluster takes over, slices of 8 CTAs that are ragged, keys in
 # global scratch.  in_bin: how many keys share the top 12 bits with the threshold, either side of the number up to which they
 # are counted straight into the cluster's sums; low: all of them differ in the last 8 bits at most, so that every pass is needed.
 @pytest.mark.parametrize("L_d,in_bin,low", [
-    (3072, 500, False), (3073, 500, False), (3073, 3073, True), (3079, 1, False), (4097, 2048, True), (9000, 2048, False),
+    (3072, 500, False), (4096, 500, False), (4097, 500, False), (4097, 4097, True), (3073, 500, False), (3073, 3073, True), (3079, 1, False), (4097, 2048, True), (9000, 2048, False),
     (9000, 2049, False), (9000, 2049, True), (40007, 12, True), (330000, 2048, True), (330000, 5000, False),
 ])
 def test_selection_whose_threshold_bin_holds_a_given_number_of_keys(L_d, in_bin, low):
