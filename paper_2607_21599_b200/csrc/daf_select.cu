@@ -66,7 +66,7 @@ __device__ __forceinline__ float add_rn_keep_subnormals(float a, float b) {
 
 // Keys sit in shared memory with one word of padding per 32, so that both access patterns are free of bank
 // conflicts: consecutive threads reading consecutive keys, and each thread walking its own run of keys.
-__host__ __device__ __forceinline__ int padded(int i) { return i + (i >> 5); }
+__host__ __device__ constexpr int padded(int i) { return i + (i >> 5); }
 
 constexpr int kSelBits = 12;                    // digits of 12, 12 and 8 bits
 constexpr int kSelBins = 1 << kSelBits;
@@ -291,6 +291,8 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
 constexpr int kSel1Threads = 1024;
 constexpr int kSel1Warps = kSel1Threads / 32;
 constexpr int kSel1MaxKeys = 4096;    // see launch_select
+constexpr int kSel1PerThread = kSel1MaxKeys / kSel1Threads;
+static_assert(kSel1PerThread * kSel1Threads == kSel1MaxKeys, "every key has a thread that loads it");
 constexpr int kSel1TopBits = 11;      // first pass, over all keys
 constexpr int kSel1TopBins = 1 << kSel1TopBits;
 constexpr int kSel1Bits = 9;          // later passes, over the candidates
@@ -365,34 +367,32 @@ select_topk_cta_kernel(const float* __restrict__ scores, int n_sig, int L_d, int
     pdl_launch_dependents();   // the gather kernel may start launching; it waits for this grid before reading idx
 
     // aggregate the signal rows in ascending row order (fp32 adds, no fusing), build keys, find their range
-    // (eight loads in flight per thread: one load per trip would serialise on memory latency)
+    // (a thread's loads of a row in flight together: one after the other would serialise on memory latency)
     uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-    for (int base = tid; base < L_d; base += 8 * kSel1Threads) {
-        float acc[8];
+    float acc[kSel1PerThread];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = base + u * kSel1Threads;
-            acc[u] = i < L_d ? scores[i] : 0.f;
-        }
-        for (int l = 1; l < n_sig; ++l) {
-            float nxt[8];
+    for (int u = 0; u < kSel1PerThread; ++u) {
+        const int i = tid + u * kSel1Threads;
+        acc[u] = i < L_d ? scores[i] : 0.f;
+    }
+    for (int l = 1; l < n_sig; ++l) {
+        float nxt[kSel1PerThread];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = base + u * kSel1Threads;
-                nxt[u] = i < L_d ? scores[(size_t)l * L_d + i] : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u] = add_rn_keep_subnormals(acc[u], nxt[u]);
+        for (int u = 0; u < kSel1PerThread; ++u) {
+            const int i = tid + u * kSel1Threads;
+            nxt[u] = i < L_d ? scores[(size_t)l * L_d + i] : 0.f;
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = base + u * kSel1Threads;
-            if (i < L_d) {
-                const uint32_t key = score_key(acc[u]);
-                keys[padded(i)] = key;
-                kmin = min(kmin, key);
-                kmax = max(kmax, key);
-            }
+        for (int u = 0; u < kSel1PerThread; ++u) acc[u] = add_rn_keep_subnormals(acc[u], nxt[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kSel1PerThread; ++u) {
+        const int i = tid + u * kSel1Threads;
+        if (i < L_d) {
+            const uint32_t key = score_key(acc[u]);
+            keys[padded(i)] = key;
+            kmin = min(kmin, key);
+            kmax = max(kmax, key);
         }
     }
     for (int i = tid; i < kSel1TopBins; i += kSel1Threads) sh->hist[i] = 0u;
@@ -774,11 +774,8 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         int dev = 0;
         cudaGetDevice(&dev);
         if (dev >= 0 && dev < 64 && !attr_done[dev].load(std::memory_order_acquire)) {
-            cudaError_t e = cudaFuncSetAttribute(select_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            const cudaError_t e = cudaFuncSetAttribute(select_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)(sizeof(SelShared) + (size_t)padded(kSelSmemKeysPerCta) * sizeof(uint32_t)));
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(select_topk_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(Sel1Shared) + ((size_t)padded(kSel1MaxKeys) + kSel1MaxKeys) * sizeof(uint32_t)));
             if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
             attr_done[dev].store(true, std::memory_order_release);
         }
@@ -787,6 +784,7 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         // 2^-17 of each other 22.9 and 24.7 at 4000, 25.6 and 27.4 at 5200; of either sign 25.1 and 23.6, 28.5 and 26.2.  Alone and back
         // to back the cluster is level at 3000 already (4.7 and 4.5): in a layer its eight CTAs start later than one.
         if (rp.L_d <= kSel1MaxKeys) {
+            static_assert(sizeof(Sel1Shared) + (padded(kSel1MaxKeys) + kSel1MaxKeys) * sizeof(uint32_t) <= 48 * 1024, "within the default limit");
             const size_t smem1 = sizeof(Sel1Shared) + ((size_t)padded(rp.L_d) + rp.L_d) * sizeof(uint32_t);   // keys and candidate list
             const cudaError_t e = launch_kernel(select_topk_cta_kernel, dim3(1), dim3(kSel1Threads), smem1, stream,
                                                 scores, n_sig, rp.L_d, rp.k, idx_out);
