@@ -37,11 +37,13 @@ DAF_KT_READER(daf_dbg_kt_select)
 //     a CTA sends about one word a clock, to one owner per range of bins where
 //     many words may have to leave one CTA: from kSelToAll keys left on, and by
 //     histogram where a CTA has more than a key per thread.
-// Clustered scores at 6k / 16k / 32k / 64k tokens 4.7 / 5.7 / 7.2 / 11.8, with a copy
-// everywhere in every pass 4.7 / 5.6 / 7.0 / 11.5; 2000 equal keys around the
-// threshold 6.2 / 7.5 / 9.5 / 13.6, each key counted by itself in every CTA 14.2 /
-// 14.0 / 12.1 / 16.9; ascending scores 5.2 / 6.2 / 8.1 / 13.7 and 6.8 / 9.4 / 13.3 /
-// 16.2; uniform ones at 64k 10.9 and 14.3.
+// Clustered scores at 6k / 16k / 32k / 64k tokens 4.9 / 6.0 / 7.5 / 12.3, with a copy
+// everywhere in every pass 4.7 / 5.6 / 7.0 / 11.5 (layers: the same); 2000 equal keys
+// around the threshold 6.5 / 7.9 / 9.8 / 14.0, each key counted by itself in every
+// CTA 14.2 / 14.0 / 12.1 / 16.9; ascending scores 5.5 / 6.6 / 8.4 / 13.7 and 6.8 / 9.4 /
+// 13.3 / 16.2; uniform ones at 64k 11.0 and 14.3.  The loops over passes and CTAs
+// stay loops: unrolled they are 0.2 to 0.5 us faster back to back, but in a layer, where
+// each kernel's code has to be fetched again, 11k 102.5 -> 105.1 us, 16k 82.3 -> 83.7.
 
 constexpr int kSelCluster = 8;
 constexpr int kSelThreads = 1024;
@@ -152,7 +154,7 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
     // Radix selection from the top digit down.  It stops as soon as every key left in the chosen bin is taken (with distinct
     // scores usually after two passes): the comparisons below then look only at the bits resolved so far.
     uint32_t prefix = 0u, mask = 0u, k_rem = (uint32_t)k, left = 0xFFFFFFFFu;    // left: keys in the chosen bin
-#pragma unroll
+#pragma unroll 1
     for (int pass = 0; pass < 3; ++pass) {
         const int shift = pass == 0 ? 32 - kSelBits : pass == 1 ? 32 - 2 * kSelBits : 0;
         const int n_bins = pass == 2 ? kSelLastBins : kSelBins;
@@ -162,12 +164,10 @@ select_topk_kernel(const float* __restrict__ scores, int n_sig, int L_d, int k,
         const int owner_shift = pass == 2 ? 32 - 2 * kSelBits - 3 : kSelBits - 3;    // CTA r owns the r-th eighth of the bins
         static_assert(kSelCluster == 1 << 3, "");
         auto add = [&](uint32_t bin, uint32_t c) {
-            if (to_all) {
-#pragma unroll
-                for (int r = 0; r < kSelCluster; ++r) atomicAdd(cluster.map_shared_rank(&total[bin], r), c);
-            } else {
-                atomicAdd(cluster.map_shared_rank(&total[bin], (int)(bin >> owner_shift)), c);
-            }
+            int r = to_all ? 0 : (int)(bin >> owner_shift);
+            const int last = to_all ? kSelCluster - 1 : r;
+#pragma unroll 1
+            for (; r <= last; ++r) atomicAdd(cluster.map_shared_rank(&total[bin], r), c);
         };
         if (pass > 0) {
             for (int base = 0; base < n_loc; base += kSelThreads) {
@@ -779,10 +779,10 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
             if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
             attr_done[dev].store(true, std::memory_order_release);
         }
-        // One CTA and the cluster of eight.  The whole layer, clustered scores: 4000 tokens of 28 / 40 / 4 heads on 4 / 8 / 4 22.8 / 25.4 /
-        // 19.8 us and 23.4 / 26.0 / 20.4, 3500 tokens of 28 26.0 and 26.5, 5200 of 28 25.8 and 25.8, 8192 36.9 and 36.6; scores within
-        // 2^-17 of each other 22.9 and 24.7 at 4000, 25.6 and 27.4 at 5200; of either sign 25.1 and 23.6, 28.5 and 26.2.  Alone and back
-        // to back the cluster is level at 3000 already (4.7 and 4.5): in a layer its eight CTAs start later than one.
+        // One CTA and the cluster of eight.  The whole layer, clustered scores: 4000 tokens of 28 / 40 / 4 heads on 4 / 8 / 4 22.6 / 25.0 /
+        // 19.0 us and 23.6 / 25.9 / 19.9, 3500 tokens of 28 25.8 and 26.5, 5200 of 28 25.8 and 25.8, 8192 36.9 and 36.6; scores within
+        // 2^-17 of each other 22.6 and 25.2 at 4000, 25.6 and 27.4 at 5200; of either sign 24.9 and 23.9, 28.5 and 26.2.  Alone and back
+        // to back the cluster is level at 3000 already (4.6 and 4.4): behind other kernels its eight CTAs start later than one.
         if (rp.L_d <= kSel1MaxKeys) {
             static_assert(sizeof(Sel1Shared) + (padded(kSel1MaxKeys) + kSel1MaxKeys) * sizeof(uint32_t) <= 48 * 1024, "within the default limit");
             const size_t smem1 = sizeof(Sel1Shared) + ((size_t)padded(rp.L_d) + rp.L_d) * sizeof(uint32_t);   // keys and candidate list
