@@ -495,21 +495,16 @@ struct GatherArgs {
     int32_t* idx_copy;        // when non-null, also receives idx (the idx_in path)
     int k, L_d, L_q, cq, ckv; // cq/ckv: 16-byte chunks per Q row / per K (or V) row
     int overwrite;
-    // kBatched only: the caller's cache in host memory (null: not written), and whether the important rows of the device's
+    // rows from host memory only: the caller's cache in host memory (null: not written), and whether the important rows of the device's
     // cache are left to update_cache_kernel because the document rows are still on their way to it
     int4* host_k; int4* host_v;
     int cache_later;
     DeviceStatus* status;
 };
 
-// kBatched: every thread requests all its chunks of the row before it stores any, so that one round trip covers them: for rows
-// that come from far away (pinned host memory, read over the host link), and where Q rows are packed as well, 9 KB a row at 28
-// heads on 4 (selection from K/V at 32k 92.3 -> 90.9 us).  For K/V rows in device memory the plain loop is the faster one inside a
-// layer (6k layer 31.1 us, 31.8 batched).  128 threads a CTA: 6k layer 31.11 -> 30.96 us, 11k 105.8 -> 104.9 against 192, whose
-// CTAs no longer all fit on the GPU at once from 1480 rows on.
-constexpr int kRowMaxChunks = 6;      // 6 x 128 x 16 B = 12 KB: a row of 32 + 2 x 8 heads
-template <bool kBatched>
-__global__ void __launch_bounds__(kRowThreads)
+// A thread requests kBatch chunks of its row before it stores any (1: the plain loop).  Which form for which row: launch_select.
+template <int kBatch, int kThreads>
+__global__ void __launch_bounds__(kThreads)
 gather_update_kernel(const GatherArgs a) {
     DAF_KT_BEGIN(1);
     pdl_wait();                // idx may come from the selection kernel launched just before; the packed buffers may still be read by the previous layer
@@ -530,19 +525,19 @@ gather_update_kernel(const GatherArgs a) {
         const int c_end = (a.k_pack != nullptr || a.overwrite) ? per_row : a.cq;
         const int c0 = (a.q_pack != nullptr ? 0 : a.cq) + threadIdx.x;
         const int k_end = min(a.cq + a.ckv, c_end);      // (a batch may reach past c_end)
-        if (kBatched) {
-            for (int base = c0; base < c_end; base += kRowThreads * kRowMaxChunks) {
-                int4 v[kRowMaxChunks];
+        if constexpr (kBatch > 1) {
+            for (int base = c0; base < c_end; base += kThreads * kBatch) {
+                int4 v[kBatch];
 #pragma unroll
-                for (int u = 0; u < kRowMaxChunks; ++u) {
-                    const int c = base + u * kRowThreads;
+                for (int u = 0; u < kBatch; ++u) {
+                    const int c = base + u * kThreads;
                     if (c < a.cq) v[u] = __ldg(a.q_fresh + qsrc + c);
                     else if (c < k_end) v[u] = __ldg(a.k_fresh + ksrc + (c - a.cq));
                     else if (c < c_end) v[u] = __ldg(a.v_fresh + ksrc + (c - a.cq - a.ckv));
                 }
 #pragma unroll
-                for (int u = 0; u < kRowMaxChunks; ++u) {
-                    const int c = base + u * kRowThreads;
+                for (int u = 0; u < kBatch; ++u) {
+                    const int c = base + u * kThreads;
                     if (c < a.cq) {
                         a.q_pack[qdst + c] = v[u];
                     } else if (c < k_end) {
@@ -559,7 +554,7 @@ gather_update_kernel(const GatherArgs a) {
                 }
             }
         } else {
-            for (int c = c0; c < c_end; c += kRowThreads) {
+            for (int c = c0; c < c_end; c += kThreads) {
                 if (c < a.cq) {
                     a.q_pack[qdst + c] = __ldg(a.q_fresh + qsrc + c);
                 } else if (c < a.cq + a.ckv) {
@@ -577,11 +572,11 @@ gather_update_kernel(const GatherArgs a) {
         }
     } else {
         const size_t off = (size_t)(a.L_d + (row - a.k)) * a.ckv;
-        for (int c = threadIdx.x; c < 2 * a.ckv; c += kRowThreads) {
+        for (int c = threadIdx.x; c < 2 * a.ckv; c += kThreads) {
             const size_t at = off + (c < a.ckv ? c : c - a.ckv);
             const int4 v = __ldg((c < a.ckv ? a.k_fresh : a.v_fresh) + at);
             (c < a.ckv ? a.kv_k : a.kv_v)[at] = v;
-            if (kBatched && a.host_k != nullptr) (c < a.ckv ? a.host_k : a.host_v)[at] = v;
+            if (kBatch > 1 && a.host_k != nullptr) (c < a.ckv ? a.host_k : a.host_v)[at] = v;
         }
     }
     DAF_KT_END(1);
@@ -829,8 +824,22 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
         // kernel to complete before it touches anything (so the result is that of a plain launch), but its CTAs are
         // already in place then -- after this library's selection kernel, and equally after the previous layer's
         // merge when layers are issued back to back.
-        cudaError_t e = far != nullptr || q_pack != nullptr ? launch_kernel(gather_update_kernel<true>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a)
-                                 : launch_kernel(gather_update_kernel<false>, dim3((unsigned)rows), dim3(kRowThreads), 0, stream, a);
+        // Rows from host memory, read over the link, in batches of 12 KB (32 + 2 x 8 heads): one round trip covers a row.  K/V rows
+        // alone by the plain loop (6k layer 31.0 us, 31.8 in batches) and 128 threads (with 192 6k layer 31.1 us, 922 rows of 32 KV
+        // heads 8.3, 6.6 with 128; from 1480 rows on they no longer all fit on the GPU at once), or 192 where that is one chunk for
+        // each (154 rows of 6 KV heads 1.54 us, 1.74 with 128).  With Q rows to pack as well, batches of 12 KB by 192 threads: 154 / 922 / 6554
+        // rows of 28 heads on 4, in L2 / from HBM, 1.8 / 1.9, 3.7 / 3.9, 21.3 / 22.6 us; the plain loop with 192 threads 2.1 / 2.0,
+        // 3.8 / 4.3, 23.1 / 24.6; batches by 128 threads 1.7 / 1.8, 4.0 / 4.1, 21.3 / 22.6, but 922 rows of 40 heads on 8 6.1 / 6.1,
+        // where 192 take 5.6 / 6.1 and the plain loop 5.4 / 6.0.  A row of no more chunks than threads has nothing to batch: 922 rows
+        // of 4 heads on 2 (128 chunks) 1.7 us, 2.5 as a batch of which all but one chunk is empty.
+        const int chunks = (q_pack != nullptr ? a.cq : 0) + (k_pack != nullptr || a.overwrite ? 2 * a.ckv : 0);   // of an important row
+        auto gather = [&](void (*kernel)(GatherArgs), int threads) {
+            return launch_kernel(kernel, dim3((unsigned)rows), dim3((unsigned)threads), 0, stream, a);
+        };
+        const cudaError_t e = far != nullptr                      ? gather(gather_update_kernel<6, 128>, 128)
+                              : chunks > 128 && chunks <= 192     ? gather(gather_update_kernel<1, 192>, 192)
+                              : chunks > 192 && q_pack != nullptr ? gather(gather_update_kernel<4, 192>, 192)
+                                                                  : gather(gather_update_kernel<1, 128>, 128);
         count_launch();
         if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }
         if (int rc = check_launch()) return rc;

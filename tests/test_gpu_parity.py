@@ -196,9 +196,10 @@ def test_selection_among_ties_takes_about_as_long_as_without():
 
 
 # --------------------------------------------------------------------------- deviation signal
-# Rows of 128, 576, 768, 896 and 1536 chunks (a thread requests six of 128 at once: less than one round, a ragged one, one full
-# round, a second that is ragged, two full ones), with packed Q rows; copies, so bit for bit.
-@pytest.mark.parametrize("Hq,Hkv", [(4, 2), (28, 4), (32, 8), (40, 8), (64, 16)])
+# Rows of 128, 144, 192, 208, 576, 768, 896 and 1536 chunks (up to 128 and up to 192 are one a thread; beyond, a thread requests
+# four of 192 at once: a ragged round, one full round, a second that is ragged, two full ones), with packed Q rows; copies, so bit
+# for bit.
+@pytest.mark.parametrize("Hq,Hkv", [(4, 2), (7, 1), (8, 2), (11, 1), (28, 4), (32, 8), (40, 8), (64, 16)])
 def test_gather_packs_rows_of_any_length(Hq, Hkv):
     L_d, L_q, r = 301, 7, 0.3
     N, k = L_d + L_q, api.daf_num_important(L_d, r)
@@ -216,6 +217,28 @@ def test_gather_packs_rows_of_any_length(Hq, Hkv):
     _ok(api.daf_select(p, None, 0, idx, qf, kf, vf, kc, vc, None, qp, kp, vp, ws), ws, "daf_select")
     for got, want in ((qp, qf[idx.long()]), (kp, kf[idx.long()]), (vp, vf[idx.long()]), (kc, want_k), (vc, want_v)):
         assert torch.equal(got, want)
+
+
+# K/V rows alone of 128, 160, 192, 224, 256, 320 and 512 chunks (one a thread up to 192), with and without packed copies, the cache's document rows written or not.
+@pytest.mark.parametrize("pack", [True, False])
+@pytest.mark.parametrize("overwrite", [0, 1])
+@pytest.mark.parametrize("Hkv", [4, 5, 6, 7, 8, 10, 16])
+def test_gather_of_k_and_v_rows_of_any_length(Hkv, overwrite, pack):
+    L_d, L_q, r = 301, 7, 0.3
+    N, k = L_d + L_q, api.daf_num_important(L_d, r)
+    p = api.make_params(L_d, L_q, r, Hkv, Hkv, overwrite_doc_kv=overwrite)
+    ws = api.alloc_workspace(p)
+    idx = torch.randperm(L_d, generator=torch.Generator().manual_seed(Hkv))[:k].sort().values.to(torch.int32).cuda()
+    qf, kf, vf, kc, vc = (_normal((N, Hkv, 128), 61 + i).cuda() for i in range(5))
+    want_k, want_v = kc.clone(), vc.clone()
+    for want, fresh in ((want_k, kf), (want_v, vf)):
+        if overwrite:
+            want[idx.long()] = fresh[idx.long()]
+        want[L_d:] = fresh[L_d:]
+    kp, vp = (torch.zeros(k, Hkv, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    _ok(api.daf_select(p, None, 0, idx, qf, kf, vf, kc, vc, None, None, kp if pack else None, vp if pack else None, ws), ws, "daf_select")
+    assert torch.equal(kc, want_k) and torch.equal(vc, want_v)
+    assert torch.equal(kp, kf[idx.long()] if pack else torch.zeros_like(kp)) and torch.equal(vp, vf[idx.long()] if pack else torch.zeros_like(vp))
 
 
 # Q rows alone (no packed K/V, the cache's document rows left as they are): right, and in the time of their own bytes.  K rows of
