@@ -672,8 +672,8 @@ __device__ __forceinline__ int4 ld_once(const int4* p) {
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p) : "memory");
     return r;
 }
-// A token's value of one layer, this lane's part of it: chunks lane, lane + 32, ... of its rows in that order, two of them
-// (eight loads) requested at a time.
+// A token's value of one layer, this lane's part of it: chunks lane, lane + 32, ... of its rows in that order, the loads of two of
+// them written ahead of the arithmetic (at 32 registers the compiler keeps about six of the eight in flight).
 __device__ __forceinline__ float sq_dev_rows(const int4* kf, const int4* vf, const int4* kc, const int4* vc, int chunks, int lane) {
     float acc = 0.f;
     int c = lane;
@@ -693,13 +693,11 @@ __device__ __forceinline__ float sq_dev_rows(const int4* kf, const int4* vf, con
     return acc;
 }
 
-// One warp per token, as many CTAs as that takes, each lane's loads of a layer (eight at four heads) requested together.  Bound by
-// HBM: three layers of 32k tokens of 4 heads, 403 MB, with the ranking and the gather behind it 92.8 us, of which 57 are this
-// pass (7.0 TB/s; it only reads).  As a grid of 8 CTAs per SM whose warps walked several tokens, of which 6 were resident and the
-// rest ran as a second wave, 104.9 and 67; CTAs of 8 and 16 warps 92.2 and 97.9, but with few tokens they reach fewer SMs (1146
-// tokens of 8 heads 23.0 us before, 18.7 with 8 warps, 16.8 with 4; 6840 tokens 48.8, 46.5, 45.4).
-constexpr int kSignalWarps = 4;
-__global__ void __launch_bounds__(32 * kSignalWarps)
+// One warp per token, as many CTAs as that takes.  Bound by HBM: three layers of 32k tokens of 4 heads, 403 MB, 57 us (7.0 TB/s; it
+// only reads).  As a grid of 8 CTAs of 8 warps per SM whose warps walked several tokens, of which 6 were resident and the rest ran
+// as a second wave, 67.  The warps of a CTA: signal_warps.
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps)
 deviation_scores_kernel(const int4* __restrict__ k_fresh, const int4* __restrict__ v_fresh,
                         const int4* __restrict__ k_cached, const int4* __restrict__ v_cached,
                         int L_d, int chunks_per_row, float* __restrict__ scores) {
@@ -729,7 +727,8 @@ struct SignalLayers {
     int n;
 };
 
-__global__ void __launch_bounds__(32 * kSignalWarps)
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps)
 deviation_sum_kernel(const SignalLayers layers, int L_d, int chunks_per_row, float* __restrict__ sums) {
     pdl_wait();
     pdl_launch_dependents();   // the selection kernel may start launching; it waits for this grid before reading sums
@@ -847,11 +846,17 @@ int launch_select(const ResolvedParams& rp, const float* scores, int n_sig, cons
     return DAF_OK;
 }
 
+// Four warps a CTA, which spreads few tokens over more SMs and leaves less of a last wave (three layers of 300 tokens of 4 heads 5.3 us,
+// 5.4 with eight; 16k tokens 30.1 and 30.6).  Where four a CTA puts 64 warps on an SM and most of the grid on the GPU at once, eight,
+// of which 48 fit, get more out of L2 and HBM: 6840 tokens of 4 heads 13.5 us, 14.4 with four (9 to 12 and 7.7 where L2 holds the
+// rows), 11003 of 8 41 and 45.6; one layer of 11003 tokens of 8 heads that L2 holds 8.3, 8 to 13 with four.
+static int signal_warps(int L_d) { return L_d > 4096 && L_d <= 12288 ? 8 : 4; }
+
 int launch_deviation_scores(const ResolvedParams& rp, const void* k_fresh, const void* v_fresh, const void* k_cached,
                             const void* v_cached, float* scores, cudaStream_t stream) {
     if (rp.L_d == 0) return DAF_OK;
-    const int warps = kSignalWarps, blocks = (rp.L_d + warps - 1) / warps;
-    const cudaError_t e = launch_kernel(deviation_scores_kernel, dim3(blocks), dim3(warps * 32), 0, stream,
+    const int warps = signal_warps(rp.L_d), blocks = (rp.L_d + warps - 1) / warps;
+    const cudaError_t e = launch_kernel(warps == 8 ? deviation_scores_kernel<8> : deviation_scores_kernel<4>, dim3(blocks), dim3(warps * 32), 0, stream,
         reinterpret_cast<const int4*>(k_fresh), reinterpret_cast<const int4*>(v_fresh),
         reinterpret_cast<const int4*>(k_cached), reinterpret_cast<const int4*>(v_cached), rp.L_d, rp.Hkv * 16, scores);
     count_launch();
@@ -872,8 +877,8 @@ int launch_deviation_sum(const ResolvedParams& rp, int n_sig, const void* const*
         layers.k_cached[l] = reinterpret_cast<const int4*>(k_cached[j]);
         layers.v_cached[l] = reinterpret_cast<const int4*>(v_cached[j]);
     }
-    const int warps = kSignalWarps, blocks = (rp.L_d + warps - 1) / warps;
-    const cudaError_t e = launch_kernel(deviation_sum_kernel, dim3(blocks), dim3(warps * 32), 0, stream, layers, rp.L_d,
+    const int warps = signal_warps(rp.L_d), blocks = (rp.L_d + warps - 1) / warps;
+    const cudaError_t e = launch_kernel(warps == 8 ? deviation_sum_kernel<8> : deviation_sum_kernel<4>, dim3(blocks), dim3(warps * 32), 0, stream, layers, rp.L_d,
                                         rp.Hkv * 16, sums);
     count_launch();
     if (e != cudaSuccess) { set_cuda_error(e); return DAF_ERR_CUDA; }

@@ -295,7 +295,8 @@ def test_fuse_copies_rows_of_any_length(Hq, mode):
 # rows of 32, 48, 80 and 96 chunks: a lane's second chunk is there for none, half or all of a warp; token counts that leave a
 # last CTA of 1 to 3 warps.  fp32 sums of Hkv * 256 non-negative terms: relative error at most that many roundings in a lane's
 # chain of 8 * ceil(Hkv / 2) * 2 products and 5 of the tree, 2^-24 each: below 2e-5 for Hkv <= 6.
-@pytest.mark.parametrize("L_d,Hkv", [(1, 2), (5, 3), (1031, 5), (1030, 6), (4099, 3)])
+# (4096, 4097, 12288, 12289: either side of where a CTA has eight warps instead of four)
+@pytest.mark.parametrize("L_d,Hkv", [(1, 2), (5, 3), (1031, 5), (1030, 6), (4099, 3), (4096, 2), (4097, 2), (12288, 1), (12289, 1)])
 def test_deviation_scores_of_rows_that_do_not_fill_a_warps_loads(L_d, Hkv):
     kf, vf, kc, vc = (_normal((L_d, Hkv, 128), 91 + i) for i in range(4))
     p = api.make_params(L_d, 0, 0.5, Hkv, Hkv)
