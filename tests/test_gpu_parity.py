@@ -61,8 +61,11 @@ def _normal(shape, seed, scale=1.0):
     (16384, 0.10, 1, "constant"), (20000, 0.3, 2, "ties"), (40960, 0.2, 1, "lognormal"), (40961, 0.2, 1, "lognormal"),
     (7, 0.5, 1, "lognormal"), (1, 1.0, 1, "lognormal"), (12000, 0.2, 1, "special"), (16384, 0.5, 1, "ties"),
     (16385, 0.5, 1, "ties"), (2048, 0.05, 1, "narrow"),
-    # either side of the size at which the cluster kernel takes over; a cluster-sized problem whose keys differ
+    # either side of the size at which the cluster kernel takes over, several rows of scores; the largest sizes of one CTA with
+    # many equal scores; either side of one key per thread of the cluster; a cluster-sized problem whose keys differ
     # only in their last byte (every radix pass is needed) and one whose keys differ only in the first two
+    (4096, 0.15, 3, "lognormal"), (4097, 0.15, 3, "lognormal"), (2500, 0.3, 2, "ties"), (3000, 0.2, 1, "constant"), (4096, 0.3, 2, "ties"),
+    (4097, 0.2, 1, "constant"),
     (8192, 0.15, 1, "lognormal"), (8193, 0.15, 1, "lognormal"), (20000, 0.2, 1, "lowbyte"), (24000, 0.1, 1, "highbytes"),
     (30000, 1.0, 1, "lognormal"), (30000, 0.0, 1, "lognormal"),
     # sums of two signal rows that are subnormal in fp32: the aggregation must keep them apart, not flush them to 0
