@@ -766,9 +766,7 @@ attn_fwd_kernel(const __grid_constant__ CUtensorMap tmap_q0, const __grid_consta
             // usually there, are asked after without waiting on either side of the wait for P, so that the answers overlap; the
             // two products stay apart, since K of t + 2 may still be on its way when P of t has come.
             // With the stores of P in two halves (softmax_core) 16k full recompute 2109 -> 2044 us, 136k layer 11983 -> 11559, 16k
-            // layer 1.3 % less.  (All three asked after by try_wait, which sleeps on a barrier that is not ready: 13 to 40 % slower.
-            // The products issued by two warps, Q K^T behind the completion of P V: 0 to 9 % slower with three K slots.  Q K^T of
-            // 128 keys as one product, one S buffer: 9 to 25 % slower.)
+            // layer 1.3 % less.  (V and K not by try_wait: it sleeps on a barrier that is not ready, 13 to 40 % slower.)
             auto step = [&](auto slot, int t) -> bool {
                 constexpr int b = decltype(slot)::value;
                 const uint32_t par = (uint32_t)((t >> 1) & 1);
